@@ -88,8 +88,12 @@ cudaError_t launch_score_simt(int dtype, int d, const CacheView& c, const BlockA
 cudaError_t launch_evict(int dtype, int d, const CacheView& c, const EvictArgs& e, cudaStream_t st);
 cudaError_t launch_decode(int dtype, int d, const CacheView& c, const void* q, const void* k, const void* v,
                           void* out, int32_t pos, float scale, int32_t target /* <0: none */, cudaStream_t st);
+int sm_count();   // multiprocessors of the current device
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                               int32_t pos, float scale, int32_t target /* <0: none */, cudaStream_t st);
+// bf16 decode step as a stream (decode_stream.cu); *taken = false: the shape does not fit it, nothing was enqueued
+cudaError_t launch_decode_stream(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
+                                 int32_t pos, float scale, bool evict_one, cudaStream_t st, bool* taken);
 size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target);
 size_t evict_smem_bytes(int n_cand, int target);
 size_t decode_smem_bytes(int d, int g, int n_rows, int target);
@@ -122,18 +126,26 @@ struct SmemConfigured {
 // still running; the kernel itself must execute pdl_wait() before it touches anything the predecessor may have
 // written, and pdl_release() lets its own successor start.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_dependent_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t st,
+                                     Args&&... args) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = grid;
   lc.blockDim = block;
   lc.dynamicSmemBytes = smem;
   lc.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&lc, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_dependent_cluster(kernel, grid, block, smem, 1, st, static_cast<Args&&>(args)...);
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -661,15 +661,6 @@ cudaError_t launch_nt(const CacheView& c, const DecodeArgs& a, cudaStream_t st, 
   return plain ? launch_nt_p<D, G, NT, true, 1>(c, a, st, no_map) : launch_nt_p<D, G, NT, false, 1>(c, a, st, no_map);
 }
 
-int sm_count() {   // of the current device
-  static int count[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  if (count[dev] == 0 && cudaDeviceGetAttribute(&count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    count[dev] = 148;
-  return count[dev];
-}
-
 template <int D, int G>
 cudaError_t launch_t(const CacheView& c, const DecodeArgs& a, cudaStream_t st) {
   // four small CTAs per SM only pay for short caches: all four must fit into shared memory (up to about 1500 pairs
@@ -695,14 +686,54 @@ cudaError_t launch_g(const CacheView& c, const DecodeArgs& a, cudaStream_t st) {
 
 }  // namespace
 
+int sm_count() {
+  static int count[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if (count[dev] == 0 && cudaDeviceGetAttribute(&count[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    count[dev] = 148;
+  return count[dev];
+}
+
 size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
   const size_t attn = smem_layout(nullptr, d, g, n_rows, kMaxWarps, nullptr);
   const size_t ev = (target >= 0 && target < n_rows) ? evict_smem_bytes(n_rows, target) : 0;
   return attn > ev ? attn : ev;
 }
 
+// Which kernel takes a step.  Measured, us per step (stream against this file's kernels; d = 128, g = 4, one pair leaves):
+// 128 caches of 512 pairs 10.5 / 10.1, of 700 pairs 12.5 / 14.6 (the instance with K in registers ends at 640 pairs);
+// 256 caches of 384 pairs 14.5 / 14.4, of 1024 pairs 30.8 / 34.2; 640 caches of 256 pairs 26.8 / 24.9, of 384 pairs
+// 31.8 / 41.7; 1024 caches of 1024 pairs 95 / 112; at d = 64 128 caches of 256 pairs 6.5 / 7.1, 1024 caches of 512 pairs
+// 40.5 / 42.3, of 700 pairs 46 / 55.  So: a cache for every SM at most -- the stream unless all of K fits the registers;
+// beyond that the stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next
+// cache's bytes: 150 KB, or 256 KB while the other kernel holds every cache of the call at once (two CTAs per SM).
+static bool stream_is_faster(int d, int n1, int units) {
+  const int sms = sm_count();
+  if (units <= sms) return d == 64 || n1 > kBatchTiles * 128;
+  return (size_t)n1 * d * 4 >= (units <= 2 * sms ? 256u : 150u) * 1024;
+}
+
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                               int32_t pos, float scale, int32_t target, cudaStream_t st) {
+  const int n1 = c.n_old + 1;
+  if (stream_is_faster(d, n1, c.nsamples * c.Hkv)) {
+    // exactly one pair leaves by a single ranking value per pair: inside the kernel; any other cut follows it
+    const bool cut = target >= 0 && target < n1;
+    const bool one = cut && target == n1 - 1 && !(c.fill && c.rule == 1) && c.rule < 3;
+    bool taken = false;
+    const cudaError_t err = launch_decode_stream(d, c, q, k, v, out, pos, scale, one, st, &taken);
+    if (err != cudaSuccess) return err;
+    if (taken) {
+      if (!cut || one) return cudaSuccess;
+      CacheView grown = c;
+      grown.n_old = n1;
+      EvictArgs e;
+      e.blk_k = nullptr; e.blk_v = nullptr; e.new_sum = nullptr;
+      e.I = 0; e.pos0 = 0; e.curr_id = pos; e.target = target;
+      return launch_evict(1, d, grown, e, st);
+    }
+  }
   DecodeArgs a{q, k, v, out, pos, scale, target};
   if (d == 64) return launch_g<64>(c, a, st);
   if (d == 128) return launch_g<128>(c, a, st);

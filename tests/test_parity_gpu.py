@@ -255,6 +255,30 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
+    (1, 3, 1, 64, 40, {}),                                  # less than one tile of rows
+    (1, 2, 4, 128, 1023, {}),                               # a cluster of 8 CTAs per cache; the step's row ends a tile
+    (1, 8, 2, 128, 1024, {}),                               # ... or starts one
+    (4, 8, 8, 64, 1100, {}),                                # 32 caches: clusters of 4
+    (6, 8, 1, 128, 1300, {}),                               # 48 caches: clusters of 2, K tiles behind the V tiles in the ring
+    (20, 8, 1, 128, 641, {}),                               # more caches than SMs: a second cache per CTA
+    (40, 8, 4, 64, 1090, {}),                               # three caches per CTA
+    (20, 8, 4, 128, 700, dict(p_dec=3)),                    # the cut follows as a launch of its own
+    (20, 8, 4, 128, 700, dict(compaction="fill")),
+    (1, 4, 2, 128, 1024, dict(compaction="fill")),
+    (1, 4, 2, 128, 900, dict(rule="sum_recent")),
+    (20, 8, 1, 128, 660, dict(rule="current_query")),
+    (3, 4, 2, 128, 700, dict(pads=[1500, 0, 700])),         # padding still cached when decoding starts
+])
+def test_decode_as_a_stream(b, Hkv, g, d, K, kw):
+    kw = dict(kw)
+    wl = tiny("stream", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 90, B=512, K=K, steps=7, dtype="bf16", d=d, p_dec=kw.pop("p_dec", 1))
+    units = [(0, 0), (b // 2, Hkv - 1), (b - 1, Hkv // 2)] if b * Hkv > 16 else all_units(wl)
+    if "pads" in kw:
+        wl = wl.with_(s=1600)
+    run_lockstep(wl, units, check_rows_every=3, **kw)
+
+
 # ------------------------------------------------------------------ unordered caches (BM_COMPACT_FILL)
 @pytest.mark.parametrize("name,kw", [
     ("f32_simt", dict(dtype="f32", d=64, Hq=4, Hkv=4, s=300, B=48, K=80, steps=12)),
