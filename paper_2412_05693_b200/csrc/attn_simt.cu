@@ -2,54 +2,111 @@
 // (outputs + log-sum-exp), and the transposed score pass that turns the normalised weights into the
 // column sums  sum_weights += sum_i attn_weights[i].  This is the production path for fp32 caches
 // (fp32 accuracy rules out the bf16 tensor-core kernels) and the fallback shape coverage for bf16.
+//
+// What bounds it: the fp32 pipes once enough warps hide the latency of the shared-memory reads (with 8 warps on an SM the
+// forward kernel issued in 41 % of the cycles and waited for fixed-latency results in most others).  A thread owns 4
+// rows x 4 keys of a logit tile and 4 rows x D/16 outputs, reads its operands as 16-byte pieces, multiplies pairs with
+// packed instructions and keeps an accumulator's two products of a step apart; 16 warps share an SM; K and V tiles
+// arrive by asynchronous copies under the arithmetic that does not need them.  Measured with 4 samples, 16 heads in
+// groups of 4, d = 128, a block of 256 against 1280 cached pairs: forward kernel 639 -> 407 us (29 TFLOP/s; busiest SM's
+// fp32 pipes 60 %, the rest is 256 CTAs on 148 SMs), score pass 324 -> 226 us, against 4 x 4 values per thread from
+// scalar reads between barriers; 8 rows per thread on half the threads: 434 us.
 #include "common.cuh"
 
 namespace bm {
 namespace {
 
-constexpr int kTile = 64;     // query rows per CTA tile and keys per tile
-constexpr int kThreads = 256;
+constexpr int kTN = 64;       // keys per tile of the forward pass
 
-// Loads 64 rows of D elements (fp32-widened) into smem with row stride D+1.  `row_ptr(r)` returns the
-// global address of tile row r or nullptr for a row that does not exist (filled with zeros).
-template <typename T, int D, typename F>
-__device__ inline void load_tile(float* dst, int tid, F row_ptr) {
-  constexpr int V = Elem<T>::kVec;
-  constexpr int CH = D / V;  // 16-byte chunks per row
-  for (int idx = tid; idx < kTile * CH; idx += kThreads) {
-    const int r = idx / CH, cv = idx % CH;
-    const T* p = row_ptr(r);
-    float f[V];
-    if (p != nullptr) {
-      Elem<T>::unpack(ld_global_16(p + cv * V), f);
-    } else {
-#pragma unroll
-      for (int e = 0; e < V; ++e) f[e] = 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < V; ++e) dst[r * (D + 1) + cv * V + e] = f[e];
-  }
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the float at the same place of CTA `rank` of the cluster
+__device__ __forceinline__ float ld_peer(const float* p, uint32_t rank) {
+  uint32_t at;
+  float v;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+  return v;
 }
 
-// 64x64 tile of dot products: thread (ty, tx) owns rows ty+16a, columns tx+16b.
-template <int D>
-__device__ inline void dot_tile(const float* sA, const float* sB, int ty, int tx, float (&acc)[4][4]) {
+typedef unsigned long long f32x2;   // two floats side by side
+__device__ __forceinline__ void fma_pair(f32x2& acc, f32x2 a, f32x2 b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ f32x2 dup(float x) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul_pair(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float lo_of(f32x2 x) { return __uint_as_float((uint32_t)x); }
+__device__ __forceinline__ float hi_of(f32x2 x) { return __uint_as_float((uint32_t)(x >> 32)); }
+
+// Rows of D elements, widened to fp32, into shared memory with row stride LD; `row_ptr(r)` is the global address of row
+// r or null for a row that does not exist (zeros).  fp32 rows are copied asynchronously (one commit group per call).
+template <typename T, int D, int LD, int ROWS, int NT, typename F>
+__device__ __forceinline__ void load_rows(float* dst, int tid, F row_ptr) {
+  constexpr int V = Elem<T>::kVec, CH = D / V;   // elements per 16-byte piece, pieces per row
+#pragma unroll 4
+  for (int idx = tid; idx < ROWS * CH; idx += NT) {
+    const int r = idx / CH, cv = idx % CH;
+    const T* p = row_ptr(r);
+    float* to = dst + r * LD + cv * V;
+    if constexpr (sizeof(T) == 4) {
+      const uint32_t s = (uint32_t)__cvta_generic_to_shared(to);
+      if (p != nullptr) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(p + cv * V) : "memory");
+      else *reinterpret_cast<float4*>(to) = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      float f[V];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+      for (int e = 0; e < V; ++e) f[e] = 0.f;
+      if (p != nullptr) Elem<T>::unpack(ld_global_16(p + cv * V), f);
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-#pragma unroll 8
-  for (int c = 0; c < D; ++c) {
-    float av[4], bv[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = sA[(ty + 16 * a) * (D + 1) + c];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) bv[b] = sB[(tx + 16 * b) * (D + 1) + c];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+      for (int e = 0; e < V; ++e) to[e] = f[e];
+    }
   }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void commit_nothing() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void wait_copies() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Dot products of rows ty + TY x of sA with rows tx + 16 y of sB (row stride LD = D + 4: the 16-byte pieces that a warp
+// reads at one time lie in different banks).  Even and odd elements are added up apart and joined at the end.
+template <int D, int LD, int TY, int RT, int KT>
+__device__ __forceinline__ void dot_rows(const float* sA, const float* sB, int ty, int tx, float (&s)[RT][KT]) {
+  f32x2 acc[RT][KT];
+#pragma unroll
+  for (int x = 0; x < RT; ++x)
+#pragma unroll
+    for (int y = 0; y < KT; ++y) acc[x][y] = 0;
+  constexpr int kUnroll = RT * KT <= 8 ? 8 : 2;   // (few accumulators: more operand reads in flight)
+#pragma unroll kUnroll
+  for (int c = 0; c < D; c += 4) {
+    ulonglong2 b[KT];
+#pragma unroll
+    for (int y = 0; y < KT; ++y) b[y] = *reinterpret_cast<const ulonglong2*>(sB + (tx + 16 * y) * LD + c);
+    ulonglong2 a[RT];
+#pragma unroll
+    for (int x = 0; x < RT; ++x) a[x] = *reinterpret_cast<const ulonglong2*>(sA + (ty + TY * x) * LD + c);
+#pragma unroll
+    for (int x = 0; x < RT; ++x)   // (an accumulator's two products lie apart: the second waits for the first)
+#pragma unroll
+      for (int y = 0; y < KT; ++y) fma_pair(acc[x][y], a[x].x, b[y].x);
+#pragma unroll
+    for (int x = 0; x < RT; ++x)
+#pragma unroll
+      for (int y = 0; y < KT; ++y) fma_pair(acc[x][y], a[x].y, b[y].y);
+  }
+#pragma unroll
+  for (int x = 0; x < RT; ++x)
+#pragma unroll
+    for (int y = 0; y < KT; ++y) s[x][y] = lo_of(acc[x][y]) + hi_of(acc[x][y]);
 }
 
 template <typename T, int D>
@@ -70,219 +127,330 @@ __device__ inline const T* query_row_ptr(const CacheView& c, const BlockArgs& a,
 
 // ------------------------------------------------------------------------------------------------
 // Forward: out = softmax(scale * q k^T) v over the n_old cached pairs and the block's causal pairs.
-// Grid: (row tiles of the unit's I*g query rows, units).  Row r of a unit = (input r / g, head r % g).
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) attn_fwd_simt(CacheView c, BlockArgs a) {
-  constexpr int LD = D + 1;
-  extern __shared__ float sm[];
+// Grid: (row tiles of the unit's I*g query rows, units).  Row r of a unit = (input r / g, head r % g).  Thread (ty, tx)
+// owns rows ty + TY x of the tile, keys tx + 16 y of a key tile and output elements 4 tx + 64 y + [0, 4).
+template <int D, int RT, int NT>
+struct FwdSmem {
+  static constexpr int TY = NT / 16, TM = TY * RT, LD = D + 4, PLD = kTN / 2 + 4;
+  static constexpr int kFloats = TM * LD + kTN * LD + kTN * D + TM * PLD;
+  static constexpr size_t kBytes = sizeof(float) * kFloats + sizeof(int) * kTN;   // 108 KB at TM = 64, D = 128: two CTAs per SM
+};
+
+template <typename T, int D, int RT, int NT>
+__global__ void __launch_bounds__(NT, 2) attn_fwd_simt(CacheView c, BlockArgs a) {
+  using L = FwdSmem<D, RT, NT>;
+  constexpr int TY = L::TY, TM = L::TM, LD = L::LD, PLD = L::PLD, CT = D / 64;
+  extern __shared__ __align__(16) float sm[];
   float* sQ = sm;
-  float* sKV = sQ + kTile * LD;
-  float* sS = sKV + kTile * LD;        // [64][65]
-  float* sM = sS + kTile * (kTile + 1);
-  float* sL = sM + kTile;
-  float* sAl = sL + kTile;
-  int* sKp = reinterpret_cast<int*>(sAl + kTile);   // [64] 1 = the tile's key is a padding pair
+  float* sK = sQ + TM * LD;
+  float* sV = sK + kTN * LD;
+  float* sP = sV + kTN * D;                         // [TM][PLD]: the probabilities of half a key tile
+  int* sKp = reinterpret_cast<int*>(sP + TM * PLD);  // [kTN] 1 = the tile's key is a padding pair
 
   const int unit = blockIdx.y, smp = unit / c.Hkv, kh = unit % c.Hkv;
   const int pad = sample_left_pad(c, smp);
-  const int R = a.I * c.g, row0 = blockIdx.x * kTile;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31, warp = tid >> 5;
-
-  load_tile<T, D>(sQ, tid, [&](int r) { return query_row_ptr<T, D>(c, a, smp, kh, row0 + r); });
-  if (tid < kTile) { sM[tid] = -INFINITY; sL[tid] = 0.f; }
-
-  float o[4][D / 16];
-#pragma unroll
-  for (int x = 0; x < 4; ++x)
-#pragma unroll
-    for (int y = 0; y < D / 16; ++y) o[x][y] = 0.f;
-
-  const int last_row = min(R - 1, row0 + kTile - 1);
+  // (row tiles are handed out last first: a later tile sees more of the block's own keys)
+  const int R = a.I * c.g, row0 = (gridDim.x - 1 - blockIdx.x) * TM;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int last_row = min(R - 1, row0 + TM - 1);
   const int n_keys = c.n_old + last_row / c.g + 1;  // keys visible to the tile's last row
-  for (int j0 = 0; j0 < n_keys; j0 += kTile) {
-    __syncthreads();  // previous iteration finished with sKV / sS
-    load_tile<T, D>(sKV, tid, [&](int r) { return key_row_ptr<T, D>(c, c.k_slab, a.k, unit, smp, kh, a.I, j0 + r); });
-    if (tid < kTile) {
-      const int j = j0 + tid;
-      int is_pad = 0;
-      if (pad > 0 && j < c.n_old + a.I)
-        is_pad = (j < c.n_old ? c.kv_ids[(size_t)unit * c.cap + j] : a.pos0 + (j - c.n_old)) < pad;
-      sKp[tid] = is_pad;
-    }
-    __syncthreads();
-    float acc[4][4];
-    dot_tile<D>(sQ, sKV, ty, tx, acc);
+
+  auto load_k = [&](int j0) {
+    load_rows<T, D, LD, kTN, NT>(sK, tid, [&](int r) { return key_row_ptr<T, D>(c, c.k_slab, a.k, unit, smp, kh, a.I, j0 + r); });
+  };
+  auto load_v = [&](int j0) {
+    load_rows<T, D, D, kTN, NT>(sV, tid, [&](int r) { return key_row_ptr<T, D>(c, c.v_slab, a.v, unit, smp, kh, a.I, j0 + r); });
+  };
+  load_rows<T, D, LD, TM, NT>(sQ, tid, [&](int r) { return query_row_ptr<T, D>(c, a, smp, kh, row0 + r); });
+  load_k(0);
+  load_v(0);
+
+  f32x2 o[RT][2 * CT];
+  float m[RT], l[RT];                               // running maximum of a row; this thread's share of its sum
+  int vis[RT];
+  bool real[RT];
 #pragma unroll
-    for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < RT; ++x) {
+    const int row = row0 + ty + TY * x;
+    m[x] = -INFINITY;
+    l[x] = 0.f;
+    vis[x] = row < R ? c.n_old + row / c.g + 1 : 1;
+    // a real query does not see padding pairs; a padding query's row is computed over everything and dropped
+    real[x] = row < R && a.pos0 + row / c.g >= pad;
 #pragma unroll
-      for (int y = 0; y < 4; ++y) sS[(ty + 16 * x) * (kTile + 1) + tx + 16 * y] = acc[x][y] * a.scale;
-    __syncthreads();
-    load_tile<T, D>(sKV, tid, [&](int r) { return key_row_ptr<T, D>(c, c.v_slab, a.v, unit, smp, kh, a.I, j0 + r); });
-    // online softmax: warp w owns rows 8w .. 8w+7, lane owns columns lane and lane+32
-    for (int rr = 0; rr < 8; ++rr) {
-      const int r = warp * 8 + rr, row = row0 + r;
-      const int vis = (row < R) ? (c.n_old + row / c.g + 1) : 1;
-      // a real query does not see padding pairs; a padding query's row is computed over everything and dropped
-      const bool real = (row < R) && (a.pos0 + row / c.g >= pad);
-      const bool ok0 = (j0 + lane) < vis && !(real && sKp[lane]);
-      const bool ok1 = (j0 + lane + 32) < vis && !(real && sKp[lane + 32]);
-      const float s0 = ok0 ? sS[r * (kTile + 1) + lane] : -INFINITY;
-      const float s1 = ok1 ? sS[r * (kTile + 1) + lane + 32] : -INFINITY;
-      float mt = fmaxf(s0, s1);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, off));
-      const float m_old = sM[r];
-      const float m_new = fmaxf(m_old, mt);
-      const float p0 = ok0 ? expf(s0 - m_new) : 0.f;
-      const float p1 = ok1 ? expf(s1 - m_new) : 0.f;
-      float ps = p0 + p1;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, off);
-      const float alpha = (m_new == -INFINITY) ? 1.f : expf(m_old - m_new);
-      __syncwarp();
-      sS[r * (kTile + 1) + lane] = p0;
-      sS[r * (kTile + 1) + lane + 32] = p1;
-      if (lane == 0) { sM[r] = m_new; sL[r] = sL[r] * alpha + ps; sAl[r] = alpha; }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const float al = sAl[ty + 16 * x];
-#pragma unroll
-      for (int y = 0; y < D / 16; ++y) o[x][y] *= al;
-    }
-#pragma unroll 4
-    for (int j = 0; j < kTile; ++j) {
-      float pv[4], vv[D / 16];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) pv[x] = sS[(ty + 16 * x) * (kTile + 1) + j];
-#pragma unroll
-      for (int y = 0; y < D / 16; ++y) vv[y] = sKV[j * LD + tx + 16 * y];
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < D / 16; ++y) o[x][y] = fmaf(pv[x], vv[y], o[x][y]);
-    }
+    for (int y = 0; y < 2 * CT; ++y) o[x][y] = 0;
   }
-  __syncthreads();
+
+  for (int j0 = 0; j0 < n_keys; j0 += kTN) {
+    const bool more = j0 + kTN < n_keys;
+    wait_copies<1>();                               // K has arrived (and Q)
+    if (pad > 0 && tid < kTN) {
+      const int j = j0 + tid;
+      sKp[tid] = j < c.n_old + a.I && (j < c.n_old ? c.kv_ids[(size_t)unit * c.cap + j] : a.pos0 + (j - c.n_old)) < pad;
+    }
+    __syncthreads();
+    float s[RT][4];
+    dot_rows<D, LD, TY, RT, 4>(sQ, sK, ty, tx, s);
+    int padded[4];
 #pragma unroll
-  for (int x = 0; x < 4; ++x) {
-    const int r = ty + 16 * x, row = row0 + r;
+    for (int y = 0; y < 4; ++y) padded[y] = pad > 0 ? sKp[tx + 16 * y] : 0;
+    __syncthreads();                                // K's place is free
+    if (more) load_k(j0 + kTN);
+    else commit_nothing();
+#pragma unroll
+    for (int x = 0; x < RT; ++x) {
+      float mt = -INFINITY;
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        const bool ok = j0 + tx + 16 * y < vis[x] && !(real[x] && padded[y]);
+        s[x][y] = ok ? s[x][y] * a.scale : -INFINITY;
+        mt = fmaxf(mt, s[x][y]);
+      }
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, off));
+      const float m_new = fmaxf(m[x], mt);
+      const float alpha = m_new == -INFINITY ? 1.f : expf(m[x] - m_new);
+      m[x] = m_new;
+      float ps = 0.f;
+#pragma unroll
+      for (int y = 0; y < 4; ++y) {
+        s[x][y] = s[x][y] == -INFINITY ? 0.f : expf(s[x][y] - m_new);
+        ps += s[x][y];
+      }
+      l[x] = l[x] * alpha + ps;
+      const f32x2 al = dup(alpha);
+#pragma unroll
+      for (int y = 0; y < 2 * CT; ++y) o[x][y] = mul_pair(o[x][y], al);
+    }
+    wait_copies<1>();                               // V has arrived
+    __syncthreads();
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {          // rows of P are written and read by the same half warp
+#pragma unroll
+      for (int x = 0; x < RT; ++x) {
+        sP[(ty + TY * x) * PLD + tx] = s[x][2 * half];
+        sP[(ty + TY * x) * PLD + tx + 16] = s[x][2 * half + 1];
+      }
+      __syncwarp();
+#pragma unroll (RT <= 2 ? 4 : 1)
+      for (int k = 0; k < kTN / 2; k += 4) {
+        float4 p[RT];
+#pragma unroll
+        for (int x = 0; x < RT; ++x) p[x] = *reinterpret_cast<const float4*>(sP + (ty + TY * x) * PLD + k);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          ulonglong2 v[CT];
+#pragma unroll
+          for (int y = 0; y < CT; ++y)
+            v[y] = *reinterpret_cast<const ulonglong2*>(sV + (half * (kTN / 2) + k + kk) * D + 4 * tx + 64 * y);
+#pragma unroll
+          for (int x = 0; x < RT; ++x) {
+            const f32x2 pp = dup(kk == 0 ? p[x].x : kk == 1 ? p[x].y : kk == 2 ? p[x].z : p[x].w);
+#pragma unroll
+            for (int y = 0; y < CT; ++y) {
+              fma_pair(o[x][2 * y], pp, v[y].x);
+              fma_pair(o[x][2 * y + 1], pp, v[y].y);
+            }
+          }
+        }
+      }
+      __syncwarp();
+    }
+    __syncthreads();                                // V's place is free
+    if (more) load_v(j0 + kTN);
+    else commit_nothing();
+  }
+#pragma unroll
+  for (int x = 0; x < RT; ++x) {
+    const int row = row0 + ty + TY * x;
+    float lt = l[x];
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) lt += __shfl_xor_sync(0xffffffffu, lt, off);
     if (row >= R) continue;
     const int i = row / c.g, h = row % c.g;
-    const bool real = a.pos0 + i >= pad;          // a padding query: zero output, and +inf so that it has no weights
-    const float inv = real ? 1.f / sL[r] : 0.f;
+    const float inv = real[x] ? 1.f / lt : 0.f;     // a padding query: zero output, and +inf so that it has no weights
     T* op = reinterpret_cast<T*>(a.out) + ((size_t)(smp * a.I + i) * c.Hq + kh * c.g + h) * D;
 #pragma unroll
-    for (int y = 0; y < D / 16; ++y) op[tx + 16 * y] = Elem<T>::to_out(o[x][y] * inv);
-    if (tx == 0) a.lse[(size_t)unit * R + row] = real ? sM[r] + logf(sL[r]) : INFINITY;
+    for (int y = 0; y < CT; ++y) {
+      const float w[4] = {lo_of(o[x][2 * y]) * inv, hi_of(o[x][2 * y]) * inv, lo_of(o[x][2 * y + 1]) * inv,
+                          hi_of(o[x][2 * y + 1]) * inv};
+      T* to = op + 4 * tx + 64 * y;
+      if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(to) = make_float4(w[0], w[1], w[2], w[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) to[e] = Elem<T>::to_out(w[e]);
+      }
+    }
+    if (tx == 0) a.lse[(size_t)unit * R + row] = real[x] ? m[x] + logf(lt) : INFINITY;
   }
 }
 
 // ------------------------------------------------------------------------------------------------
 // Score pass: for every candidate pair j (cached or new) the column sum over all query rows of the
 // block of exp(scale * q.k_j - lse_row), i.e. sum_i attn_weights[i][j] added over the group's heads.
-// Grid: (key tiles, units).  Sums are formed in a fixed order (deterministic, no float atomics).
-template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) score_simt(CacheView c, BlockArgs a) {
-  constexpr int LD = D + 1;
-  extern __shared__ float sm[];
-  float* sQ = sm;
-  float* sK = sQ + kTile * LD;
-  float* sRed = sK + kTile * LD;  // [16][64]
-  float* sLse = sRed + 16 * kTile;
+// Grid: (tiles of 16 KT keys, units); query tiles of TM rows, the next one on its way while one is multiplied.
+// Sums are formed in a fixed order (deterministic, no float atomics).
+template <int D, int KT, int RT, int NT>
+struct ScoreSmemSimt {
+  static constexpr int TY = NT / 16, TM = TY * RT, LD = D + 4, kKeys = 16 * KT;
+  static constexpr size_t kBytes = sizeof(float) * (kKeys * LD + 2 * TM * LD + 2 * TM + TY * kKeys);
+};
+
+template <typename T, int D, int KT, int RT, int NT>
+__global__ void __launch_bounds__(NT, 2) score_simt(CacheView c, BlockArgs a) {
+  using L = ScoreSmemSimt<D, KT, RT, NT>;
+  constexpr int TY = L::TY, TM = L::TM, LD = L::LD, NK = L::kKeys;
+  extern __shared__ __align__(16) float sm[];
+  float* sK = sm;
+  float* sQ = sK + NK * LD;                         // [2] tiles
+  float* sLse = sQ + 2 * TM * LD;                  // [2][TM]
+  float* sRed = sLse + 2 * TM;                     // [TY][NK]
 
   const int unit = blockIdx.y, smp = unit / c.Hkv, kh = unit % c.Hkv;
-  const int R = a.I * c.g, j0 = blockIdx.x * kTile, n_c = c.n_old + a.I;
+  uint32_t rank, C;                                 // CTAs of a cluster share a key tile and take its query tiles in turn
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  const int R = a.I * c.g, j0 = blockIdx.x / C * NK, n_c = c.n_old + a.I;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-
-  load_tile<T, D>(sK, tid, [&](int r) { return key_row_ptr<T, D>(c, c.k_slab, a.k, unit, smp, kh, a.I, j0 + r); });
-  float col[4] = {0.f, 0.f, 0.f, 0.f}, col_sq[4] = {0.f, 0.f, 0.f, 0.f};
   const int counted_from = rule_first_counted_row(c.rule, c.window, a.I, c.g);   // rules that look at the last queries only
   const int first_row = (j0 > c.n_old) ? (j0 - c.n_old) * c.g : 0;  // earlier rows cannot see this tile
-  for (int row0 = (first_row / kTile) * kTile; row0 < R; row0 += kTile) {
-    __syncthreads();
-    load_tile<T, D>(sQ, tid, [&](int r) { return query_row_ptr<T, D>(c, a, smp, kh, row0 + r); });
-    if (tid < kTile)
-      sLse[tid] = (row0 + tid < R && row0 + tid >= counted_from) ? a.lse[(size_t)unit * R + row0 + tid] : INFINITY;
-    __syncthreads();
-    float acc[4][4];
-    dot_tile<D>(sQ, sK, ty, tx, acc);
+  const int first_tile = (first_row / TM + (int)rank) * TM, step = (int)C * TM;
+
+  auto load_q = [&](int row0, int b) {
+    load_rows<T, D, LD, TM, NT>(sQ + b * TM * LD, tid, [&](int r) { return query_row_ptr<T, D>(c, a, smp, kh, row0 + r); });
+    if (tid < TM)
+      sLse[b * TM + tid] = (row0 + tid < R && row0 + tid >= counted_from) ? a.lse[(size_t)unit * R + row0 + tid] : INFINITY;
+  };
+  load_rows<T, D, LD, NK, NT>(sK, tid, [&](int r) { return key_row_ptr<T, D>(c, c.k_slab, a.k, unit, smp, kh, a.I, j0 + r); });
+  load_q(first_tile, 0);
+  float col[KT], col_sq[KT];
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int j = j0 + tx + 16 * y;
-      float part = 0.f, part_sq = 0.f;
+  for (int y = 0; y < KT; ++y) col[y] = col_sq[y] = 0.f;
+  int b = 0;
+  for (int row0 = first_tile; row0 < R; row0 += step, b ^= 1) {
+    if (row0 + step < R) load_q(row0 + step, b ^ 1);   // (its place was last read before the barrier that ended the previous tile)
+    else commit_nothing();
+    wait_copies<1>();
+    __syncthreads();
+    float s[RT][KT];
+    dot_rows<D, LD, TY, RT, KT>(sQ + b * TM * LD, sK, ty, tx, s);
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int r = ty + 16 * x, row = row0 + r;
-        const bool vis = (row < R) && (j < c.n_old + row / c.g + 1);
-        const float w = vis ? expf(acc[x][y] * a.scale - sLse[r]) : 0.f;
-        part += w;
-        part_sq = fmaf(w, w, part_sq);
+    for (int x = 0; x < RT; ++x) {
+      const int row = row0 + ty + TY * x;
+      const float lse = sLse[b * TM + ty + TY * x];
+      const int vis = row < R ? c.n_old + row / c.g + 1 : 0;
+#pragma unroll
+      for (int y = 0; y < KT; ++y) {
+        const float w = j0 + tx + 16 * y < vis ? expf(s[x][y] * a.scale - lse) : 0.f;
+        col[y] += w;
+        col_sq[y] = fmaf(w, w, col_sq[y]);
       }
-      col[y] += part;
-      col_sq[y] += part_sq;
     }
+    __syncthreads();
   }
-  __syncthreads();
+  // sum of key tid over the TY groups of rows of every CTA of the cluster (CTA 0's copy is used), in a fixed order
+  auto reduce = [&](const float (&v)[KT]) {
 #pragma unroll
-  for (int y = 0; y < 4; ++y) sRed[ty * kTile + tx + 16 * y] = col[y];
-  __syncthreads();
-  if (tid < kTile) {
-    const int j = j0 + tid;
-    if (j < n_c) {
-      float tot = 0.f;
+    for (int y = 0; y < KT; ++y) sRed[ty * NK + tx + 16 * y] = v[y];
+    __syncthreads();
+    float tot = 0.f;
+    if (tid < NK)
 #pragma unroll
-      for (int t = 0; t < 16; ++t) tot += sRed[t * kTile + tid];
-      const int pad = sample_left_pad(c, smp);
-      if (pad > 0 && (j < c.n_old ? c.kv_ids[(size_t)unit * c.cap + j] : a.pos0 + (j - c.n_old)) < pad)
-        tot = 0.f;                                  // a padding pair is masked for every query
-      if (j < c.n_old) {
-        if (rule_overwrites(c.rule)) c.sum_weights[(size_t)unit * c.cap + j] = tot;   // nothing is carried over
-        else c.sum_weights[(size_t)unit * c.cap + j] += tot;
-      }
-      else a.new_sum[(size_t)unit * a.I + (j - c.n_old)] = tot;
+      for (int t = 0; t < TY; ++t) tot += sRed[t * NK + tid];
+    __syncthreads();
+    if (C > 1) {
+      if (tid < NK) sRed[tid] = tot;
+      cluster_barrier();
+      if (rank == 0 && tid < NK)
+        for (uint32_t p = 1; p < C; ++p) tot += ld_peer(&sRed[tid], p);
+      cluster_barrier();                             // nobody leaves, or writes again, before the sums have been read
     }
+    return tot;
+  };
+  float tot = reduce(col);
+  const int j = j0 + tid;
+  const bool mine = rank == 0 && tid < NK && j < n_c;
+  if (mine) {
+    const int pad = sample_left_pad(c, smp);
+    if (pad > 0 && (j < c.n_old ? c.kv_ids[(size_t)unit * c.cap + j] : a.pos0 + (j - c.n_old)) < pad)
+      tot = 0.f;                                    // a padding pair is masked for every query
+    if (j < c.n_old) {
+      if (rule_overwrites(c.rule)) c.sum_weights[(size_t)unit * c.cap + j] = tot;   // nothing is carried over
+      else c.sum_weights[(size_t)unit * c.cap + j] += tot;
+    }
+    else a.new_sum[(size_t)unit * a.I + (j - c.n_old)] = tot;
   }
   if (c.sum_sq != nullptr) {    // rule 4: the same reduction over the squares
-    __syncthreads();
-#pragma unroll
-    for (int y = 0; y < 4; ++y) sRed[ty * kTile + tx + 16 * y] = col_sq[y];
-    __syncthreads();
-    if (tid < kTile && j0 + tid < n_c) {
-      const int j = j0 + tid;
-      float tot = 0.f;
-#pragma unroll
-      for (int t = 0; t < 16; ++t) tot += sRed[t * kTile + tid];
+    tot = reduce(col_sq);
+    if (mine) {
       if (j < c.n_old) c.sum_sq[(size_t)unit * c.cap + j] += tot;
       else a.new_sq[(size_t)unit * a.I + (j - c.n_old)] = tot;
     }
   }
 }
 
-template <typename T, int D>
-cudaError_t launch_attn_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (2 * kTile * (D + 1) + kTile * (kTile + 1) + 4 * kTile);
+template <typename T, int D, int RT, int NT>
+cudaError_t launch_attn_rt(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+  using L = FwdSmem<D, RT, NT>;
   static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(attn_fwd_simt<T, D>, (size_t)(smem)); e != cudaSuccess) return e;
-  const int R = a.I * c.g;
-  dim3 grid((R + kTile - 1) / kTile, c.nsamples * c.Hkv);
+  if (cudaError_t e = configured.ensure(attn_fwd_simt<T, D, RT, NT>, L::kBytes); e != cudaSuccess) return e;
+  dim3 grid((a.I * c.g + L::TM - 1) / L::TM, c.nsamples * c.Hkv);
   ProfileScope prof(kAttnFwd, st);
-  attn_fwd_simt<T, D><<<grid, kThreads, smem, st>>>(c, a);
+  attn_fwd_simt<T, D, RT, NT><<<grid, NT, L::kBytes, st>>>(c, a);
   count_launch();
   return cudaGetLastError();
 }
 
+// Rows per tile: as many as still give every SM a CTA (small tiles re-read K and V more often and multiply fewer rows per
+// operand read, but leave no SM idle).  2 samples, 4 heads, d = 64, 64 inputs against 128 pairs: 45 us with tiles of 64
+// rows (8 CTAs), 16 us with tiles of 8 (64 CTAs); 2 samples, 16 heads in groups of 4, 128 inputs against 512 pairs: 201
+// us with 64 rows (64 CTAs), 82 us with 16 (256 CTAs).
+template <typename T, int D>
+cudaError_t launch_attn_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    const int rows = a.I * c.g, units = c.nsamples * c.Hkv;
+    auto fills = [&](int tm) { return (rows + tm - 1) / tm * units >= sm_count(); };
+    if (!fills(16)) return launch_attn_rt<T, D, 1, 128>(c, a, st);
+    if (!fills(64)) return launch_attn_rt<T, D, 2, 128>(c, a, st);
+  }
+  return launch_attn_rt<T, D, 4, 256>(c, a, st);
+}
+
+template <typename T, int D, int KT, int RT, int NT>
+cudaError_t launch_score_kt(const CacheView& c, const BlockArgs& a, int cluster, cudaStream_t st) {
+  using L = ScoreSmemSimt<D, KT, RT, NT>;
+  static SmemConfigured configured;
+  if (cudaError_t e = configured.ensure(score_simt<T, D, KT, RT, NT>, L::kBytes); e != cudaSuccess) return e;
+  const dim3 grid((c.n_old + a.I + L::kKeys - 1) / L::kKeys * cluster, c.nsamples * c.Hkv);
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid;
+  lc.blockDim = dim3(NT);
+  lc.dynamicSmemBytes = L::kBytes;
+  lc.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  lc.attrs = attr;
+  lc.numAttrs = cluster > 1 ? 1 : 0;
+  ProfileScope prof(kScore, st);
+  const cudaError_t e = cudaLaunchKernelEx(&lc, score_simt<T, D, KT, RT, NT>, c, a);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Key tiles of 64; a grid of fewer than four CTAs per SM shares each key tile among a cluster as long as there are
+// query tiles to share (16 caches, 1024 query rows against 256 keys: 84 -> 45 us with clusters of 8; against 1536 keys
+// 261 -> 226 us with clusters of 2, 287 with none below two CTAs per SM), and takes key tiles of 16 if SMs would still be idle.
 template <typename T, int D>
 cudaError_t launch_score_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (2 * kTile * (D + 1) + 16 * kTile + kTile);
-  static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(score_simt<T, D>, (size_t)(smem)); e != cudaSuccess) return e;
-  dim3 grid((c.n_old + a.I + kTile - 1) / kTile, c.nsamples * c.Hkv);
-  ProfileScope prof(kScore, st);
-  score_simt<T, D><<<grid, kThreads, smem, st>>>(c, a);
-  count_launch();
-  return cudaGetLastError();
+  const int tiles = (c.n_old + a.I + 63) / 64 * c.nsamples * c.Hkv, q_tiles = (a.I * c.g + 63) / 64;
+  int cluster = 1;
+  while (cluster < 8 && 2 * cluster <= q_tiles && tiles * cluster < 4 * sm_count()) cluster *= 2;
+  if constexpr (sizeof(T) == 4)
+    if (tiles * cluster < sm_count()) return launch_score_kt<T, D, 1, 4, 256>(c, a, cluster, st);
+  return launch_score_kt<T, D, 4, 4, 256>(c, a, cluster, st);
 }
 
 }  // namespace

@@ -255,6 +255,18 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", [
+    (1, 1, 1, 64, 7, 30),       # one tile of 8 rows, keys past the end
+    (2, 4, 2, 128, 65, 64),     # tiles of 8 rows; key tiles of 16 in the score pass
+    (3, 6, 4, 64, 77, 50),      # tiles of 16 rows; a cluster shares the query tiles of a key tile
+    (2, 3, 8, 128, 130, 70),    # ... a cluster of 8 with a ragged last query tile
+    (5, 8, 4, 128, 100, 129),   # tiles of 64 rows
+])
+def test_f32_kernels_by_grid_size(b, Hkv, g, d, B, K):
+    wl = tiny("f32_grid", b=b, Hq=g * Hkv, Hkv=Hkv, s=2 * B + 9, B=B, K=K, steps=2, dtype="f32", d=d)
+    run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1)
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
     (1, 3, 1, 64, 40, {}),                                  # less than one tile of rows
     (1, 2, 4, 128, 1023, {}),                               # a cluster of 8 CTAs per cache; the step's row ends a tile
