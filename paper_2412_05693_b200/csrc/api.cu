@@ -215,6 +215,8 @@ CacheView make_view(const bm_cache* c, int layer, int sample0, int nsamples, int
   v.fill = c->cfg.compaction == BM_COMPACT_FILL ? 1 : 0;
   v.sum_sq = c->sum_sq != nullptr ? c->sum_sq + row0 : nullptr;
   v.window = c->cfg.window; v.pool = c->cfg.pool; v.std_permille = c->cfg.std_share_permille;
+  v.layer_units = c->cfg.batch * c->cfg.n_kv_heads;
+  v.in_l2 = per_sample_bytes(&c->cfg) * (size_t)c->cfg.batch <= (size_t)60 << 20;
   v.moved = c->count_moves ? reinterpret_cast<unsigned long long*>(c->status + 16) : nullptr;
   return v;
 }

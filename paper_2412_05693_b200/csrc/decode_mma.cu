@@ -702,22 +702,23 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 }
 
 // Which kernel takes a step.  Measured, us per step (stream against this file's kernels; d = 128, g = 4, one pair leaves):
-// 128 caches of 512 pairs 10.5 / 10.1, of 700 pairs 12.5 / 14.6 (the instance with K in registers ends at 640 pairs);
+// at most one cache per SM -- 8 caches of 512 pairs 7.7 / 8.7, 32 caches 8.7 / 11.5, 128 caches 10.9 / 12.9, of 256
+// pairs 7.9 / 8.9; with the caches in L2 (a handle of few layers) 32 caches of 512 pairs 9.1 / 9.1, 64 caches 9.5 / 9.1,
+// 128 caches 10.2 / 9.5, where this file's instance with K in registers is ahead (it ends at 640 pairs).  More caches --
 // 256 caches of 384 pairs 14.5 / 14.4, of 1024 pairs 30.8 / 34.2; 640 caches of 256 pairs 26.8 / 24.9, of 384 pairs
-// 31.8 / 41.7; 1024 caches of 1024 pairs 95 / 112; at d = 64 128 caches of 256 pairs 6.5 / 7.1, 1024 caches of 512 pairs
-// 40.5 / 42.3, of 700 pairs 46 / 55.  So: a cache for every SM at most -- the stream unless all of K fits the registers;
-// beyond that the stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next
-// cache's bytes: 150 KB, or 256 KB while the other kernel holds every cache of the call at once (two CTAs per SM).
-static bool stream_is_faster(int d, int n1, int units) {
+// 31.8 / 41.7; 1024 caches of 1024 pairs 95 / 112; at d = 64 1024 caches of 512 pairs 40.5 / 42.3, of 700 pairs 46 / 55:
+// the stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes,
+// 150 KB, or 256 KB while the other kernel holds every cache of the call at once (two CTAs per SM).
+static bool stream_is_faster(int d, int n1, int units, bool in_l2) {
   const int sms = sm_count();
-  if (units <= sms) return d == 64 || n1 > kBatchTiles * 128;
+  if (units <= sms) return d == 64 || n1 > kBatchTiles * 128 || !in_l2 || units <= sms / 4;
   return (size_t)n1 * d * 4 >= (units <= 2 * sms ? 256u : 150u) * 1024;
 }
 
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                               int32_t pos, float scale, int32_t target, cudaStream_t st) {
   const int n1 = c.n_old + 1;
-  if (stream_is_faster(d, n1, c.nsamples * c.Hkv)) {
+  if (stream_is_faster(d, n1, c.layer_units, c.in_l2 != 0)) {
     // exactly one pair leaves by a single ranking value per pair: inside the kernel; any other cut follows it
     const bool cut = target >= 0 && target < n1;
     const bool one = cut && target == n1 - 1 && !(c.fill && c.rule == 1) && c.rule < 3;

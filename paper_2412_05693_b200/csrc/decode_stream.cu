@@ -17,7 +17,8 @@
 //
 // What bounds it: HBM once there is a cache for every SM; below that the latency of one cache's chain (first tile ->
 // softmax -> last tile -> moves), which is what splitting a cache over a cluster shortens.  One pair leaving per step,
-// caches of 1024 pairs, d = 128, us per step against the kernel in decode_mma.cu: 8 caches (g = 4) 10.1 / 16.7, 128
+// caches of 1024 pairs, d = 128, us per step against the kernel in decode_mma.cu: 8 caches (g = 4) 8.3 / 15.4 (10.1 with
+// exchanges by plain remote stores and releasing arrivals, which wait for the sender's global stores), 128
 // caches 16.8 / 19.1, 1024 caches 95 / 112 (5.9 against 5.0 TB/s of algorithmic bytes), 3072 caches 267 / 304 (6.3 TB/s),
 // 1024 caches without groups 88 / 104 (6.3 TB/s).  Not kept: tiles of 32 KB with two tiles' fragments in flight per warp
 // (spills; 111 against 94 us at 1024 caches), the per-row loops four rows at a time (+2 to 8 %), sums and ids written by
@@ -61,10 +62,10 @@ struct StreamMaps {
 template <int D, int G>
 struct StreamSmem {
   static constexpr int TR = kTile / (2 * D);     // rows per tile: 64 (d = 128) or 128 (d = 64)
-  // barriers: ring full / empty (up to 16 stages each), K-move full, hole known, moves done, cluster exchanges [3]
+  // barriers: ring full / empty (up to 16 stages each), K-move full, hole known, moves done, cluster exchanges [3], the piece before has been read (V, K)
   static constexpr int kMaxStages = 16;
   static constexpr int B_FULL = 0, B_EMPTY = kMaxStages, B_KM = 2 * kMaxStages, B_HOLE = B_KM + kMoveTiles, B_MOVED = B_HOLE + 1,
-                       B_X = B_MOVED + 1, B_COUNT = B_X + 3;
+                       B_X = B_MOVED + 1, B_PREV = B_X + 3, B_COUNT = B_PREV + 2;
   static constexpr int kMisc = 4 * D + 16 * (kCWarps + kMaxCluster)              // first rows; minima
                                + 4 * (2 * kCWarps * G + kMaxCluster * 2 * G + G * D)   // maxima, sums, statistics, outputs
                                + 8 * B_COUNT + 8 + 4 * G + 64;                      // barriers, flags, slack
@@ -81,8 +82,15 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+// Stores into a peer's shared memory that count themselves on the peer's barrier `bar` (transaction bytes): the receiver
+// waits for the bytes, and the sender needs no release fence, which would wait for its outstanding global stores.
+__device__ __forceinline__ void st_peer(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_peer4(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(addr), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
@@ -230,7 +238,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
     for (int x = 0; x < kMoveTiles; ++x) mbar_init(&bars[L::B_KM + x], 1);
     mbar_init(&bars[L::B_HOLE], 1);
     mbar_init(&bars[L::B_MOVED], 2);
-    for (int x = 0; x < 3; ++x) mbar_init(&bars[L::B_X + x], C);
+    for (int x = 0; x < 5; ++x) mbar_init(&bars[L::B_X + x], 1);
     mbar_fence_init();
   }
   if (tid == kConsumers) {
@@ -246,6 +254,17 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   pdl_wait();
   pdl_release();
   const bool shift = a.evict_one && !c.fill;
+  // (x = 0: V, 1: K) This CTA has read the rows of its piece: the next one may move its first row to the last of them.
+  // The own first row goes there likewise, once the CTA before has said so.
+  auto first_row_up = [&](int x, T* slab, int hole, const uint4& own) {
+    __syncwarp();
+    if (rank + 1 < C && lane == 0) arrive_cluster(mapa(smem_u32(&bars[L::B_PREV + x]), rank + 1));
+    if (shift && rank > 0 && hole < r0) {
+      wait_cluster(&bars[L::B_PREV + x], 0, abort_flag, c.status);
+      if (lane < PR && row_ok(c, r0 - 1))   // (r0 may be the step's own pair)
+        st_global_16(slab + (size_t)(r0 - 1) * D + lane * 8, r0 == n_old ? own : reinterpret_cast<const uint4*>(s_first + (x == 0 ? D : 0))[lane]);
+    }
+  };
 
   if (warp == kCWarps) {
     // ---------------------------------------------------------------- producer
@@ -311,6 +330,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       const bool mine = c.fill && a.evict_one ? (hole >= r0 && hole < r0 + nr) : (has_new && !(shift && r0 == n_old));
       if (hole != n_old && mine && lane < PR && row_ok(c, dst))
         st_global_16(vslab + (size_t)dst * D + lane * 8, own);
+      if (C > 1) first_row_up(0, vslab, hole, own);
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[L::B_MOVED]);
     }
@@ -380,6 +400,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       const bool mine = c.fill && a.evict_one ? (hole >= r0 && hole < r0 + nr) : (has_new && !(shift && r0 == n_old));
       if (hole != n_old && mine && lane < PR && row_ok(c, dst))
         st_global_16(kslab + (size_t)dst * D + lane * 8, own);
+      if (C > 1) first_row_up(1, kslab, hole, own);
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[L::B_MOVED]);
     }
@@ -563,16 +584,16 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
 #pragma unroll
         for (int h = 0; h < G; ++h) f[h] = q_real ? 1.f / f[h] : 0.f;
       } else {
+        if (tid == 0) mbar_expect_tx(&bars[L::B_X], C * 2 * G * 4);
         if (tid < (int)C) {                                 // this CTA's statistics to every peer
-          const uint32_t dst = mapa(smem_u32(s_xstat + rank * 2 * G), tid);
+          const uint32_t dst = mapa(smem_u32(s_xstat + rank * 2 * G), tid), bar = mapa(smem_u32(&bars[L::B_X]), tid);
           float t[G];
           all_warps(s_wsum, t, [](float x, float y) { return x + y; });
 #pragma unroll
           for (int h = 0; h < G; ++h) {
-            st_cluster(dst + 4 * h, mc[h]);
-            st_cluster(dst + 4 * (G + h), t[h]);
+            st_peer(dst + 4 * h, mc[h], bar);
+            st_peer(dst + 4 * (G + h), t[h], bar);
           }
-          arrive_cluster(mapa(smem_u32(&bars[L::B_X]), tid));
         }
         wait_cluster(&bars[L::B_X], it & 1, abort_flag, c.status);
 #pragma unroll
@@ -646,13 +667,10 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         named_bar_sync(1, kConsumers);
         if (C == 1 || warp == 0) read_best(s_best, kCWarps);
         if (C > 1) {
-          if (tid < (int)C) {
-            const uint32_t dst = mapa(smem_u32(s_xbest + rank), tid);
-            st_cluster(dst, __uint_as_float(best_key));
-            st_cluster(dst + 4, __int_as_float(best_j));
-            st_cluster(dst + 8, __int_as_float(best_id));
-            arrive_cluster(mapa(smem_u32(&bars[L::B_X + 1]), tid));
-          }
+          if (tid == 0) mbar_expect_tx(&bars[L::B_X + 1], C * 16);
+          if (tid < (int)C)
+            st_peer4(mapa(smem_u32(s_xbest + rank), tid), best_key, (uint32_t)best_j, (uint32_t)best_id, 0u,
+                     mapa(smem_u32(&bars[L::B_X + 1]), tid));
           wait_cluster(&bars[L::B_X + 1], it & 1, abort_flag, c.status);
           read_best(s_xbest, (int)C);
         }
@@ -754,6 +772,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
             }
       } else {
         const int dc = D / (int)C;                          // elements of every head that one CTA adds up
+        if (tid == 0) mbar_expect_tx(&bars[L::B_X + 2], G * D * 4);
         if (kg == 0)
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf)
@@ -763,25 +782,15 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
               float fh = 0.f;
 #pragma unroll
               for (int g = 0; g < G; ++g) fh = g == h ? f[g] : fh;
-              if (h < G) st_cluster(mapa(smem_u32(s_xout + ((int)rank * G + h) * dc + d % dc), d / dc), o[hf][hh] * fh);
+              if (h < G)
+                st_peer(mapa(smem_u32(s_xout + ((int)rank * G + h) * dc + d % dc), d / dc), o[hf][hh] * fh,
+                        mapa(smem_u32(&bars[L::B_X + 2]), d / dc));
             }
-        // the moves of this CTA are over as well: its peers may overwrite the row below its piece
-        mbar_wait(&bars[L::B_MOVED], it & 1, abort_flag, c.status);
-        named_bar_sync(1, kConsumers);
-        if (tid < (int)C) arrive_cluster(mapa(smem_u32(&bars[L::B_X + 2]), tid));
         wait_cluster(&bars[L::B_X + 2], it & 1, abort_flag, c.status);
         for (int x = tid; x < G * dc; x += kConsumers) {
           float t = 0.f;
           for (int p = 0; p < (int)C; ++p) t += s_xout[p * G * dc + x];   // fixed order
           op[(x / dc) * D + (int)rank * dc + x % dc] = __float2bfloat16_rn(t);
-        }
-        if (shift && rank > 0 && hole < r0 && tid < 2 * PR && row_ok(c, r0 - 1)) {   // the piece's first row, one row up
-          const bool is_v = tid >= PR;
-          const int pc = tid % PR;
-          T* slab = reinterpret_cast<T*>(is_v ? c.v_slab : c.k_slab) + base * D;
-          const T* own = reinterpret_cast<const T*>(is_v ? a.v : a.k) + (size_t)unit * D;   // r0 may be the step's own pair
-          const uint4 w = r0 == n_old ? ld_global_16(own + pc * 8) : reinterpret_cast<const uint4*>(s_first + (is_v ? D : 0))[pc];
-          st_global_16(slab + (size_t)(r0 - 1) * D + pc * 8, w);
         }
       }
       named_bar_sync(1, kConsumers);                        // the per-row arrays belong to the next cache
@@ -814,7 +823,7 @@ bool plan_for(int C, int n1, int units, int sms, Plan* p) {
   p->single = units <= sms;
   const int move = p->single ? 0 : kMoveTiles;
   const size_t fixed = L::total(p->rows, move);
-  if (fixed + 4 * kTile > kMaxDynamicSmem) return false;
+  if (L::total(p->rows, kMoveTiles + 4) > kMaxDynamicSmem) return false;   // (whatever the call's share of the caches)
   p->stages = (int)std::min<size_t>((kMaxDynamicSmem - fixed) / kTile, L::kMaxStages);
   p->keep_k = p->single && p->stages >= 2 * piece;
   if (p->keep_k) p->stages = 2 * piece;
@@ -822,21 +831,24 @@ bool plan_for(int C, int n1, int units, int sms, Plan* p) {
   return true;
 }
 
-// Cluster size.  A cluster shortens the time a cache takes to stream through one SM (about 60 KB per microsecond) and
-// costs its exchanges: a step over 8 caches of 1024 pairs (d = 128, g = 4) took 13.7, 13.4, 11.2 and 9.8 us with 1, 2,
-// 4 and 8 CTAs per cache, one over caches of 256 pairs 6.5 us with one CTA and 7.8 with four -- hence the constants.
+// Cluster size.  A cluster shortens the time a cache takes to pass through one SM and costs its exchanges.  us per step
+// with 1, 2, 4 and 8 CTAs per cache, d = 128, g = 4: 8 caches of 384 pairs 6.9 / 7.7 / 7.0 / 7.7, of 1024 pairs 12.6 /
+// 11.2 / 9.0 / 8.3; 32 caches of 1024 pairs 13.9 / 12.1 / 11.2; 64 caches of 700 pairs 10.7 / 11.5, of 1024 pairs 14.5 /
+// 13.3; at d = 64 8 caches of 1024 pairs 9.1 / 9.2 / 7.8 / 7.6 -- the line through these is the estimate below.
 // Only calls whose clusters are all resident at once are split (a GPC holds few clusters of 8: at 16 caches the second
-// wave made the step 1.7 times as long as with clusters of 4).
+// wave made the step 1.5 times as long as with clusters of 4), and the handle's caches of a layer decide, not the call's:
+// sample ranges of one batch may be in flight together and must sum in the same order as the whole batch.
 template <int D, int G>
-Plan choose_plan(int n1, int units, int sms) {
+Plan choose_plan(int n1, int units, int layer_units, int sms) {
   constexpr int kMostCaches[] = {0, 64, 32, 8};   // for C = 2, 4, 8 on 148 SMs
   Plan best;
   double best_us = 0;
   for (int x = 0, C = 1; C <= kMaxCluster; ++x, C *= 2) {
     Plan p;
-    if (C > 1 && (units > kMostCaches[x] || units * C > sms)) continue;
+    if (C > 1 && (layer_units > kMostCaches[x] || layer_units * C > sms)) continue;
     if (!plan_for<D, G>(C, n1, units, sms, &p)) continue;
-    const double us = (double)n1 * D * 4 / C / 60e3 + (C == 1 ? 5.0 : 8.7);
+    const double stream = n1 * (4.0 * D + 80) / C / 57e3;   // us: row bytes, and the work per row
+    const double us = stream + (C == 1 ? 3.2 : 6.0 + 0.1 * C + 1.5 * layer_units * C / sms);
     if (best.C == 0 || us < best_us) { best = p; best_us = us; }
   }
   return best;
@@ -845,7 +857,7 @@ Plan choose_plan(int n1, int units, int sms) {
 template <int D, int G>
 cudaError_t launch_stream(const CacheView& c, StreamArgs a, cudaStream_t st, bool* taken) {
   a.units = c.nsamples * c.Hkv;
-  const Plan p = choose_plan<D, G>(c.n_old + 1, a.units, sm_count());
+  const Plan p = choose_plan<D, G>(c.n_old + 1, a.units, c.layer_units, sm_count());
   if (p.C == 0) return cudaSuccess;
   a.stages = p.stages; a.single = p.single; a.keep_k = p.keep_k; a.rows_cta = p.rows;
   StreamMaps m;

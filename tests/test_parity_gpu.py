@@ -255,6 +255,30 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,d,K", [(2, 4, 128, 1024), (4, 8, 64, 1500), (24, 8, 128, 700)])
+def test_decode_stream_is_bitwise_independent_of_sample_ranges(b, Hkv, d, K):
+    import torch
+    from paper_2412_05693_b200 import BatchMaxCache, Config
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen).bfloat16()
+    prompt = (f(b, K, 2 * Hkv, d), f(b, K, Hkv, d), f(b, K, Hkv, d))
+    steps = [(f(b, 2 * Hkv, d), f(b, Hkv, d), f(b, Hkv, d)) for _ in range(3)]
+    runs = []
+    for parts in (1, 2, b):
+        cache = BatchMaxCache(Config(batch=b, n_q_heads=2 * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=K, block_max=K))
+        cache.prefill_block(*prompt, 0)
+        ns, outs = b // parts, []
+        for q, k, v in steps:
+            outs.append(torch.cat([cache.decode_step(q[s:s + ns], k[s:s + ns], v[s:s + ns], evict_to=K, sample0=s)
+                                   for s in range(0, b, ns)]))
+        assert cache.status() == 0
+        runs.append((outs, cache.export(0, b - 1, Hkv - 1, rows=True)))
+        cache.close()
+    for outs, state in runs[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(outs, runs[0][0]))
+        assert all(torch.equal(x, y) for x, y in zip(state, runs[0][1]))
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", [
     (1, 1, 1, 64, 7, 30),       # one tile of 8 rows, keys past the end
     (2, 4, 2, 128, 65, 64),     # tiles of 8 rows; key tiles of 16 in the score pass
