@@ -7,22 +7,46 @@ namespace {
 
 constexpr int kEvictThreads = 512;
 
-template <typename T, int D, bool FILL>
-__global__ void __launch_bounds__(kEvictThreads) evict_kernel(CacheView c, EvictArgs e) {
+template <typename T, int D, bool FILL, int W>
+__global__ void __launch_bounds__(kEvictThreads, W > 8 ? 1 : 2) evict_kernel(CacheView c, EvictArgs e) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int unit = blockIdx.x;
-  evict_body_impl<T, D, kEvictThreads, FILL>(c, unit, unit / c.Hkv, unit % c.Hkv, e, smem_raw);
+  uint32_t rank, count;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(count));
+  const int unit = blockIdx.x / count;
+  EvictShare share;
+  share.rank = (int)rank;
+  share.count = (int)count;
+  pdl_wait();
+  evict_body_impl<T, D, kEvictThreads, FILL, W>(c, unit, unit / c.Hkv, unit % c.Hkv, e, smem_raw, share);
 }
 
-template <typename T, int D, bool FILL>
-cudaError_t launch_f(const CacheView& c, const EvictArgs& e, cudaStream_t st) {
+template <typename T, int D, bool FILL, int W>
+cudaError_t launch_w(const CacheView& c, const EvictArgs& e, int cluster, cudaStream_t st) {
   const size_t smem = evict_smem_bytes(c.n_old + e.I, e.target);
   static SmemConfigured configured;
-  if (cudaError_t err = configured.ensure(evict_kernel<T, D, FILL>, smem); err != cudaSuccess) return err;
+  if (cudaError_t err = configured.ensure(evict_kernel<T, D, FILL, W>, smem); err != cudaSuccess) return err;
   ProfileScope prof(kEvict, st);
-  evict_kernel<T, D, FILL><<<c.nsamples * c.Hkv, kEvictThreads, smem, st>>>(c, e);
+  const cudaError_t err = launch_dependent_cluster(evict_kernel<T, D, FILL, W>, dim3(c.nsamples * c.Hkv * cluster),
+                                                   dim3(kEvictThreads), smem, cluster, st, c, e);
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
+}
+
+// A call of few caches shares each among a cluster, so that more SMs move rows -- at most 8 CTAs (64 bytes of a row
+// each), only clusters that are all resident at once, and at least 96 KB of rows for each CTA (a cluster's barrier costs
+// about 1 us).  Grids of at most one CTA per SM with more than a chunk of 64 KB to move keep twice as many pieces in
+// flight (a chunk is one round trip to memory).  us per call, against one CTA per cache with 64 KB chunks: 8 caches cut
+// from 1536 to 1024 pairs of 512 bytes 10.9 -> 8.6 (clusters of 8), 16 caches cut from 1024 to 512 pairs of 1 KB 12.2 ->
+// 8.7 (4), 32 caches of 1024 to 512 pairs of 512 bytes 9.5 -> 8.3 (4), 128 caches of 768 to 512 pairs 10.5 -> 10.0.
+template <typename T, int D, bool FILL>
+cudaError_t launch_f(const CacheView& c, const EvictArgs& e, cudaStream_t st) {
+  const int units = c.nsamples * c.Hkv, most = units <= 8 ? 8 : units <= 32 ? 4 : units <= 64 ? 2 : 1;
+  const size_t bytes = (size_t)e.target * D * 2 * sizeof(T);   // that may move per cache
+  int cluster = 1;
+  while (cluster < most && bytes > (size_t)cluster * (96 << 10)) cluster *= 2;
+  const bool wide = cluster * units <= sm_count() && bytes > (size_t)cluster * (64 << 10);
+  return wide ? launch_w<T, D, FILL, 16>(c, e, cluster, st) : launch_w<T, D, FILL, 8>(c, e, 1, st);
 }
 
 template <typename T, int D>

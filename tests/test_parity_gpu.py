@@ -255,6 +255,20 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,d,dtype,K,kw", [
+    (1, 2, 128, "bf16", 1100, {}),                          # clusters of 8, a ragged last chunk
+    (2, 8, 64, "bf16", 900, {}),                            # clusters of 2 (less than 96 KB of rows per further CTA)
+    (3, 8, 64, "f32", 700, {}),                             # clusters of 4
+    (1, 4, 128, "f32", 513, dict(compaction="fill")),       # unordered rows, shared among a cluster
+    (1, 4, 128, "bf16", 600, dict(rule="average_std")),     # the second accumulator is read after the first select
+    (1, 4, 128, "bf16", 600, dict(rule="window_pooled", rule_params=dict(window=16, pool=5))),
+    (20, 8, 128, "bf16", 130, {}),                          # more caches than SMs: small chunks
+])
+def test_evictions_by_grid_size(b, Hkv, d, dtype, K, kw):
+    wl = tiny("evict_grid", b=b, Hq=Hkv, Hkv=Hkv, s=K + 150, B=120, K=K, steps=2, dtype=dtype, d=d)
+    run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=2, **kw)
+
+
 @pytest.mark.parametrize("b,Hkv,d,K", [(2, 4, 128, 1024), (4, 8, 64, 1500), (24, 8, 128, 700)])
 def test_decode_stream_is_bitwise_independent_of_sample_ranges(b, Hkv, d, K):
     import torch
