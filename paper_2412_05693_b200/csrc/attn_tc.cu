@@ -7,6 +7,7 @@
 //                 in a fixed order (deterministic, no atomics).
 // Query rows of a unit are ordered r = i * g + h (input i, head h of the group), so a tile of 128 rows shares
 // its K/V tiles among the g heads of the group.
+#include <algorithm>
 #include <type_traits>
 
 #include "tc_common.cuh"
@@ -46,6 +47,7 @@ struct TcArgs {
   int rule;
   int first_row;     // query rows below it add nothing to the column sums (rules that look at the last queries only)
   int overwrite;     // 1: the column sums replace sum_weights instead of being added
+  int key_tiles;     // key tiles per CTA of the score pass (QRES)
   float* sum_sq;     // rule 4: sums of squared weights (cached pairs / the block's pairs), else null
   float* new_sq;
 };
@@ -54,7 +56,8 @@ struct TcArgs {
 #include "attn_onepass.cuh"
 
 // ------------------------------------------------------------------------------------------------------
-// Score pass.  CTA = (tile of 128 candidate keys, unit).  A = the key tile (loaded once), B = the unit's query
+// Score pass.  CTA = (tile of 128 candidate keys, unit), or with QRES (a single query tile) CTA = (run of key tiles,
+// unit): the query tile is loaded once and the key tiles are streamed.  A = the key tile (loaded once), B = the unit's query
 // tiles streamed through a ring; S^T lands in TMEM with lane = key, column = query row.  The pass is bound by
 // one exponential per visible pair, so two reducer warpgroups (one TMEM buffer each, query tiles taken round
 // robin) keep the special-function units busy; their partial sums are added in a fixed order.
@@ -77,7 +80,7 @@ enum { C_KFULL = 0, C_QFULL = 1, C_QEMPTY = C_QFULL + kQStages, C_SFULL = C_QEMP
        C_SFREE = C_SFULL + kScoreWG, C_COUNT = C_SFREE + kScoreWG };
 
 // SQ: the sums of squared weights are taken as well (rule 4; an instance of its own, so that the others carry none of it)
-template <int D, bool SQ, int EMU>
+template <int D, bool SQ, int EMU, bool QRES>
 __global__ void __launch_bounds__(kScoreThreads, 2)
 score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
   using L = ScoreSmem<D>;
@@ -94,27 +97,29 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
   const int unit = blockIdx.y, smp = unit / a.Hkv, kh = unit % a.Hkv;
   const int R = a.I * a.g;
   const int t_old = (a.n_old + kTileN - 1) / kTileN;
-  const int kt = blockIdx.x;                       // key tile: old tiles first, then the block's own
-  const bool is_old = kt < t_old;
-  const int c0 = is_old ? 0 : (kt - t_old) * kTileN;  // first block position of a new-key tile
-  const int qpt = kTileM / a.g;
   const int n_qt = (R + kTileM - 1) / kTileM;
-  const int qt0 = is_old ? 0 : c0 / qpt;           // earlier query tiles cannot see these keys
-  const int T = n_qt - qt0;
+  // key tiles in order: cached ones first, then the block's own.  kt0: the (first) key tile of this CTA
+  const int kt0 = QRES ? blockIdx.x * a.key_tiles : blockIdx.x;
+  const int qpt = kTileM / a.g;
+  const int qt0 = kt0 < t_old || QRES ? 0 : (kt0 - t_old) * kTileN / qpt;   // earlier query tiles cannot see a new-key tile
+  // items: query tiles qt0 + t against one key tile, or key tiles kt0 + t against one query tile
+  const int T = QRES ? min(a.key_tiles, t_old + (a.I + kTileN - 1) / kTileN - kt0) : n_qt - qt0;
 
-  auto load_k = [&]() {
-    mbar_expect_tx(&bars[C_KFULL], L::kTileBytes);
+  auto load_keys = [&](unsigned char* dst, int kt, uint64_t* bar) {
+    mbar_expect_tx(bar, L::kTileBytes);
     for (int c = 0; c < L::kChunks; ++c) {
-      if (is_old) tma_load_3d(sm + L::kK + c * 16384, &maps.k_slab, c * 64, kt * kTileN, unit, &bars[C_KFULL]);
-      else tma_load_4d(sm + L::kK + c * 16384, &maps.k_blk, c * 64, kh, c0, smp, &bars[C_KFULL]);
+      if (kt < t_old) tma_load_3d(dst + c * 16384, &maps.k_slab, c * 64, kt * kTileN, unit, bar);
+      else tma_load_4d(dst + c * 16384, &maps.k_blk, c * 64, kh, (kt - t_old) * kTileN, smp, bar);
     }
   };
-  auto load_q = [&](int t) {
-    const int s = t % kQStages;
-    mbar_expect_tx(&bars[C_QFULL + s], L::kTileBytes);
-    for (int c = 0; c < L::kChunks; ++c)
-      tma_load_5d(sm + L::kQ + s * L::kTileBytes + c * 16384, &maps.q, c * 64, 0, kh, (qt0 + t) * qpt, smp,
-                  &bars[C_QFULL + s]);
+  auto load_queries = [&](unsigned char* dst, int qt, uint64_t* bar) {
+    mbar_expect_tx(bar, L::kTileBytes);
+    for (int c = 0; c < L::kChunks; ++c) tma_load_5d(dst + c * 16384, &maps.q, c * 64, 0, kh, qt * qpt, smp, bar);
+  };
+  auto load_item = [&](int t) {          // of the streamed operand
+    unsigned char* dst = sm + L::kQ + (t % kQStages) * L::kTileBytes;
+    if (QRES) load_keys(dst, kt0 + t, &bars[C_QFULL + t % kQStages]);
+    else load_queries(dst, qt0 + t, &bars[C_QFULL + t % kQStages]);
   };
   if (warp == kTmaWarp && lane == 0) {   // barriers and the first loads before the CTA-wide barrier (overlaps TMEM allocation)
     *abort_flag = 0;
@@ -122,8 +127,9 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
     for (int s = 0; s < kQStages; ++s) { mbar_init(&bars[C_QFULL + s], 1); mbar_init(&bars[C_QEMPTY + s], 1); }
     for (int b = 0; b < kScoreWG; ++b) { mbar_init(&bars[C_SFULL + b], 1); mbar_init(&bars[C_SFREE + b], 128); }
     mbar_fence_init();
-    load_k();
-    for (int t = 0; t < min(kQStages, T); ++t) load_q(t);
+    if (QRES) load_queries(sm + L::kK, 0, &bars[C_KFULL]);
+    else load_keys(sm + L::kK, kt0, &bars[C_KFULL]);
+    for (int t = 0; t < min(kQStages, T); ++t) load_item(t);
   }
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, 128 * kScoreWG);
   tc_fence_before();
@@ -135,27 +141,31 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
     if (lane == 0) {
       for (int t = kQStages; t < T; ++t) {
         mbar_wait(&bars[C_QEMPTY + t % kQStages], ((t / kQStages) - 1) & 1, abort_flag, a.status);
-        load_q(t);
+        load_item(t);
       }
     }
   } else if (warp == kMmaWarp) {
     if (lane == 0) {
       const uint32_t idesc = instr_desc(kTileN, kTileM, 0, 0);
+      // (the last query tile: whole chunks of 32 columns up to its last row, as they are read back)
+      const uint32_t idesc_last = instr_desc(kTileN, (min(kTileM, R - (n_qt - 1) * kTileM) + 31) & ~31, 0, 0);
       const uint64_t d_hi = smem_desc(0, 16, 1024) & 0xffffffff00000000ull;
       const uint32_t d_lo = (uint32_t)(smem_desc(0, 16, 1024) & 0xffffffffull);
-      const uint32_t k_lo = d_lo + (smem_u32(sm + L::kK) >> 4);
+      const uint32_t res_lo = d_lo + (smem_u32(sm + L::kK) >> 4);   // resident operand
       mbar_wait(&bars[C_KFULL], 0, abort_flag, a.status);
       for (int t = 0; t < T; ++t) {
         const int s = t % kQStages, b = t % kScoreWG;
         mbar_wait(&bars[C_QFULL + s], (t / kQStages) & 1, abort_flag, a.status);
         if (t >= kScoreWG) mbar_wait(&bars[C_SFREE + b], ((t / kScoreWG) - 1) & 1, abort_flag, a.status);
         tc_fence_after();
-        const uint32_t q_lo = d_lo + ((smem_u32(sm + L::kQ) >> 4) + s * (L::kTileBytes >> 4));
+        const uint32_t str_lo = d_lo + ((smem_u32(sm + L::kQ) >> 4) + s * (L::kTileBytes >> 4));
+        const uint32_t k_lo = QRES ? str_lo : res_lo, q_lo = QRES ? res_lo : str_lo;
+        const uint32_t id = QRES || qt0 + t == n_qt - 1 ? idesc_last : idesc;
         const uint32_t ts = tmem + b * 128;
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {   // only the start-address word of the descriptors changes
           const uint32_t off = (ks >> 2) * 1024 + (ks & 3) * 2;
-          mma_ss(ts, d_hi | (k_lo + off), d_hi | (q_lo + off), idesc, ks > 0 ? 1u : 0u);
+          mma_ss(ts, d_hi | (k_lo + off), d_hi | (q_lo + off), id, ks > 0 ? 1u : 0u);
         }
         mma_commit(&bars[C_SFULL + b]);
         mma_commit(&bars[C_QEMPTY + s]);
@@ -168,10 +178,28 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
     const uint32_t ts = tmem + wg * 128 + ((uint32_t)(quad * 32) << 16);
     const float* lse_w = sLse + wg * 128;
     float acc = 0.f, acc_sq = 0.f;
+    // a key tile's column sums into their places
+    auto write_sums = [&](int kt, float tot, float tot_sq) {
+      const bool is_old = kt < t_old;
+      const int jk = is_old ? kt * kTileN + key : (kt - t_old) * kTileN + key;
+      if (jk >= (is_old ? a.n_old : a.I)) return;
+      if (a.left_pad != nullptr) {                  // a padding pair is masked for every query
+        const int pad = a.left_pad[smp];
+        if (pad > 0 && (is_old ? a.kv_ids[(size_t)unit * a.cap + jk] : a.pos0 + jk) < pad) tot = 0.f;
+      }
+      if (is_old) {
+        if (a.overwrite) a.sum_weights[(size_t)unit * a.cap + jk] = tot;   // nothing is carried over
+        else a.sum_weights[(size_t)unit * a.cap + jk] += tot;
+        if (SQ) a.sum_sq[(size_t)unit * a.cap + jk] += tot_sq;
+      } else {
+        a.new_sum[(size_t)unit * a.I + jk] = tot;
+        if (SQ) a.new_sq[(size_t)unit * a.I + jk] = tot_sq;
+      }
+    };
     for (int t = wg; t < T; t += kScoreWG) {
-      const int qrow0 = (qt0 + t) * kTileM;
-      // this tile's log2-sum-exp values; +inf for rows past the block's end (weight 0)
-      {
+      const int qrow0 = QRES ? 0 : (qt0 + t) * kTileM, kt = QRES ? kt0 + t : kt0;
+      // this query tile's log2-sum-exp values; +inf for rows past the block's end (weight 0)
+      if (!QRES || t == wg) {
         const int rr = qrow0 + key;
         sLse[wg * 128 + key] = (rr < R && rr >= a.first_row) ? a.lse2[(size_t)unit * R + rr] : INFINITY;
       }
@@ -179,8 +207,9 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
       mbar_wait(&bars[C_SFULL + wg], (t / kScoreWG) & 1, abort_flag, a.status);
       tc_fence_after();
       // first query row of the tile that may see this key (causal mask inside the block)
-      const int first_vis = is_old ? 0 : max(0, (c0 + key) * a.g - qrow0);
-      const bool nomask = __all_sync(0xffffffffu, first_vis == 0);
+      const int first_vis = kt < t_old ? 0 : max(0, ((kt - t_old) * kTileN + key) * a.g - qrow0);
+      const int ncols = min(kTileM, R - qrow0);    // query rows of the tile: no exponentials of chunks past them
+      const bool nomask = ncols == kTileM && __all_sync(0xffffffffu, first_vis == 0);
       float p0 = 0.f, p1 = 0.f, q0 = 0.f, q1 = 0.f;
       // (the loop exists with and without the causal mask: as one loop with a test inside, the compiler evaluated
       // the mask of every tile, two more instructions per exponential)
@@ -190,6 +219,7 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
         tmem_wait_ld();
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) {
+          if (decltype(masked)::value && cc * 32 >= ncols) break;
           if (cc < 3) tmem_ld32(ts + (cc + 1) * 32, nxt);   // next chunk loads while this one is used
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
@@ -215,39 +245,29 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
       };
       if (nomask) reduce_tile(std::false_type{});
       else reduce_tile(std::true_type{});
-      acc += p0 + p1;
-      if (SQ) acc_sq += q0 + q1;
       tc_fence_before();
       mbar_arrive(&bars[C_SFREE + wg]);
-      named_bar_sync(1 + wg, 128);                 // everyone is done with this tile's sLse before it is rewritten
+      if (QRES) {
+        write_sums(kt, p0 + p1, q0 + q1);
+      } else {
+        acc += p0 + p1;
+        if (SQ) acc_sq += q0 + q1;
+        named_bar_sync(1 + wg, 128);               // everyone is done with this tile's sLse before it is rewritten
+      }
     }
-    sPart[wg * 128 + key] = acc;
-    if (SQ) sLse[wg * 128 + key] = acc_sq;         // (the last tile's values are no longer needed: barrier above)
-    named_bar_sync(1 + kScoreWG, 128 * kScoreWG);
-    if (wg == 0) {
-      float tot = 0.f, tot_sq = 0.f;
+    if (!QRES) {
+      sPart[wg * 128 + key] = acc;
+      if (SQ) sLse[wg * 128 + key] = acc_sq;       // (the last tile's values are no longer needed: barrier above)
+      named_bar_sync(1 + kScoreWG, 128 * kScoreWG);
+      if (wg == 0) {
+        float tot = 0.f, tot_sq = 0.f;
 #pragma unroll
-      for (int w = 0; w < kScoreWG; ++w) tot += sPart[w * 128 + key];   // fixed order
-      if (SQ) {
+        for (int w = 0; w < kScoreWG; ++w) tot += sPart[w * 128 + key];   // fixed order
+        if (SQ) {
 #pragma unroll
-        for (int w = 0; w < kScoreWG; ++w) tot_sq += sLse[w * 128 + key];
-      }
-      const int j = is_old ? kt * kTileN + key : c0 + key;
-      if (a.left_pad != nullptr) {                  // a padding pair is masked for every query
-        const int pad = a.left_pad[smp];
-        const bool in_range = is_old ? j < a.n_old : j < a.I;
-        if (pad > 0 && in_range && (is_old ? a.kv_ids[(size_t)unit * a.cap + j] : a.pos0 + j) < pad) tot = 0.f;
-      }
-      if (is_old) {
-        if (j < a.n_old) {
-          if (a.overwrite) a.sum_weights[(size_t)unit * a.cap + j] = tot;   // nothing is carried over
-          else a.sum_weights[(size_t)unit * a.cap + j] += tot;
-          if (SQ) a.sum_sq[(size_t)unit * a.cap + j] += tot_sq;
+          for (int w = 0; w < kScoreWG; ++w) tot_sq += sLse[w * 128 + key];
         }
-      }
-      else if (j < a.I) {
-        a.new_sum[(size_t)unit * a.I + j] = tot;
-        if (SQ) a.new_sq[(size_t)unit * a.I + j] = tot_sq;
+        write_sums(kt0, tot, tot_sq);
       }
     }
   }
@@ -322,6 +342,7 @@ TcArgs make_args(const CacheView& c, const BlockArgs& a) {
   t.first_row = rule_first_counted_row(c.rule, c.window, a.I, c.g);
   t.overwrite = rule_overwrites(c.rule) ? 1 : 0;
   t.sum_sq = c.sum_sq; t.new_sq = a.new_sq;
+  t.key_tiles = 1;
   return t;
 }
 
@@ -370,14 +391,16 @@ cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st
   return c.left_pad != nullptr ? launch_fwd_split<D, true>(c, a, st) : launch_fwd_split<D, false>(c, a, st);
 }
 
-template <int D, bool SQ, int EMU>
-cudaError_t launch_score_emu(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+template <int D, bool SQ, int EMU, bool QRES>
+cudaError_t launch_score_emu(const CacheView& c, const BlockArgs& a, int key_tiles, cudaStream_t st) {
   static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(score_tc<D, SQ, EMU>, (size_t)(ScoreSmem<D>::kTotal)); e != cudaSuccess) return e;
+  if (cudaError_t e = configured.ensure(score_tc<D, SQ, EMU, QRES>, (size_t)(ScoreSmem<D>::kTotal)); e != cudaSuccess) return e;
   const int t_old = (c.n_old + kTileN - 1) / kTileN, t_new = (a.I + kTileN - 1) / kTileN;
-  dim3 grid(t_old + t_new, c.nsamples * c.Hkv);
+  dim3 grid((t_old + t_new + key_tiles - 1) / key_tiles, c.nsamples * c.Hkv);
+  TcArgs args = make_args(c, a);
+  args.key_tiles = key_tiles;
   ProfileScope prof(kScore, st);
-  score_tc<D, SQ, EMU><<<grid, kScoreThreads, ScoreSmem<D>::kTotal, st>>>(g_maps, make_args(c, a));
+  score_tc<D, SQ, EMU, QRES><<<grid, kScoreThreads, ScoreSmem<D>::kTotal, st>>>(g_maps, args);
   count_launch();
   return cudaGetLastError();
 }
@@ -388,7 +411,13 @@ cudaError_t launch_score_emu(const CacheView& c, const BlockArgs& a, cudaStream_
 constexpr int kScoreEmu = 4;
 template <int D, bool SQ>
 cudaError_t launch_score_sq(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
-  return launch_score_emu<D, SQ, kScoreEmu>(c, a, st);
+  if (a.I * c.g > kTileM) return launch_score_emu<D, SQ, kScoreEmu, false>(c, a, 1, st);
+  // A single query tile: a CTA per key tile would load the query tile as often as there are key tiles and be set up for
+  // one product each, so a CTA takes as many key tiles as leave two CTAs for every SM (640 caches of 960 pairs, 64
+  // query rows: 87 -> 41 us; 128 caches, 100 rows: 18 -> 14 us).
+  const int tiles = (c.n_old + kTileN - 1) / kTileN + (a.I + kTileN - 1) / kTileN, units = c.nsamples * c.Hkv;
+  const int parts = std::min(tiles, std::max(1, (2 * sm_count() + units - 1) / units));
+  return launch_score_emu<D, SQ, kScoreEmu, true>(c, a, (tiles + parts - 1) / parts, st);
 }
 template <int D>
 cudaError_t launch_score_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {

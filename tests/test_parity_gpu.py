@@ -255,6 +255,21 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,B,K,kw", [
+    (1, 2, 1, 128, 64, 700, {}),                            # one query tile, a key tile per CTA
+    (40, 8, 1, 64, 33, 530, {}),                            # ... all key tiles of a cache in one CTA, a chunk past the last row
+    (10, 8, 4, 128, 32, 640, {}),                           # ... exactly 128 rows, several key tiles per CTA
+    (2, 2, 8, 128, 16, 777, dict(rule="average_std")),
+    (2, 2, 2, 64, 50, 601, dict(rule="window_pooled", rule_params=dict(window=16, pool=5))),
+    (2, 2, 1, 128, 150, 600, {}),                           # two query tiles, the last with a single chunk of rows
+])
+def test_score_pass_of_short_blocks_against_long_caches(b, Hkv, g, d, B, K, kw):
+    wl = tiny("short_score", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 3 * B, B=B, K=K, steps=1, dtype="bf16", d=d)
+    calls = [("prefill", p, min(300, K - p), -1) for p in range(0, K, 300)]
+    calls += [("prefill", K + i * B, B, K) for i in range(3)]
+    run_lockstep(wl.with_(B=300), [(0, 0), (b - 1, Hkv - 1)], calls=calls, check_rows_every=2, **kw)
+
+
 @pytest.mark.parametrize("b,Hkv,d,dtype,K,kw", [
     (1, 2, 128, "bf16", 1100, {}),                          # clusters of 8, a ragged last chunk
     (2, 8, 64, "bf16", 900, {}),                            # clusters of 2 (less than 96 KB of rows per further CTA)
