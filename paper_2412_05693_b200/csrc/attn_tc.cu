@@ -1,7 +1,8 @@
 // bf16 tensor-core path of the block forward pass (Sec. 3.2) for sm_100a:
-//   attn_fwd_split (attn_fwd_split.cuh): out = softmax(scale q k^T) v over the cached pairs and the block's causal
-//                 pairs, plus the log2-sum-exp of every query row.  QK^T and PV run on tcgen05 with TMA-staged
-//                 tiles and TMEM accumulators; one CTA owns one tile of 128 query rows, two CTAs share an SM.
+//   attn_fwd_split (attn_fwd_split.cuh) and, for large grids, attn_fwd_pair (attn_fwd_pair.cuh):
+//                 out = softmax(scale q k^T) v over the cached pairs and the block's causal pairs, plus the
+//                 log2-sum-exp of every query row.  QK^T and PV run on tcgen05 with TMA-staged
+//                 tiles and TMEM accumulators; an SM works on two tiles of 128 query rows at a time.
 //   score_tc    : sum_weights += sum_i attn_weights[i].  Recomputes the transposed logits S^T = K Q^T so that
 //                 a TMEM lane is a key; each thread then sums exp2(s - lse) over the queries of its own key
 //                 in a fixed order (deterministic, no atomics).
@@ -53,6 +54,7 @@ struct TcArgs {
 };
 
 #include "attn_fwd_split.cuh"
+#include "attn_fwd_pair.cuh"
 #include "attn_onepass.cuh"
 
 // ------------------------------------------------------------------------------------------------------
@@ -386,8 +388,25 @@ cudaError_t launch_onepass(const CacheView& c, const BlockArgs& a, cudaStream_t 
 }
 
 template <int D>
+cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+  using L = PairSmem<D>;
+  static SmemConfigured configured;
+  if (cudaError_t e = configured.ensure(attn_fwd_pair<D>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
+  const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
+  ProfileScope prof(kAttnFwd, st);
+  attn_fwd_pair<D><<<dim3((tiles + 1) / 2, c.nsamples * c.Hkv), L::kThreads, L::kTotal, st>>>(g_maps, make_args(c, a));
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <int D>
 cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
   if (onepass_applies(c, a)) return launch_onepass<D>(c, a, st);
+  // Two tiles per CTA where the handle's batch makes 1024 pairs of tiles or more (512 pairs at d = 64: 99 against 96 us
+  // for one tile per CTA, 768 pairs at d = 128: 104 against 102, 1152 pairs at d = 64: 156 against 162, 3072 pairs at
+  // d = 128: 549 against 563; few pairs leave SMs idle that single tiles would fill).
+  const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
+  if (c.left_pad == nullptr && (long long)(tiles / 2) * c.layer_units >= 1024) return launch_fwd_pair<D>(c, a, st);
   return c.left_pad != nullptr ? launch_fwd_split<D, true>(c, a, st) : launch_fwd_split<D, false>(c, a, st);
 }
 

@@ -57,6 +57,21 @@ __device__ __forceinline__ void mbar_wait(uint64_t* b, uint32_t parity, volatile
   atomicExch(status, kErrTimeout);
 }
 
+// The same for a single thread whose wake-up is on the critical path: plain tests, never suspended.
+constexpr int kPollLimit = 1 << 26;
+__device__ __forceinline__ void mbar_poll(uint64_t* b, uint32_t parity, volatile int* abort_flag, int* status) {
+  const uint32_t addr = smem_u32(b);
+  for (int it = 0; it < kPollLimit; ++it) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.b32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(addr), "r"(parity) : "memory");
+    if (ok) return;
+    if ((it & 255) == 255 && *abort_flag) return;
+  }
+  *abort_flag = 1;
+  atomicExch(status, kErrTimeout);
+}
+
 // TMA tile loads (no multicast): box lands in shared memory, completion counted on an mbarrier.
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, uint64_t* bar) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -145,6 +160,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
                  "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
@@ -216,6 +237,23 @@ __device__ __forceinline__ void ex2_poly2(float x0, float x1, float& r0, float& 
   fma2g(p0, p1, p0, p1, f0, f1, 0.24024981260299683f, 0.24024981260299683f);
   fma2g(p0, p1, p0, p1, f0, f1, 0.6931219696998596f, 0.6931219696998596f);
   fma2g(p0, p1, p0, p1, f0, f1, 0.9999991655349731f, 0.9999991655349731f);
+  r0 = __int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23));
+  r1 = __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23));
+}
+// The same with a polynomial of degree 5 (relative error 2.2e-7 in fp32, what ex2.approx has).
+__device__ __forceinline__ void ex2_poly2_deg5(float x0, float x1, float& r0, float& r1) {
+  constexpr float kMagic = 12582912.f;
+  x0 = fmaxf(x0, -126.f);
+  x1 = fmaxf(x1, -126.f);
+  float t0, t1, n0, n1, f0, f1, p0, p1;
+  add2g(t0, t1, x0, x1, kMagic, kMagic);
+  add2g(n0, n1, t0, t1, -kMagic, -kMagic);
+  add2g(f0, f1, x0, x1, -n0, -n1);
+  fma2g(p0, p1, f0, f1, 0.0013276472454890609f, 0.0013276472454890609f, 0.009675541892647743f, 0.009675541892647743f);
+  fma2g(p0, p1, p0, p1, f0, f1, 0.05550713092088699f, 0.05550713092088699f);
+  fma2g(p0, p1, p0, p1, f0, f1, 0.24022120237350464f, 0.24022120237350464f);
+  fma2g(p0, p1, p0, p1, f0, f1, 0.6931469440460205f, 0.6931469440460205f);
+  fma2g(p0, p1, p0, p1, f0, f1, 1.0000001192092896f, 1.0000001192092896f);
   r0 = __int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23));
   r1 = __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23));
 }

@@ -255,6 +255,39 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+# the forward kernel with two row tiles per CTA: the handle's batch makes 1024 pairs of tiles
+PAIR_GRIDS = [(64, 16, 1, 64, 200, 150),     # the second tile ragged, and it sees one key tile more than the first
+              (64, 16, 1, 128, 300, 129),    # three tiles: the last CTA's second tile has no rows
+              (64, 8, 4, 128, 130, 140),     # five tiles of which the last holds 8 rows
+              (32, 8, 8, 64, 200, 260)]
+
+
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS)
+def test_forward_on_pairs_of_row_tiles(b, Hkv, g, d, B, K):
+    wl = tiny("pair", b=b, Hq=g * Hkv, Hkv=Hkv, s=2 * B + 5, B=B, K=K, steps=1, dtype="bf16", d=d)
+    run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=2)
+
+
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS[1:3])
+def test_forward_on_pairs_of_row_tiles_when_the_maximum_grows(b, Hkv, g, d, B, K):
+    # later keys with ever larger logits: the accumulator is rescaled at every key tile
+    import torch
+    from paper_2412_05693_b200 import BatchMaxCache, Config
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen)
+    q, k, v = (x.bfloat16() for x in (f(b, B, g * Hkv, d), f(b, B, Hkv, d), f(b, B, Hkv, d)))
+    grow = torch.linspace(1, 12, B, device="cuda")
+    k = (k * grow[None, :, None, None]).bfloat16()
+    cache = BatchMaxCache(Config(batch=b, n_q_heads=g * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=B, block_max=B))
+    out = cache.prefill_block(q, k, v, 0)
+    assert cache.status() == 0
+    for s, h in ((0, 0), (b - 1, Hkv - 1)):
+        logits = torch.einsum("igd,jd->gij", q[s, :, h * g:(h + 1) * g].float(), k[s, :, h].float()) / d ** 0.5
+        logits.masked_fill_(torch.ones(B, B, device="cuda", dtype=torch.bool).triu(1), -float("inf"))
+        want = torch.einsum("gij,jd->igd", logits.softmax(-1), v[s, :, h].float())
+        assert (out[s, :, h * g:(h + 1) * g].float() - want).abs().max() < 2e-2
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,B,K,kw", [
     (1, 2, 1, 128, 64, 700, {}),                            # one query tile, a key tile per CTA
     (40, 8, 1, 64, 33, 530, {}),                            # ... all key tiles of a cache in one CTA, a chunk past the last row
