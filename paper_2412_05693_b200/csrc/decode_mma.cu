@@ -702,8 +702,8 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 }
 
 // Which kernel takes a step.  Measured, us per step (stream against this file's kernels; d = 128, g = 4, one pair leaves):
-// at most one cache per SM -- 8 caches of 512 pairs 7.7 / 8.7, 32 caches 8.7 / 11.5, 128 caches 10.9 / 12.9, of 256
-// pairs 7.9 / 8.9; with the caches in L2 (a handle of few layers) 32 caches of 512 pairs 9.1 / 9.1, 64 caches 9.5 / 9.1,
+// at most one cache per SM -- 8 caches of 512 pairs 6.2 / 8.7, 32 caches 8.0 / 11.5, 128 caches 10.9 / 12.9, of 256
+// pairs 7.9 / 8.9; with the caches in L2 (a handle of few layers) 32 caches of 512 pairs 7.6 / 9.1, 64 caches 9.2 / 9.1,
 // 128 caches 10.2 / 9.5, where this file's instance with K in registers is ahead (it ends at 640 pairs).  More caches --
 // 256 caches of 384 pairs 14.5 / 14.4, of 1024 pairs 30.8 / 34.2; 640 caches of 256 pairs 26.8 / 24.9, of 384 pairs
 // 31.8 / 41.7; 1024 caches of 1024 pairs 95 / 112; at d = 64 1024 caches of 512 pairs 40.5 / 42.3, of 700 pairs 46 / 55:

@@ -17,8 +17,9 @@
 //
 // What bounds it: HBM once there is a cache for every SM; below that the latency of one cache's chain (first tile ->
 // softmax -> last tile -> moves), which is what splitting a cache over a cluster shortens.  One pair leaving per step,
-// caches of 1024 pairs, d = 128, us per step against the kernel in decode_mma.cu: 8 caches (g = 4) 8.3 / 15.4 (10.1 with
-// exchanges by plain remote stores and releasing arrivals, which wait for the sender's global stores), 128
+// caches of 1024 pairs, d = 128, us per step against the kernel in decode_mma.cu: 8 caches (g = 4) 6.6 / 15.4 (10.1 with
+// exchanges by plain remote stores and releasing arrivals, which wait for the sender's global stores; 8.2 with a loop
+// over the peers' statistics and a releasing barrier at the end), 128
 // caches 16.8 / 19.1, 1024 caches 95 / 112 (5.9 against 5.0 TB/s of algorithmic bytes), 3072 caches 267 / 304 (6.3 TB/s),
 // 1024 caches without groups 88 / 104 (6.3 TB/s).  Not kept: tiles of 32 KB with two tiles' fragments in flight per warp
 // (spills; 111 against 94 us at 1024 caches), the per-row loops four rows at a time (+2 to 8 %), sums and ids written by
@@ -259,9 +260,9 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   auto first_row_up = [&](int x, T* slab, int hole, const uint4& own) {
     __syncwarp();
     if (rank + 1 < C && lane == 0) arrive_cluster(mapa(smem_u32(&bars[L::B_PREV + x]), rank + 1));
-    if (shift && rank > 0 && hole < r0) {
+    if (rank > 0) {
       wait_cluster(&bars[L::B_PREV + x], 0, abort_flag, c.status);
-      if (lane < PR && row_ok(c, r0 - 1))   // (r0 may be the step's own pair)
+      if (shift && hole < r0 && lane < PR && row_ok(c, r0 - 1))   // (r0 may be the step's own pair)
         st_global_16(slab + (size_t)(r0 - 1) * D + lane * 8, r0 == n_old ? own : reinterpret_cast<const uint4*>(s_first + (x == 0 ? D : 0))[lane]);
     }
   };
@@ -589,24 +590,47 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           const uint32_t dst = mapa(smem_u32(s_xstat + rank * 2 * G), tid), bar = mapa(smem_u32(&bars[L::B_X]), tid);
           float t[G];
           all_warps(s_wsum, t, [](float x, float y) { return x + y; });
+          if constexpr (G % 4 == 0) {
 #pragma unroll
-          for (int h = 0; h < G; ++h) {
-            st_peer(dst + 4 * h, mc[h], bar);
-            st_peer(dst + 4 * (G + h), t[h], bar);
+            for (int h = 0; h < G; h += 4) {
+              st_peer4(dst + 4 * h, __float_as_uint(mc[h]), __float_as_uint(mc[h + 1]), __float_as_uint(mc[h + 2]),
+                       __float_as_uint(mc[h + 3]), bar);
+              st_peer4(dst + 4 * (G + h), __float_as_uint(t[h]), __float_as_uint(t[h + 1]), __float_as_uint(t[h + 2]),
+                       __float_as_uint(t[h + 3]), bar);
+            }
+          } else {
+#pragma unroll
+            for (int h = 0; h < G; ++h) {
+              st_peer(dst + 4 * h, mc[h], bar);
+              st_peer(dst + 4 * (G + h), t[h], bar);
+            }
           }
         }
         wait_cluster(&bars[L::B_X], it & 1, abort_flag, c.status);
+        // lane p holds what CTA p said; the sum runs over the lanes in a fixed order (a loop over the peers, head by head,
+        // was 3000 cycles of dependent reads and exponentials with 8 CTAs)
+        float m[G], t[G];
+        {
+          const float* from = s_xstat + (lane & (kMaxCluster - 1)) * 2 * G;
+          const bool there = (lane & (kMaxCluster - 1)) < (int)C;
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-          float m = s_xstat[h];
-          for (int p = 1; p < (int)C; ++p) m = fmaxf(m, s_xstat[p * 2 * G + h]);
-          float t = 0.f;
-          for (int p = 0; p < (int)C; ++p) {
-            const float mp = s_xstat[p * 2 * G + h];
-            t += mp == -INFINITY ? 0.f : s_xstat[p * 2 * G + G + h] * ex2(mp - m);
-          }
-          f[h] = (q_real && mc[h] != -INFINITY) ? ex2(mc[h] - m) / t : 0.f;
+          for (int h = 0; h < G; ++h) { m[h] = there ? from[h] : -INFINITY; t[h] = there ? from[G + h] : 0.f; }
         }
+        float top[G];
+#pragma unroll
+        for (int h = 0; h < G; ++h) top[h] = m[h];
+#pragma unroll
+        for (int off = kMaxCluster / 2; off > 0; off >>= 1)
+#pragma unroll
+          for (int h = 0; h < G; ++h) top[h] = fmaxf(top[h], __shfl_xor_sync(0xffffffffu, top[h], off));
+#pragma unroll
+        for (int h = 0; h < G; ++h) t[h] = m[h] == -INFINITY ? 0.f : t[h] * ex2(m[h] - top[h]);
+#pragma unroll
+        for (int off = kMaxCluster / 2; off > 0; off >>= 1)
+#pragma unroll
+          for (int h = 0; h < G; ++h) t[h] += __shfl_xor_sync(0xffffffffu, t[h], off);
+#pragma unroll
+        for (int h = 0; h < G; ++h) f[h] = (q_real && mc[h] != -INFINITY) ? ex2(mc[h] - top[h]) / t[h] : 0.f;
       }
       // ---- sum_weights += attn_weights (heads added in a fixed order), candidate for eviction, bf16 exponentials
       // (the pair with the smallest ranking value leaves; ties: the higher position -- kv_ids, not rows: the rows of an
@@ -771,7 +795,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
               if (h < G) op[h * D + 16 * ws + gid + 8 * hf] = __float2bfloat16_rn(o[hf][hh] * fh);
             }
       } else {
-        const int dc = D / (int)C;                          // elements of every head that one CTA adds up
+        const int lc = 31 - __clz((int)C), ldc = (D == 128 ? 7 : 6) - lc, dc = 1 << ldc;   // elements of every head that one CTA adds up
         if (tid == 0) mbar_expect_tx(&bars[L::B_X + 2], G * D * 4);
         if (kg == 0)
 #pragma unroll
@@ -783,22 +807,29 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
 #pragma unroll
               for (int g = 0; g < G; ++g) fh = g == h ? f[g] : fh;
               if (h < G)
-                st_peer(mapa(smem_u32(s_xout + ((int)rank * G + h) * dc + d % dc), d / dc), o[hf][hh] * fh,
-                        mapa(smem_u32(&bars[L::B_X + 2]), d / dc));
+                st_peer(mapa(smem_u32(s_xout + (((int)rank * G + h) << ldc) + (d & (dc - 1))), d >> ldc), o[hf][hh] * fh,
+                        mapa(smem_u32(&bars[L::B_X + 2]), d >> ldc));
             }
         wait_cluster(&bars[L::B_X + 2], it & 1, abort_flag, c.status);
         for (int x = tid; x < G * dc; x += kConsumers) {
+          float part[kMaxCluster];
+#pragma unroll
+          for (int p = 0; p < kMaxCluster; ++p) part[p] = p < (int)C ? s_xout[(p * G << ldc) + x] : 0.f;
           float t = 0.f;
-          for (int p = 0; p < (int)C; ++p) t += s_xout[p * G * dc + x];   // fixed order
-          op[(x / dc) * D + (int)rank * dc + x % dc] = __float2bfloat16_rn(t);
+#pragma unroll
+          for (int p = 0; p < kMaxCluster; ++p) t += part[p];   // fixed order
+          op[(x >> ldc) * D + ((int)rank << ldc) + (x & (dc - 1))] = __float2bfloat16_rn(t);
         }
       }
       named_bar_sync(1, kConsumers);                        // the per-row arrays belong to the next cache
     }
   }
-  if (C > 1) {   // no CTA leaves while a peer may still write into its shared memory
+  // No CTA of a cluster leaves while a peer may still write into its shared memory.  It has waited for all that is sent
+  // to it (B_X, B_PREV), so the barrier need not order memory (a releasing arrival waits for the global stores, 1000
+  // cycles); it is there for a CTA whose waits gave up.
+  if (C > 1) {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   }
 }
@@ -832,9 +863,10 @@ bool plan_for(int C, int n1, int units, int sms, Plan* p) {
 }
 
 // Cluster size.  A cluster shortens the time a cache takes to pass through one SM and costs its exchanges.  us per step
-// with 1, 2, 4 and 8 CTAs per cache, d = 128, g = 4: 8 caches of 384 pairs 6.9 / 7.7 / 7.0 / 7.7, of 1024 pairs 12.6 /
-// 11.2 / 9.0 / 8.3; 32 caches of 1024 pairs 13.9 / 12.1 / 11.2; 64 caches of 700 pairs 10.7 / 11.5, of 1024 pairs 14.5 /
-// 13.3; at d = 64 8 caches of 1024 pairs 9.1 / 9.2 / 7.8 / 7.6 -- the line through these is the estimate below.
+// with 1, 2, 4 and 8 CTAs per cache, d = 128, g = 4: 8 caches of 200 pairs 5.5 / 5.6 / 5.4 / 6.2, of 700 pairs 9.4 / 8.4 /
+// 6.6 / 6.3, of 1024 pairs 12.6 / 10.1 / 7.8 / 6.6; 32 caches of 200 pairs 6.2 / 6.4 / 6.7, of 1024 pairs 14.1 / 11.4 /
+// 9.9; 64 caches of 384 pairs 8.3 / 8.3, of 1024 pairs 14.7 / 12.3; at d = 64 8 caches of 1024 pairs 9.1 / 8.1 / 6.6 /
+// 6.0 -- the line through these is the estimate below.
 // Only calls whose clusters are all resident at once are split (a GPC holds few clusters of 8: at 16 caches the second
 // wave made the step 1.5 times as long as with clusters of 4), and the handle's caches of a layer decide, not the call's:
 // sample ranges of one batch may be in flight together and must sum in the same order as the whole batch.
@@ -848,7 +880,7 @@ Plan choose_plan(int n1, int units, int layer_units, int sms) {
     if (C > 1 && (layer_units > kMostCaches[x] || layer_units * C > sms)) continue;
     if (!plan_for<D, G>(C, n1, units, sms, &p)) continue;
     const double stream = n1 * (4.0 * D + 80) / C / 57e3;   // us: row bytes, and the work per row
-    const double us = stream + (C == 1 ? 3.2 : 6.0 + 0.1 * C + 1.5 * layer_units * C / sms);
+    const double us = stream + (C == 1 ? 3.3 : 4.1 + 0.1 * C) + 1.9 * layer_units * C / sms;
     if (best.C == 0 || us < best_us) { best = p; best_us = us; }
   }
   return best;
