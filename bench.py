@@ -339,7 +339,7 @@ def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch
     at_max = bool(clocks and clocks.get("sm_mhz") and clocks.get("sm_max_mhz")
                   and clocks["sm_mhz"] >= 0.97 * clocks["sm_max_mhz"])
     peak = burst if at_max else sust
-    return {"bound": "tensor", "kernel": "prefill-block attention forward (attn_fwd_split)", "achieved": achieved,
+    return {"bound": "tensor", "kernel": "prefill-block attention forward (attn_fwd_pair, attn_fwd_split on small grids)", "achieved": achieved,
             "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "frac_of_burst_peak": achieved / burst, "frac_of_sustained_peak": achieved / sust,
             "peak_source": f"{pk_src} bf16 matmul, " + ("burst figure: the sampled SM clock stayed at its maximum"
@@ -487,7 +487,7 @@ def run_max_batch(args, name, rank, world, local_rank, sampler):
         gbs = dec_bytes / (kernel_ms["decode"] * 1e-3) / 1e9
         gbs_mv = (dec_bytes + move_bytes) / (kernel_ms["decode"] * 1e-3) / 1e9
         rooflines["decode"] = {
-            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_mma_kernel)",
+            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_stream_kernel, decode_mma_kernel on short caches)",
             "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": gbs / pk["hbm_gbs"],
             "achieved_with_compaction_writes": gbs_mv, "frac_with_compaction_writes": gbs_mv / pk["hbm_gbs"],
             "rows_moved_per_cache_and_step": moved.get("decode", 0) / max(1, wl.b * wl.Hkv * wl.L * wl.steps),
@@ -785,7 +785,7 @@ def run_resident(args, wl, rank, world, local_rank, sampler, light=False):
         one_step(moved=moved).close()             # one more eager pass with the device-side counters on
         move_bytes = moved.get("decode", 0) * 2.0 * wl.d * wl.elem_bytes
         rooflines["decode"] = {
-            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_mma_kernel)",
+            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_stream_kernel, decode_mma_kernel on short caches)",
             "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": gbs / pk["hbm_gbs"],
             "achieved_with_per_launch_events": dec_bytes / (dec_ms * 1e-3) / 1e9, "ms_in_timed_region": in_region_ms,
             "achieved_with_compaction_writes": (dec_bytes + move_bytes) / (in_region_ms * 1e-3) / 1e9,
