@@ -345,7 +345,7 @@ def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch
             "peak_source": f"{pk_src} bf16 matmul, " + ("burst figure: the sampled SM clock stayed at its maximum"
                                                          if at_max else
                                                          "sustained figure: the sampled SM clock was below its maximum"),
-            "traffic": dram_traffic("attn_fwd_split", samples_per_launch),
+            "traffic": dram_traffic("attn_fwd_pair", samples_per_launch),
             "launches_per_step": attn_n, "avg_launch_ms": attn_ms / max(attn_n, 1),
             "algorithmic": "4*d FLOP per visible (query, key) pair; the score pass's recompute is not counted"}
 
@@ -491,7 +491,7 @@ def run_max_batch(args, name, rank, world, local_rank, sampler):
             "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": gbs / pk["hbm_gbs"],
             "achieved_with_compaction_writes": gbs_mv, "frac_with_compaction_writes": gbs_mv / pk["hbm_gbs"],
             "rows_moved_per_cache_and_step": moved.get("decode", 0) / max(1, wl.b * wl.Hkv * wl.L * wl.steps),
-            "traffic": dram_traffic("decode_mma_kernel", DECODE_MICRO),
+            "traffic": dram_traffic("decode_stream_kernel", DECODE_MICRO),
             "peak_source": f"{pk_src} (HBM copy)", "launches_per_step": kernel_n["decode"],
             "avg_launch_ms": kernel_ms["decode"] / max(kernel_n["decode"], 1),
             "algorithmic": "(n+1)*(2*d*e+16) + 2*d*e + 2*g*d*e bytes per cache and step, compaction moves not counted"}
