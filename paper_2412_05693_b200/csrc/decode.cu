@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
       if (s.id[j] < pad) ave = -1.f;
       else if (c.rule == 0) ave = sw / ((float)G * (float)(a.pos + 1 - s.id[j]));
       else ave = (c.rule == 1 && j >= n1 - a.target / 2) ? INFINITY : sw;
+      ave = fminf(ave, INFINITY);   // NaN (a NaN in the step's queries or keys) ranks like +inf: some row is always found
       if (ave <= best_ave) { best_ave = ave; best_j = j; }   // j ascends: ties move to the higher position
     } else if (row_ok(c, j)) {
       c.sum_weights[base + j] = sw;

@@ -381,6 +381,7 @@ __global__ void __launch_bounds__(NT, KD > 1 ? 1 : 512 / NT) decode_mma_kernel(C
       // fast division: the IEEE routine takes a slow path for the tiny sums of long-evicted histories (4 % of the step)
       else if (rule == 0) ave = __fdividef(sw, (float)G * (float)(a.pos + 1 - s.id[j]));
       else ave = (rule == 1 && j >= n1 - a.target / 2) ? INFINITY : sw;
+      ave = fminf(ave, INFINITY);   // NaN (a NaN in the step's queries or keys) ranks like +inf: some row is always found
       // ties: the higher position leaves (kv_ids, not rows: the rows of an unordered cache are in no order)
       if (ave < best_ave || (ave == best_ave && s.id[j] > best_id)) { best_ave = ave; best_j = j; best_id = s.id[j]; }
     } else if (row_ok(c, j)) {

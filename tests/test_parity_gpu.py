@@ -255,6 +255,43 @@ def test_decode_with_one_cache_per_sm(K, g):
     assert st["evictions"] >= 6 * 14
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,dtype,kw", [
+    (8, 8, 4, 128, 200, "bf16", {}),                            # one cache per SM, in L2: K in registers, moves by TMA
+    (40, 8, 2, 64, 60, "bf16", {}),                             # small CTAs
+    (40, 8, 2, 64, 60, "bf16", dict(compaction="fill")),
+    (40, 8, 2, 64, 60, "bf16", dict(rule="sum_recent")),
+    (1, 4, 2, 128, 900, "bf16", {}),                            # the stream, a cache over a cluster
+    (20, 8, 1, 128, 700, "bf16", {}),                           # ... several caches per CTA
+    (3, 2, 2, 64, 100, "f32", {}),
+])
+def test_evicting_decode_step_with_a_nan_query(b, Hkv, g, d, K, dtype, kw):
+    # every ranking value of a cache is NaN: still exactly one of its pairs leaves (the highest position), and no other
+    # cache changes
+    wl = tiny("nan_query", b=b, Hq=g * Hkv, Hkv=Hkv, s=K, B=K, K=K, steps=2, dtype=dtype, d=d)
+    inp = Inputs(wl, "cuda")
+    prompt, steps = inp.block(0, 0, K), [tuple(x[:, 0].contiguous() for x in inp.block(0, K + t, 1)) for t in range(2)]
+    smp, kh = b // 2, Hkv - 1
+    states = []
+    for nan in (False, True):
+        cache = bm.BatchMaxCache(make_config(wl, **kw))
+        cache.prefill_block(*prompt, 0)
+        before = cache.export(0, smp, kh, rows=True)
+        for q, k, v in steps:
+            q = q.clone()
+            if nan:
+                q[smp, kh * g, 3] = float("nan")
+            cache.decode_step(q, k, v, evict_to=K)
+        assert cache.status() == 0
+        states.append({u: cache.export(0, *u, rows=True) for u in all_units(wl, {0, max(0, smp - 1), smp, min(b - 1, smp + 1), b - 1})})
+        cache.close()
+    for u, want in states[0].items():
+        if u != (smp, kh):
+            assert all(torch.equal(x, y) for x, y in zip(states[1][u], want))
+    ids, sums, k_rows, v_rows = states[1][(smp, kh)]
+    assert torch.isnan(sums).all()
+    assert torch.equal(ids, before[0]) and torch.equal(k_rows, before[2]) and torch.equal(v_rows, before[3])
+
+
 # the forward kernel with two row tiles per CTA: the handle's batch makes 1024 pairs of tiles
 PAIR_GRIDS = [(64, 16, 1, 64, 200, 150),     # the second tile ragged, and it sees one key tile more than the first
               (64, 16, 1, 128, 300, 129),    # three tiles: the last CTA's second tile has no rows
