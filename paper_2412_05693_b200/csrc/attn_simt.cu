@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(NT, 2) score_simt(CacheView c, BlockArgs a) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int counted_from = rule_first_counted_row(c.rule, c.window, a.I, c.g);   // rules that look at the last queries only
   const int first_row = (j0 > c.n_old) ? (j0 - c.n_old) * c.g : 0;  // earlier rows cannot see this tile
-  const int first_tile = (first_row / TM + (int)rank) * TM, step = (int)C * TM;
+  // query tile t is CTA t % C's whatever the first one is, so that key tiles of 16 and of 64 add up in the same order
+  const int t0 = first_row / TM, first_tile = (t0 + (((int)rank - t0) & ((int)C - 1))) * TM, step = (int)C * TM;
 
   auto load_q = [&](int row0, int b) {
     load_rows<T, D, LD, TM, NT>(sQ + b * TM * LD, tid, [&](int r) { return query_row_ptr<T, D>(c, a, smp, kh, row0 + r); });
@@ -342,8 +343,9 @@ __global__ void __launch_bounds__(NT, 2) score_simt(CacheView c, BlockArgs a) {
       const int vis = row < R ? c.n_old + row / c.g + 1 : 0;
 #pragma unroll
       for (int y = 0; y < KT; ++y) {
-        const float w = j0 + tx + 16 * y < vis ? expf(s[x][y] * a.scale - lse) : 0.f;
-        col[y] += w;
+        // (roundings spelled out: the instances with key tiles of 16 and of 64 agree bit by bit)
+        const float w = j0 + tx + 16 * y < vis ? expf(fmaf(s[x][y], a.scale, -lse)) : 0.f;
+        col[y] = __fadd_rn(col[y], w);
         col_sq[y] = fmaf(w, w, col_sq[y]);
       }
     }
@@ -440,16 +442,18 @@ cudaError_t launch_score_kt(const CacheView& c, const BlockArgs& a, int cluster,
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Key tiles of 64; a grid of fewer than four CTAs per SM shares each key tile among a cluster as long as there are
-// query tiles to share (16 caches, 1024 query rows against 256 keys: 84 -> 45 us with clusters of 8; against 1536 keys
-// 261 -> 226 us with clusters of 2, 287 with none below two CTAs per SM), and takes key tiles of 16 if SMs would still be idle.
+// Key tiles of 64; a handle whose caches of a layer make fewer than four CTAs per SM shares each key tile among a cluster
+// as long as there are query tiles to share (16 caches, 1024 query rows against 256 keys: 84 -> 45 us with clusters of 8;
+// against 1536 keys 261 -> 226 us with clusters of 2, 287 with none below two CTAs per SM).  The cluster decides the
+// order of the column sums, so the handle's caches decide it and not the call's.  Key tiles of 16, which add up in the
+// same order, if SMs would still be idle.
 template <typename T, int D>
 cudaError_t launch_score_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
-  const int tiles = (c.n_old + a.I + 63) / 64 * c.nsamples * c.Hkv, q_tiles = (a.I * c.g + 63) / 64;
+  const int tiles = (c.n_old + a.I + 63) / 64, q_tiles = (a.I * c.g + 63) / 64;
   int cluster = 1;
-  while (cluster < 8 && 2 * cluster <= q_tiles && tiles * cluster < 4 * sm_count()) cluster *= 2;
+  while (cluster < 8 && 2 * cluster <= q_tiles && (long long)tiles * c.layer_units * cluster < 4 * sm_count()) cluster *= 2;
   if constexpr (sizeof(T) == 4)
-    if (tiles * cluster < sm_count()) return launch_score_kt<T, D, 1, 4, 256>(c, a, cluster, st);
+    if ((long long)tiles * c.nsamples * c.Hkv * cluster < sm_count()) return launch_score_kt<T, D, 1, 4, 256>(c, a, cluster, st);
   return launch_score_kt<T, D, 4, 4, 256>(c, a, cluster, st);
 }
 

@@ -390,6 +390,18 @@ def test_f32_kernels_by_grid_size(b, Hkv, g, d, B, K):
     run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1)
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", [
+    (4, 4, 4, 128, 256, 1280),   # the whole batch would share a key tile among 2 CTAs, a single sample among 8
+    (4, 4, 4, 128, 256, 512),    # ... 4 and 8
+    (6, 2, 2, 64, 130, 300),     # key tiles of 16 for a single sample
+])
+def test_f32_blocks_are_bitwise_independent_of_sample_ranges(b, Hkv, g, d, B, K):
+    wl = tiny("f32_ranges", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 2 * B, B=B, K=K, steps=0, dtype="f32", d=d)
+    base = run_free(wl)
+    assert_same_run(base, run_free(wl, micro=b // 2))
+    assert_same_run(base, run_free(wl, micro=1))
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
     (1, 3, 1, 64, 40, {}),                                  # less than one tile of rows
     (1, 2, 4, 128, 1023, {}),                               # a cluster of 8 CTAs per cache; the step's row ends a tile
