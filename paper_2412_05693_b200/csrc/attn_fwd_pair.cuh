@@ -201,16 +201,19 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
 #pragma unroll
           for (int e = 0; e < 32; ++e) s[c][e] = 32 * c + e < nvis ? s[c][e] : 0xff800000u;
       }
+      // A NaN or +inf among a row's visible logits makes the row NaN, through its maximum: the polynomial of every fourth
+      // pair takes NaN for its lowest argument.
       float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
       for (int e = 0; e < 32; e += 2)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) m4[c] = max3(m4[c], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
-      const float mx2 = fmaxf(max3(m4[0], m4[1], m4[2]), m4[3]) * a.scale_log2;
+        for (int c = 0; c < 4; ++c) m4[c] = max3_nan(m4[c], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
+      float mx2 = max3_nan(max3_nan(m4[0], m4[1], m4[2]), m4[3], -INFINITY) * a.scale_log2;
+      if (mx2 == INFINITY) mx2 = __uint_as_float(0x7fffffffu);
       bool rescale = false;
       float alpha = 1.f;
       if (j == 0) m_used = mx2;
-      else if (mx2 > m_used + kRescaleThreshold) { alpha = ex2(m_used - mx2); m_used = mx2; rescale = true; }
+      else if (!(mx2 <= m_used + kRescaleThreshold)) { alpha = ex2(m_used - mx2); m_used = mx2; rescale = true; }
       // S(j) being complete implies the previous P.V into O has completed, so O may be touched here (rarely)
       if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll 1

@@ -325,6 +325,27 @@ def test_forward_on_pairs_of_row_tiles_when_the_maximum_grows(b, Hkv, g, d, B, K
         assert (out[s, :, h * g:(h + 1) * g].float() - want).abs().max() < 2e-2
 
 
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS[1:3])
+def test_forward_on_pairs_of_row_tiles_with_nan_and_inf_keys(b, Hkv, g, d, B, K, value):
+    # one such element in one key of every cache, at every position of a block: a row is NaN where fp32 attention says
+    # so, and as without that key where its weight is 0 or the row does not see it
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen).bfloat16()
+    q, k, v = f(b, B, g * Hkv, d), f(b, B, Hkv, d), f(b, B, Hkv, d)
+    for u in range(b * Hkv):
+        k[u // Hkv, u % B, u % Hkv, 3] = value
+    cache = bm.BatchMaxCache(bm.Config(batch=b, n_q_heads=g * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=B, block_max=B))
+    out = cache.prefill_block(q, k, v, 0).float()
+    assert cache.status() == 0
+    hidden = torch.ones(B, B, device="cuda", dtype=torch.bool).triu(1)
+    for s in range(b):
+        logits = torch.einsum("ihgd,jhd->hgij", q[s].float().view(B, Hkv, g, d), k[s].float()) / d ** 0.5
+        want = torch.einsum("hgij,jhd->ihgd", logits.masked_fill_(hidden, -float("inf")).softmax(-1), v[s].float())
+        assert torch.equal(torch.isnan(out[s]), torch.isnan(want).reshape(B, g * Hkv, d))
+        assert (out[s] - want.reshape(B, g * Hkv, d)).nan_to_num_(0.0).abs().max() < 2e-2
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,B,K,kw", [
     (1, 2, 1, 128, 64, 700, {}),                            # one query tile, a key tile per CTA
     (40, 8, 1, 64, 33, 530, {}),                            # ... all key tiles of a cache in one CTA, a chunk past the last row
