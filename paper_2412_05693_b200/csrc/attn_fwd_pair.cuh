@@ -51,12 +51,13 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
   const int R = a.I * a.g;
   const int qpt = kTileM / a.g;                  // inputs (positions) covered by a row tile
   const int t_old = (a.n_old + kTileN - 1) / kTileN;
-  // pairs of row tiles are handed out last first (a later tile sees more of the block's own keys)
-  const int rt0 = 2 * (gridDim.x - 1 - blockIdx.x);
+  // pairs of row tiles (or single ones: tile B has no rows) are handed out last first (a later tile sees more of the
+  // block's own keys)
+  const int rt0 = a.row_tiles * (gridDim.x - 1 - blockIdx.x);
   // key tiles a row tile sees: the cached ones and the block's up to its last input; no rows, no tiles
   auto n_tiles = [&](int x) {
     const int i0 = (rt0 + x) * qpt;
-    return i0 >= a.I ? 0 : t_old + min(a.I - 1, i0 + qpt - 1) / kTileN + 1;
+    return x >= a.row_tiles || i0 >= a.I ? 0 : t_old + min(a.I - 1, i0 + qpt - 1) / kTileN + 1;
   };
   const int T0 = n_tiles(0), T1 = n_tiles(1), T = max(T0, T1);   // T1 >= T0 unless tile B has no rows
 

@@ -49,6 +49,7 @@ struct TcArgs {
   int first_row;     // query rows below it add nothing to the column sums (rules that look at the last queries only)
   int overwrite;     // 1: the column sums replace sum_weights instead of being added
   int key_tiles;     // key tiles per CTA of the score pass (QRES)
+  int row_tiles;     // row tiles per CTA of attn_fwd_pair: 2 or 1
   float* sum_sq;     // rule 4: sums of squared weights (cached pairs / the block's pairs), else null
   float* new_sq;
 };
@@ -345,6 +346,7 @@ TcArgs make_args(const CacheView& c, const BlockArgs& a) {
   t.overwrite = rule_overwrites(c.rule) ? 1 : 0;
   t.sum_sq = c.sum_sq; t.new_sq = a.new_sq;
   t.key_tiles = 1;
+  t.row_tiles = 2;
   return t;
 }
 
@@ -393,8 +395,13 @@ cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t
   static SmemConfigured configured;
   if (cudaError_t e = configured.ensure(attn_fwd_pair<D>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
   const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
+  TcArgs args = make_args(c, a);
+  // One tile per CTA while each has an SM to itself (8 caches, a block of 512: 29 us against 34 on half as many SMs; 32
+  // caches of 4 tiles 23 against 25; 24 caches of 10 tiles 47 against 31): a row's arithmetic is the same either way.
+  args.row_tiles = tiles * c.nsamples * c.Hkv <= sm_count() ? 1 : 2;
   ProfileScope prof(kAttnFwd, st);
-  attn_fwd_pair<D><<<dim3((tiles + 1) / 2, c.nsamples * c.Hkv), L::kThreads, L::kTotal, st>>>(g_maps, make_args(c, a));
+  const dim3 grid((tiles + args.row_tiles - 1) / args.row_tiles, c.nsamples * c.Hkv);
+  attn_fwd_pair<D><<<grid, L::kThreads, L::kTotal, st>>>(g_maps, args);
   count_launch();
   return cudaGetLastError();
 }
@@ -402,9 +409,10 @@ cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t
 template <int D>
 cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
   if (onepass_applies(c, a)) return launch_onepass<D>(c, a, st);
-  // Two tiles per CTA where the handle's batch makes 1024 pairs of tiles or more (512 pairs at d = 64: 99 against 96 us
-  // for one tile per CTA, 768 pairs at d = 128: 104 against 102, 1152 pairs at d = 64: 156 against 162, 3072 pairs at
-  // d = 128: 549 against 563; few pairs leave SMs idle that single tiles would fill).
+  // Two tiles per CTA (launch_fwd_pair) where the handle's batch makes 1024 pairs of tiles or more (512 pairs at d = 64:
+  // 99 against 96 us for one tile per CTA, 768 pairs at d = 128: 104 against 102, 1152 pairs at d = 64: 156 against 162,
+  // 3072 pairs at d = 128: 549 against 563).  The handle's caches decide and not the call's: the two kernels round
+  // differently, and outputs do not depend on how a batch is cut into sample ranges.
   const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
   if (c.left_pad == nullptr && (long long)(tiles / 2) * c.layer_units >= 1024) return launch_fwd_pair<D>(c, a, st);
   return c.left_pad != nullptr ? launch_fwd_split<D, true>(c, a, st) : launch_fwd_split<D, false>(c, a, st);

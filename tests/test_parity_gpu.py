@@ -325,6 +325,15 @@ def test_forward_on_pairs_of_row_tiles_when_the_maximum_grows(b, Hkv, g, d, B, K
         assert (out[s, :, h * g:(h + 1) * g].float() - want).abs().max() < 2e-2
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS)
+def test_forward_on_pairs_of_row_tiles_is_bitwise_independent_of_sample_ranges(b, Hkv, g, d, B, K):
+    # a single sample's tiles have an SM each: one tile per CTA
+    wl = tiny("pair_ranges", b=b, Hq=g * Hkv, Hkv=Hkv, s=2 * B + 5, B=B, K=K, steps=0, dtype="bf16", d=d)
+    base = run_free(wl)
+    assert_same_run(base, run_free(wl, micro=b // 2))
+    assert_same_run(base, run_free(wl, micro=1))
+
+
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS[1:3])
 def test_forward_on_pairs_of_row_tiles_with_nan_and_inf_keys(b, Hkv, g, d, B, K, value):
