@@ -211,6 +211,7 @@ CacheView make_view(const bm_cache* c, int layer, int sample0, int nsamples, int
   v.nsamples = nsamples;
   v.status = c->status;
   v.left_pad = (c->has_pad && with_pad) ? c->left_pad + sample0 : nullptr;
+  v.padded = c->has_pad ? 1 : 0;
   v.rule = c->cfg.rule;
   v.fill = c->cfg.compaction == BM_COMPACT_FILL ? 1 : 0;
   v.sum_sq = c->sum_sq != nullptr ? c->sum_sq + row0 : nullptr;

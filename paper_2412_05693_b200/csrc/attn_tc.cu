@@ -412,9 +412,10 @@ cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st
   // Two tiles per CTA (launch_fwd_pair) where the handle's batch makes 1024 pairs of tiles or more (512 pairs at d = 64:
   // 99 against 96 us for one tile per CTA, 768 pairs at d = 128: 104 against 102, 1152 pairs at d = 64: 156 against 162,
   // 3072 pairs at d = 128: 549 against 563).  The handle's caches decide and not the call's: the two kernels round
-  // differently, and outputs do not depend on how a batch is cut into sample ranges.
+  // differently, and outputs do not depend on how a batch is cut into sample ranges -- ranges of a padded handle that
+  // hold no padding included, since there is no padding instance of the pair kernel.
   const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
-  if (c.left_pad == nullptr && (long long)(tiles / 2) * c.layer_units >= 1024) return launch_fwd_pair<D>(c, a, st);
+  if (!c.padded && (long long)(tiles / 2) * c.layer_units >= 1024) return launch_fwd_pair<D>(c, a, st);
   return c.left_pad != nullptr ? launch_fwd_split<D, true>(c, a, st) : launch_fwd_split<D, false>(c, a, st);
 }
 

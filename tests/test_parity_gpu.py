@@ -327,11 +327,13 @@ def test_forward_on_pairs_of_row_tiles_when_the_maximum_grows(b, Hkv, g, d, B, K
 
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS)
 def test_forward_on_pairs_of_row_tiles_is_bitwise_independent_of_sample_ranges(b, Hkv, g, d, B, K):
-    # a single sample's tiles have an SM each: one tile per CTA
-    wl = tiny("pair_ranges", b=b, Hq=g * Hkv, Hkv=Hkv, s=2 * B + 5, B=B, K=K, steps=0, dtype="bf16", d=d)
-    base = run_free(wl)
-    assert_same_run(base, run_free(wl, micro=b // 2))
-    assert_same_run(base, run_free(wl, micro=1))
+    # a single sample's tiles have an SM each: one tile per CTA.  With one padded sample: no range takes another kernel
+    # (short blocks do, so there is none)
+    for tail, pads in ((5, None), (0, [0] * (b - 1) + [B + 7])):
+        wl = tiny("pair_ranges", b=b, Hq=g * Hkv, Hkv=Hkv, s=2 * B + tail, B=B, K=K, steps=0, dtype="bf16", d=d)
+        base = run_free(wl, pads=pads)
+        assert_same_run(base, run_free(wl, micro=b // 2, pads=pads))
+        assert_same_run(base, run_free(wl, micro=1, pads=pads))
 
 
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
@@ -793,10 +795,12 @@ def test_bounded_wait_times_out_and_context_survives():
     assert st["calls"] == 2
 
 
-def run_free(wl, host=False, micro=None):
+def run_free(wl, host=False, micro=None, pads=None):
     """Whole schedule on the GPU only; returns final state and all outputs (for determinism / variants)."""
     cfg = make_config(wl)
     cache = bm.BatchMaxCache(cfg)
+    if pads is not None:
+        cache.set_left_pad(pads)
     inp = Inputs(wl, "cuda")
     outs, keep = [], []
     for kind, pos0, I, ev in schedule(wl):
