@@ -27,7 +27,7 @@ struct CacheView {
   int32_t window, pool;     // rule 3: queries observed / recent pairs kept; width of the max-pooling (odd)
   int32_t std_permille;     // rule 4: share of the kept pairs chosen by standard deviation, in 1/1000
   int32_t padded;           // 1: some sample of the handle is left-padded (left_pad is null for calls that meet no padding)
-  int32_t in_l2;            // 1: all of the handle's caches together fit into half of the L2 cache
+  int32_t in_l2;            // 1: all of the handle's caches together stay in the L2 cache
   int32_t layer_units;      // caches of the handle in one layer: what a kernel is chosen by where the choice changes the order
                             // of a sum, so that results do not depend on how a batch is cut into sample ranges
 };
@@ -95,6 +95,7 @@ cudaError_t launch_decode(int dtype, int d, const CacheView& c, const void* q, c
 int sm_count();   // multiprocessors of the current device
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                               int32_t pos, float scale, int32_t target /* <0: none */, cudaStream_t st);
+constexpr int kMostSharedCaches = 64;   // caches of a layer up to which the stream shares each among a cluster (on 148 SMs)
 // bf16 decode step as a stream (decode_stream.cu); *taken = false: the shape does not fit it, nothing was enqueued
 cudaError_t launch_decode_stream(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                                  int32_t pos, float scale, bool evict_one, cudaStream_t st, bool* taken);

@@ -702,27 +702,49 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
   return attn > ev ? attn : ev;
 }
 
-// Which kernel takes a step.  Measured, us per step (stream against this file's kernels; d = 128, g = 4, one pair leaves):
-// at most one cache per SM -- 8 caches of 512 pairs 6.2 / 8.7, 32 caches 8.0 / 11.5, 128 caches 10.9 / 12.9, of 256
-// pairs 7.9 / 8.9; with the caches in L2 (a handle of few layers) 32 caches of 512 pairs 7.6 / 9.1, 64 caches 9.2 / 9.1,
-// 128 caches 10.2 / 9.5, where this file's instance with K in registers is ahead (it ends at 640 pairs).  More caches --
-// 256 caches of 384 pairs 14.5 / 14.4, of 1024 pairs 30.8 / 34.2; 640 caches of 256 pairs 26.8 / 24.9, of 384 pairs
-// 31.8 / 41.7; 1024 caches of 1024 pairs 95 / 112; at d = 64 1024 caches of 512 pairs 40.5 / 42.3, of 700 pairs 46 / 55:
-// the stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes,
-// 150 KB, or 256 KB while the other kernel holds every cache of the call at once (two CTAs per SM).
-static bool stream_is_faster(int d, int n1, int units, bool in_l2) {
-  const int sms = sm_count();
-  if (units <= sms) return d == 64 || n1 > kBatchTiles * 128 || !in_l2 || units <= sms / 4;
-  return (size_t)n1 * d * 4 >= (units <= 2 * sms ? 256u : 150u) * 1024;
+// Which kernel takes a step: the stream, or this file's kernels.  By the handle's caches of a layer and not the call's, so
+// that sample ranges of a batch take one kernel.  Measured, us per step (stream / this file; d = 128, g = 4, one pair leaves
+// by its average and the rows behind it move up, unless said otherwise):
+//   Caches out of HBM (several layers or ranges in turn): 8 caches of 500 pairs 8.1 / 10.2, 128 caches of 500 11.0 / 12.1,
+//   of 1024 18.4 / 25.3, 192 of 400 15.6 / 16.8, 320 of 400 21.0 / 24.7, 512 of 330 25.2 / 23.5, of 500 29.7 / 31.3, 800 of
+//   320 34.4 / 38.1, 1024 of 1024 95 / 112; d = 64 512 caches of 700 25.6 / 27.7; ranking by raw sums 512 of 330 27.1 /
+//   31.7.  The stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's
+//   bytes: 150 KB, 172 KB where an SM has up to four caches (and the last round of them is a large part; not under the
+//   other rules or with padding, where this file's instance is the slower one), or 256 KB while this file's kernel holds
+//   every cache of the call at once (two CTAs per SM).
+//   Caches in L2 (a handle of few layers):
+//   - shared by clusters: 64 caches of 512 pairs 9.8 / 9.2 (K in registers, which ends at 640 pairs), of 1024 14.4 / 16.0;
+//   - at most one per SM: 128 caches of 700 pairs 13.1 / 12.2, of 1024 17.4 / 16.2, but where no row moves 1024 11.1 / 15.0
+//     and by raw sums 18.3 / 21.9; by the current query alone, which moves most rows, 28.2 / 27.4; d = 64, g = 1 300 pairs
+//     7.0 / 6.3, g = 4 1024 pairs 11.4 / 12.4;
+//   - more: 192 of 600 18.6 / 15.7, 320 of 330 18.6 / 16.1, 512 of 330 25.0 / 18.0; unordered 320 of 330 17.3 / 15.8, of 500
+//     20.0 / 21.7; d = 64 192 of 1024 18.3 / 15.7, unordered 16.5 / 15.2.
+//   A cut by more than one value per pair follows the stream as a launch of its own: under rule 4 8 caches of 300 pairs
+//   16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 96 of 700 26.1 / 24.7, 512 of 700 69 / 64; unordered with a recent window 512
+//   of 700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
+static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
+  const int sms = sm_count(), n1 = c.n_old + 1, caches = c.layer_units;
+  const size_t bytes = (size_t)n1 * d * 4;
+  const bool plain = c.rule == 0 && !c.padded, moves = one && !c.fill;
+  if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) &&
+      (caches > kMostSharedCaches || (c.rule == 4 && bytes < (size_t)200 << 10))) return false;
+  if (caches <= kMostSharedCaches) return d == 64 || n1 > kBatchTiles * 128 || !c.in_l2 || caches <= sms / 4;
+  if (caches <= sms) {
+    if (!c.in_l2) return true;
+    if (d == 64) return n1 > 512 || !plain || !moves;
+    return n1 > kBatchTiles * 128 && !(moves && (plain || c.rule == 2));
+  }
+  if (c.in_l2 && plain && (moves || d == 64)) return false;
+  return bytes >= (size_t)(caches <= 2 * sms ? 256 : plain && caches <= 4 * sms ? 172 : 150) << 10;
 }
 
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,
                               int32_t pos, float scale, int32_t target, cudaStream_t st) {
   const int n1 = c.n_old + 1;
-  if (stream_is_faster(d, n1, c.layer_units, c.in_l2 != 0)) {
-    // exactly one pair leaves by a single ranking value per pair: inside the kernel; any other cut follows it
-    const bool cut = target >= 0 && target < n1;
-    const bool one = cut && target == n1 - 1 && !(c.fill && c.rule == 1) && c.rule < 3;
+  // exactly one pair leaves by a single ranking value per pair: inside the streaming kernel; any other cut follows it
+  const bool cut = target >= 0 && target < n1;
+  const bool one = cut && target == n1 - 1 && !(c.fill && c.rule == 1) && c.rule < 3;
+  if (stream_is_faster(c, d, cut, one)) {
     bool taken = false;
     const cudaError_t err = launch_decode_stream(d, c, q, k, v, out, pos, scale, one, st, &taken);
     if (err != cudaSuccess) return err;

@@ -872,7 +872,7 @@ bool plan_for(int C, int n1, int units, int sms, Plan* p) {
 // sample ranges of one batch may be in flight together and must sum in the same order as the whole batch.
 template <int D, int G>
 Plan choose_plan(int n1, int units, int layer_units, int sms) {
-  constexpr int kMostCaches[] = {0, 64, 32, 8};   // for C = 2, 4, 8 on 148 SMs
+  constexpr int kMostCaches[] = {0, kMostSharedCaches, 32, 8};   // for C = 2, 4, 8 on 148 SMs
   Plan best;
   double best_us = 0;
   for (int x = 0, C = 1; C <= kMaxCluster; ++x, C *= 2) {

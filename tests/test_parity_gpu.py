@@ -443,6 +443,9 @@ def test_f32_blocks_are_bitwise_independent_of_sample_ranges(b, Hkv, g, d, B, K)
     (20, 8, 1, 128, 641, {}),                               # more caches than SMs: a second cache per CTA
     (40, 8, 4, 64, 1090, {}),                               # three caches per CTA
     (20, 8, 4, 128, 700, dict(p_dec=3)),                    # the cut follows as a launch of its own
+    (1, 4, 2, 64, 1100, dict(rule="average_std")),
+    (9, 8, 2, 128, 660, {}),                                # 72 caches in L2: the other kernel, beyond its rows in registers
+    (9, 8, 2, 128, 660, dict(compaction="fill")),
     (20, 8, 4, 128, 700, dict(compaction="fill")),
     (1, 4, 2, 128, 1024, dict(compaction="fill")),
     (1, 4, 2, 128, 900, dict(rule="sum_recent")),
