@@ -1,5 +1,7 @@
 // Stand-alone eviction kernel: one CTA per (sample, kv-head) cache.  Used after a prefill block
 // (candidates = cached pairs + the block's pairs) and by bm_evict (candidates = cached pairs).
+#include <algorithm>
+
 #include "evict.cuh"
 
 namespace bm {
@@ -33,25 +35,22 @@ cudaError_t launch_w(const CacheView& c, const EvictArgs& e, int cluster, cudaSt
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 
-// A call of few caches shares each among a cluster, so that more SMs move rows -- at most 8 CTAs (64 bytes of a row
-// each), only clusters that are all resident at once, and at least 96 KB of rows for each CTA (a cluster's barrier costs
-// about 1 us).  Grids of at most one CTA per SM with more than a chunk of 64 KB to move keep twice as many pieces in
-// flight (a chunk is one round trip to memory).  us per call, against one CTA per cache with 64 KB chunks: 8 caches cut
-// from 1536 to 1024 pairs of 512 bytes 10.9 -> 8.6 (clusters of 8), 16 caches cut from 1024 to 512 pairs of 1 KB 12.2 ->
-// 8.7 (4), 32 caches of 1024 to 512 pairs of 512 bytes 9.5 -> 8.3 (4), 128 caches of 768 to 512 pairs 10.5 -> 10.0.
-template <typename T, int D, bool FILL>
-cudaError_t launch_f(const CacheView& c, const EvictArgs& e, cudaStream_t st) {
-  const int units = c.nsamples * c.Hkv, most = units <= 8 ? 8 : units <= 32 ? 4 : units <= 64 ? 2 : 1;
-  const size_t bytes = (size_t)e.target * D * 2 * sizeof(T);   // that may move per cache
-  int cluster = 1;
-  while (cluster < most && bytes > (size_t)cluster * (96 << 10)) cluster *= 2;
-  const bool wide = cluster * units <= sm_count() && bytes > (size_t)cluster * (64 << 10);
-  return wide ? launch_w<T, D, FILL, 16>(c, e, cluster, st) : launch_w<T, D, FILL, 8>(c, e, 1, st);
-}
-
+// A call of few caches shares each among a cluster of 8, 4 or 2 CTAs, so that more SMs move rows, as long as all are
+// resident at once and 256 KB and 64 KB for each CTA may move (a cluster's barrier costs about 1 us); its threads keep
+// twice as many pieces in flight.  us per prefill call, all three kernels (cluster / one CTA per cache): 8 caches cut from
+// 1536 to 1024 pairs of 512 bytes 40.0 / 41.2, 16 caches likewise 43.0 / 46.0 (4 CTAs), 32 caches from 1024 to 512 pairs 38.0
+// / 40.0 and from 2012 to 1500 63.4 / 69.0, 64 caches from 768 to 512 37.0 / 38.2 (2) and from 1536 to 1024 70.0 / 73.0; less
+// to move: 8 caches from 1024 to 512 32.0 / 31.5, 16 caches from 600 to 300 28.3 / 27.0.  Unordered caches move little and
+// gained nothing (8 caches to 1024 pairs 40.2 / 39.4); as many pieces in flight without a cluster cost 1 to 4 us (128
+// caches from 768 to 512 50.6 / 48.8).
 template <typename T, int D>
 cudaError_t launch_t(const CacheView& c, const EvictArgs& e, cudaStream_t st) {
-  return c.fill ? launch_f<T, D, true>(c, e, st) : launch_f<T, D, false>(c, e, st);
+  if (c.fill) return launch_w<T, D, true, 8>(c, e, 1, st);
+  const int units = c.nsamples * c.Hkv, cluster = units <= 8 ? 8 : units <= 32 ? 4 : units <= 64 ? 2 : 1;
+  const size_t bytes = (size_t)e.target * D * 2 * sizeof(T);   // that may move per cache
+  if (cluster > 1 && cluster * units <= sm_count() && bytes >= std::max((size_t)256 << 10, (size_t)cluster << 16))
+    return launch_w<T, D, false, 16>(c, e, cluster, st);
+  return launch_w<T, D, false, 8>(c, e, 1, st);
 }
 
 }  // namespace

@@ -71,7 +71,7 @@ __device__ inline void block_exclusive_scan2(int a, int b, int32_t* wsum /*[64]*
   __syncthreads();
 }
 
-// CTAs that share one cache (a cluster of `count`): every one of them ranks the candidates, each moves its own
+// CTAs that share one cache with ordered rows (a cluster of `count`): every one of them ranks the candidates, each moves its own
 // columns of the rows, and CTA 0 writes sum_weights and kv_ids once all have read them.
 struct EvictShare {
   int rank = 0, count = 1;
@@ -83,7 +83,7 @@ struct EvictShare {
   }
 };
 
-// W: 16-byte pieces a thread has in flight while rows move.
+// W: 16-byte pieces a thread has in flight while rows move; 16 in clusters.
 // FILL: the cache's rows are an unordered set (CacheView::fill); a template parameter, so that the instance for
 // ordered rows carries none of that code (with both in one function the ordered instance ran 15 % slower).
 template <typename T, int D, int NT, bool FILL, int W = 8>
@@ -201,9 +201,8 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
       if (k && (j >= target || j >= n_old)) s.src[sb++] = j;
     }
     __syncthreads();
-    share.everyone_has_read();
-    if (c.moved != nullptr && tid == 0 && share.rank == 0) atomicAdd(&c.moved[unit & 15], (unsigned long long)nf);
-    for (int k = share.rank == 0 ? tid : nf; k < nf; k += NT) {
+    if (c.moved != nullptr && tid == 0) atomicAdd(&c.moved[unit & 15], (unsigned long long)nf);
+    for (int k = tid; k < nf; k += NT) {
       const int j = s.src[k], r = s.dst[k];
       if (!row_ok(c, r)) continue;
       c.sum_weights[base + r] = s.score[j];
@@ -213,7 +212,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     constexpr int PRF = D * (int)sizeof(T) / 16;
     T* kslab = reinterpret_cast<T*>(c.k_slab) + base * D;
     T* vslab = reinterpret_cast<T*>(c.v_slab) + base * D;
-    for (int x0 = share.rank * 4 * NT; x0 < nf * PRF; x0 += share.count * 4 * NT) {
+    for (int x0 = 0; x0 < nf * PRF; x0 += 4 * NT) {
       uint4 kb[4], vb[4];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
@@ -365,10 +364,9 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
 
   // ---- rows: ascending chunks, every source row index >= its destination, loads of a chunk complete
   // (barrier) before its stores; later chunks only read rows above everything written so far.  The 2 PR pieces of a
-  // row (key, then value) are dealt out to the CTAs of the cache in contiguous shares where a cache has an SM or more to
-  // itself.
+  // row (key, then value) are dealt out to the CTAs of a cluster in contiguous shares.
   constexpr int PR = D * (int)sizeof(T) / 16;  // 16-byte pieces per row and tensor
-  if constexpr (W > 8) {   // a grid of at most one CTA per SM
+  if constexpr (W > 8) {
     const int PC = 2 * PR / share.count;         // pieces per row of this CTA (a power of two)
     const int RC = NT * W / PC;                  // rows per chunk
     const int pc = share.rank * PC + (tid & (PC - 1)), rt = tid / PC;   // this thread's piece, its first row in a chunk

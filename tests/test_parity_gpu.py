@@ -374,10 +374,16 @@ def test_score_pass_of_short_blocks_against_long_caches(b, Hkv, g, d, B, K, kw):
 
 @pytest.mark.parametrize("b,Hkv,d,dtype,K,kw", [
     (1, 2, 128, "bf16", 1100, {}),                          # clusters of 8, a ragged last chunk
-    (2, 8, 64, "bf16", 900, {}),                            # clusters of 2 (less than 96 KB of rows per further CTA)
+    (2, 8, 64, "bf16", 900, {}),                            # too little to move for a cluster
     (3, 8, 64, "f32", 700, {}),                             # clusters of 4
-    (1, 4, 128, "f32", 513, dict(compaction="fill")),       # unordered rows, shared among a cluster
+    (1, 4, 128, "f32", 513, dict(compaction="fill")),       # unordered rows
     (1, 4, 128, "bf16", 600, dict(rule="average_std")),     # the second accumulator is read after the first select
+    (1, 4, 128, "bf16", 1100, dict(rule="average_std")),    # ... in a cluster of 8
+    (1, 8, 128, "bf16", 1030, dict(rule="window_pooled", rule_params=dict(window=16, pool=5))),
+    (1, 8, 128, "bf16", 1024, {}),                          # exactly enough rows for clusters of 8
+    (2, 8, 128, "bf16", 512, {}),                           # ... of 4
+    (5, 8, 128, "bf16", 512, {}),                           # ... of 2
+    (8, 8, 64, "f32", 600, {}),                             # clusters of 2
     (1, 4, 128, "bf16", 600, dict(rule="window_pooled", rule_params=dict(window=16, pool=5))),
     (20, 8, 128, "bf16", 130, {}),                          # more caches than SMs: small chunks
 ])
