@@ -33,8 +33,9 @@ __host__ __device__ inline size_t evict_smem_layout(unsigned char* base, int n_c
   size_t o_score = take(sizeof(float) * n_cand), o_id = take(sizeof(int32_t) * n_cand);
   size_t o_bits = take(sizeof(uint32_t) * n_cand);
   size_t o_src = take(sizeof(int32_t) * (target > 0 ? target : 1)), o_dst = take(sizeof(int32_t) * (target > 0 ? target : 1));
-  // (the histograms lie where src and dst will be: they are done with when those are written)
-  const size_t o_hist = target >= 512 ? o_src : take(sizeof(uint32_t) * 1024);
+  // (the histograms lie where src and dst will be: they are done with when those are written.  The 1 KB that is kept
+  // behind these holds nothing: the size decides which calls are refused, and those stay the same.)
+  const size_t o_tail = take(sizeof(uint32_t) * (target >= 512 ? 256 : 1024)), o_hist = target >= 512 ? o_src : o_tail;
   size_t o_misc = take(sizeof(int32_t) * 8), o_wsum = take(sizeof(int32_t) * 64);
   if (s != nullptr) {
     s->score = reinterpret_cast<float*>(base + o_score);

@@ -392,6 +392,21 @@ def test_evictions_by_grid_size(b, Hkv, d, dtype, K, kw):
     run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=2, **kw)
 
 
+def test_largest_cut_of_a_call():
+    # the largest candidate set: the cut's work arrays fit a CTA's shared memory up to 10460 pairs kept
+    f = lambda h: torch.zeros(1, 12288, h, 64, device="cuda", dtype=torch.bfloat16)
+    for keep in (10461, 10460):
+        cache = bm.BatchMaxCache(bm.Config(batch=1, n_q_heads=1, n_kv_heads=1, head_dim=64, kv_max=keep, block_max=12288))
+        if keep > 10460:
+            with pytest.raises(bm.BMError) as err:
+                cache.prefill_block(f(1), f(1), f(1), 0, evict_to=keep)
+            assert err.value.code == 3 and cache.length()[0] == 0
+        else:
+            cache.prefill_block(f(1), f(1), f(1), 0, evict_to=keep)
+            assert cache.status() == 0 and cache.length()[0] == keep
+        cache.close()
+
+
 @pytest.mark.parametrize("b,Hkv,d,K", [(2, 4, 128, 1024), (4, 8, 64, 1500), (24, 8, 128, 700)])
 def test_decode_stream_is_bitwise_independent_of_sample_ranges(b, Hkv, d, K):
     import torch
