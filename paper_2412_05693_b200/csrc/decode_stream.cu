@@ -630,7 +630,8 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
 #pragma unroll
           for (int h = 0; h < G; ++h) t[h] += __shfl_xor_sync(0xffffffffu, t[h], off);
 #pragma unroll
-        for (int h = 0; h < G; ++h) f[h] = (q_real && mc[h] != -INFINITY) ? ex2(mc[h] - top[h]) / t[h] : 0.f;
+        for (int h = 0; h < G; ++h)   // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
+          f[h] = (q_real && (mc[h] != -INFINITY || top[h] == -INFINITY)) ? ex2(mc[h] - top[h]) / t[h] : 0.f;
       }
       // ---- sum_weights += attn_weights (heads added in a fixed order), candidate for eviction, bf16 exponentials
       // (the pair with the smallest ranking value leaves; ties: the higher position -- kv_ids, not rows: the rows of an

@@ -407,6 +407,21 @@ def test_largest_cut_of_a_call():
         cache.close()
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K", [(1, 4, 2, 128, 1024), (2, 8, 1, 64, 900), (20, 8, 4, 128, 700), (40, 8, 2, 64, 60)])
+def test_decode_step_with_logits_that_are_all_minus_infinity(b, Hkv, g, d, K):
+    # softmax of such a row is NaN whatever the kernel and the cluster, and stays in its own cache
+    f = lambda *s: torch.rand(*s, device="cuda").bfloat16() + 0.5
+    k = f(b, K, Hkv, d)
+    k[b // 2, :, 1] = -float("inf")
+    cache = bm.BatchMaxCache(bm.Config(batch=b, n_q_heads=g * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=K, block_max=K))
+    cache.prefill_block(f(b, K, g * Hkv, d), k, f(b, K, Hkv, d), 0)
+    out = cache.decode_step(f(b, g * Hkv, d), k[:, 0].contiguous(), f(b, Hkv, d)).view(b, Hkv, g, d)
+    assert cache.status() == 0
+    nan = torch.zeros(b, Hkv, dtype=torch.bool, device="cuda")
+    nan[b // 2, 1] = True
+    assert torch.equal(torch.isnan(out).all(-1).all(-1), nan) and torch.equal(torch.isnan(out).any(-1).any(-1), nan)
+
+
 @pytest.mark.parametrize("b,Hkv,d,K", [(2, 4, 128, 1024), (4, 8, 64, 1500), (24, 8, 128, 700)])
 def test_decode_stream_is_bitwise_independent_of_sample_ranges(b, Hkv, d, K):
     import torch
