@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "smem_configured.h"
+
 namespace bm {
 
 // Device-side view of one layer's slabs for a contiguous range of samples (Sec. 3: one cache per
@@ -107,25 +109,6 @@ cudaError_t launch_wait_timeout_selftest(int* status, cudaStream_t st);
 cudaError_t launch_row_check_selftest(const CacheView& c, cudaStream_t st);
 cudaError_t launch_attn_tc(int d, const CacheView& c, const BlockArgs& a, cudaStream_t st, int* used);
 cudaError_t launch_score_tc(int d, const CacheView& c, const BlockArgs& a, cudaStream_t st, int* used);
-
-// cudaFuncSetAttribute applies to the current device only, so the largest dynamic shared-memory size a kernel has
-// been configured for is remembered per device (a process may hold handles on several GPUs).
-struct SmemConfigured {
-  size_t bytes[64] = {};
-  template <typename Kernel>
-  cudaError_t ensure(Kernel kernel, size_t smem) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (smem > bytes[dev]) {
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      bytes[dev] = smem;
-    }
-    return cudaSuccess;
-  }
-};
 
 // Launch as a programmatic dependent of the stream's previous kernel: the grid may be started while that kernel is
 // still running; the kernel itself must execute pdl_wait() before it touches anything the predecessor may have
