@@ -330,7 +330,27 @@ def cfg_dict(wl, extra=None):
     return d
 
 
-def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch):
+def forward_kernel(wl, padded=False):
+    """The kernel that a full block's forward pass runs on, by the library's rule (launch_fwd_t in csrc/attn_tc.cu)."""
+    tiles = -(-wl.B * wl.g // 128)
+    if wl.dtype != "bf16":
+        return "attn_fwd_simt"
+    return "attn_fwd_pair" if not padded and tiles // 2 * wl.b * wl.Hkv >= 1024 else "attn_fwd_split"
+
+
+def decode_kernel(wl):
+    """The kernel of an evicting decode step on caches of K pairs that do not stay in L2 (or do, where there is no more than
+    one per SM), by the library's rule (stream_is_faster in csrc/decode_mma.cu); None where neither table row applies."""
+    caches, kib, mib = wl.b * wl.Hkv, (wl.K + 1) * wl.d * 4 / 1024, wl.b * wl.Hkv * wl.L * (wl.K + 1) * (4 * wl.d + 8) / 2 ** 20
+    if wl.dtype != "bf16":
+        return None
+    if mib <= 104:
+        return "decode_mma_kernel" if wl.d == 128 and caches > 64 else None
+    return "decode_stream_kernel" if caches <= 148 or kib >= (256 if caches <= 296 else 172 if caches <= 592 else 150) \
+        else "decode_mma_kernel"
+
+
+def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch, padded=False):
     """Tensor-core roofline of the forward kernel: useful FLOPs (4*d per visible pair) over its launches' time."""
     flops = 4.0 * wl.d * prefill_pairs(wl) * wl.b * wl.Hq * wl.L
     achieved = flops / (attn_ms * 1e-3) / 1e12
@@ -339,13 +359,13 @@ def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch
     at_max = bool(clocks and clocks.get("sm_mhz") and clocks.get("sm_max_mhz")
                   and clocks["sm_mhz"] >= 0.97 * clocks["sm_max_mhz"])
     peak = burst if at_max else sust
-    return {"bound": "tensor", "kernel": "prefill-block attention forward (attn_fwd_pair, attn_fwd_split on small grids)", "achieved": achieved,
+    return {"bound": "tensor", "kernel": f"prefill-block attention forward ({forward_kernel(wl, padded)})", "achieved": achieved,
             "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "frac_of_burst_peak": achieved / burst, "frac_of_sustained_peak": achieved / sust,
             "peak_source": f"{pk_src} bf16 matmul, " + ("burst figure: the sampled SM clock stayed at its maximum"
                                                          if at_max else
                                                          "sustained figure: the sampled SM clock was below its maximum"),
-            "traffic": dram_traffic("attn_fwd_pair", samples_per_launch),
+            "traffic": dram_traffic(forward_kernel(wl, padded), samples_per_launch),
             "launches_per_step": attn_n, "avg_launch_ms": attn_ms / max(attn_n, 1),
             "algorithmic": "4*d FLOP per visible (query, key) pair; the score pass's recompute is not counted"}
 
@@ -487,11 +507,11 @@ def run_max_batch(args, name, rank, world, local_rank, sampler):
         gbs = dec_bytes / (kernel_ms["decode"] * 1e-3) / 1e9
         gbs_mv = (dec_bytes + move_bytes) / (kernel_ms["decode"] * 1e-3) / 1e9
         rooflines["decode"] = {
-            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_stream_kernel, decode_mma_kernel on short caches)",
+            "bound": "hbm", "kernel": "decode step with score update and eviction" + (f" ({decode_kernel(wl)})" if decode_kernel(wl) else ""),
             "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": gbs / pk["hbm_gbs"],
             "achieved_with_compaction_writes": gbs_mv, "frac_with_compaction_writes": gbs_mv / pk["hbm_gbs"],
             "rows_moved_per_cache_and_step": moved.get("decode", 0) / max(1, wl.b * wl.Hkv * wl.L * wl.steps),
-            "traffic": dram_traffic("decode_stream_kernel", DECODE_MICRO),
+            "traffic": dram_traffic(decode_kernel(wl), DECODE_MICRO),
             "peak_source": f"{pk_src} (HBM copy)", "launches_per_step": kernel_n["decode"],
             "avg_launch_ms": kernel_ms["decode"] / max(kernel_n["decode"], 1),
             "algorithmic": "(n+1)*(2*d*e+16) + 2*d*e + 2*g*d*e bytes per cache and step, compaction moves not counted"}
@@ -775,7 +795,8 @@ def run_resident(args, wl, rank, world, local_rank, sampler, light=False):
     rooflines = {}
     attn_ms, attn_n = prof["attn_fwd"]
     if attn_ms > 0:
-        rooflines["attn_fwd"] = forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, wl.b)
+        rooflines["attn_fwd"] = forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, wl.b,
+                                                  args.ragged)
     dec_ms, dec_n = prof.get("decode", (0.0, 0))
     if dec_ms > 0:
         dec_bytes = decode_bytes_per_cache(wl, calls) * wl.b * wl.Hkv * wl.L
@@ -785,12 +806,12 @@ def run_resident(args, wl, rank, world, local_rank, sampler, light=False):
         one_step(moved=moved).close()             # one more eager pass with the device-side counters on
         move_bytes = moved.get("decode", 0) * 2.0 * wl.d * wl.elem_bytes
         rooflines["decode"] = {
-            "bound": "hbm", "kernel": "decode step with score update and eviction (decode_stream_kernel, decode_mma_kernel on short caches)",
+            "bound": "hbm", "kernel": "decode step with score update and eviction" + (f" ({decode_kernel(wl)})" if decode_kernel(wl) else ""),
             "achieved": gbs, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": gbs / pk["hbm_gbs"],
             "achieved_with_per_launch_events": dec_bytes / (dec_ms * 1e-3) / 1e9, "ms_in_timed_region": in_region_ms,
             "achieved_with_compaction_writes": (dec_bytes + move_bytes) / (in_region_ms * 1e-3) / 1e9,
             "rows_moved_per_cache_and_step": moved.get("decode", 0) / max(1, wl.b * wl.Hkv * dec_n),
-            "traffic": dram_traffic("decode_mma_kernel", wl.b),
+            "traffic": dram_traffic(decode_kernel(wl), wl.b),
             "in_timed_region": (f"every decode step runs as {n_ranges} concurrent launches, one per sample range; "
                                 "achieved = bytes of all of them / their time in the region") if n_ranges > 1 else
                                "one launch per decode step",

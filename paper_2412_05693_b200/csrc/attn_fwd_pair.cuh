@@ -2,19 +2,17 @@
 // TcArgs): the softmax of one tile runs under the MMAs of the other.
 //
 // Per tile the chain logits -> softmax -> P.V -> next logits is serial, because the bf16 probabilities take the place of
-// the logits in tensor memory (S 128 + O 128 columns per tile: two tiles fill it).  That chain is what bounds the kernel:
-// 3800 cycles a key tile in steady state -- tensor-memory read 150, maximum 300, exponentials and publication 1600 (1100
-// where nothing else uses the scheduler), from the last arrival to the issuing thread 300, four MMAs of P.V 300, eight
-// of Q.K 650, to the waiting softmax 370 -- while the two tiles' MMAs take 2100 of it and their softmaxes, side by side,
-// 1820.  A thread holds all 128 logits of its row in registers: one read of tensor memory, no exchange of maxima.  Every
-// fourth pair of exponentials is a polynomial of degree 5 on the FMA and integer pipes (all on the special-function
-// unit: 7 % slower; an eighth: the same); a warp arrives once on a barrier, not lane by lane (9 % slower).
+// the logits in tensor memory (S 128 + O 128 columns per tile: two tiles fill it).  That chain is what bounds the kernel
+// (ncu, profiles/kernels_48_samples.md: tensor pipe busy 48 % of the cycles, special-function unit 37 %, issue slots 39 %,
+// DRAM 14 %; most stalls are waits on tensor memory and barriers).  A thread holds all 128 logits of its row in registers:
+// one read of tensor memory, no exchange of maxima.  Every fourth pair of exponentials is a polynomial of degree 5 on the
+// FMA and integer pipes (all on the special-function unit: 7 % slower; an eighth: the same); a warp arrives once on a
+// barrier, not lane by lane (9 % slower).
 //
 // Measured at 48 samples, 32 heads in groups of 4, d = 128, a block of 512 against 1024 pairs: 936 -> 963 TFLOP/s against
 // the kernel with one tile per CTA and two CTAs per SM; 32 samples, 32 heads, a block of 1024: 930 -> 955; d = 64, 701
-// pairs, groups of 8: 162 -> 156 us.  Not kept: one issuing thread for both tiles (936: 1600 of its 3900 cycles were
-// waits on complete barriers and commits), issuers without turns (745: the tiles fall into step), publishing after 96
-// keys instead of 64 (882), exponentials relative to the running maximum with the tile's formed beside them (866), two
+// pairs, groups of 8: 162 -> 156 us.  Not kept: one issuing thread for both tiles (936), issuers without turns (745: the
+// tiles fall into step), publishing after 96 keys instead of 64 (882), exponentials relative to the running maximum with the tile's formed beside them (866), two
 // threads per row (934), tile B started half a period later (936 to 955), polling softmax warps (952).
 //
 // Warps 0-3: rows of tile A, 4-7: rows of tile B, 8 and 9: MMA issue for A and B, 10: TMA producer.  Shared memory: Q_A |
@@ -113,8 +111,8 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
           load_stage(e);
         }
     } else if (warp < kTmaWarp && lane == 0) {
-      // ---------------------------------------------------------------- MMA issuer of tile x (one thread each: a single
-      // one spent 1600 of a pair's 3900 cycles on waits for barriers that were complete and on commits)
+      // ---------------------------------------------------------------- MMA issuer of tile x (one thread each: a
+      // single one for both was 3 % slower)
       const int x = warp - kMmaWarp, Tx = x ? T1 : T0;
       const uint32_t idesc_qk = instr_desc(kTileM, kTileN, 0, 0);
       const uint32_t idesc_pv = instr_desc(kTileM, D, 0, 1);  // V is MN-major: d contiguous, keys along K
@@ -135,7 +133,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
       };
       auto wait = [&](int b, uint32_t parity) { mbar_poll(&bars[b], parity, abort_flag, a.status); };
       // The two issuers take turns, so that one tile's MMAs run behind each other and not between the other's: left to
-      // themselves the tiles fell into step, both in their softmax and then both in their MMAs (4200 cycles a pair).
+      // themselves the tiles fell into step, both in their softmax and then both in their MMAs (745 against 963 TFLOP/s).
       auto my_turn = [&](int e) {                // A's e-th turn comes after B's e-1st, B's after A's e-th
         if (T1 > 0 && (x == 1 || e > 0)) wait(B_TURN + x, (uint32_t)(x ? e : e - 1) & 1);
       };

@@ -8,8 +8,8 @@
 // rows x 4 keys of a logit tile and 4 rows x D/16 outputs, reads its operands as 16-byte pieces, multiplies pairs with
 // packed instructions and keeps an accumulator's two products of a step apart; 16 warps share an SM; K and V tiles
 // arrive by asynchronous copies under the arithmetic that does not need them.  Measured with 4 samples, 16 heads in
-// groups of 4, d = 128, a block of 256 against 1280 cached pairs: forward kernel 639 -> 407 us (29 TFLOP/s; busiest SM's
-// fp32 pipes 60 %, the rest is 256 CTAs on 148 SMs), score pass 324 -> 226 us, against 4 x 4 values per thread from
+// groups of 4, d = 128, a block of 256 against 1280 cached pairs: forward kernel 639 -> 407 us (29 TFLOP/s; fp32 pipes
+// busy 56 % of the active cycles, 256 CTAs on 148 SMs: profiles/kernels_48_samples.md), score pass 324 -> 226 us, against 4 x 4 values per thread from
 // scalar reads between barriers; 8 rows per thread on half the threads: 434 us.
 #include "common.cuh"
 
