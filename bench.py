@@ -330,12 +330,9 @@ def cfg_dict(wl, extra=None):
     return d
 
 
-def forward_kernel(wl, padded=False):
-    """The kernel that a full block's forward pass runs on, by the library's rule (launch_fwd_t in csrc/attn_tc.cu)."""
-    tiles = -(-wl.B * wl.g // 128)
-    if wl.dtype != "bf16":
-        return "attn_fwd_simt"
-    return "attn_fwd_pair" if not padded and tiles // 2 * wl.b * wl.Hkv >= 1024 else "attn_fwd_split"
+def forward_kernel(wl):
+    """The kernel that a full block's forward pass runs on (csrc/attn_tc.cu, csrc/attn_simt.cu)."""
+    return "attn_fwd_pair" if wl.dtype == "bf16" else "attn_fwd_simt"
 
 
 def decode_kernel(wl):
@@ -359,13 +356,13 @@ def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch
     at_max = bool(clocks and clocks.get("sm_mhz") and clocks.get("sm_max_mhz")
                   and clocks["sm_mhz"] >= 0.97 * clocks["sm_max_mhz"])
     peak = burst if at_max else sust
-    return {"bound": "tensor", "kernel": f"prefill-block attention forward ({forward_kernel(wl, padded)})", "achieved": achieved,
+    return {"bound": "tensor", "kernel": f"prefill-block attention forward ({forward_kernel(wl)})", "achieved": achieved,
             "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "frac_of_burst_peak": achieved / burst, "frac_of_sustained_peak": achieved / sust,
             "peak_source": f"{pk_src} bf16 matmul, " + ("burst figure: the sampled SM clock stayed at its maximum"
                                                          if at_max else
                                                          "sustained figure: the sampled SM clock was below its maximum"),
-            "traffic": dram_traffic(forward_kernel(wl, padded), samples_per_launch),
+            "traffic": dram_traffic(forward_kernel(wl), samples_per_launch),
             "launches_per_step": attn_n, "avg_launch_ms": attn_ms / max(attn_n, 1),
             "algorithmic": "4*d FLOP per visible (query, key) pair; the score pass's recompute is not counted"}
 

@@ -56,13 +56,9 @@ __global__ void __launch_bounds__(320, 1) attn_block_onepass(const __grid_consta
   auto load_tile = [&](int t, bool is_v) {                   // key tile t into slot t
     unsigned char* dst = sm + L::kKV + t * L::kTileBytes;
     mbar_expect_tx(&bars[B_KVFULL + t], L::kTileBytes);
-    for (int c = 0; c < L::kChunks; ++c) {
-      if (t < t_old)
-        tma_load_3d(dst + c * 16384, is_v ? &maps.v_slab : &maps.k_slab, c * 64, t * kTileN, unit, &bars[B_KVFULL + t]);
-      else
-        tma_load_4d(dst + c * 16384, is_v ? &maps.v_blk : &maps.k_blk, c * 64, kh, (t - t_old) * kTileN, smp,
-                    &bars[B_KVFULL + t]);
-    }
+    const bool old = t < t_old;
+    const CUtensorMap* m = old ? (is_v ? &maps.v_slab : &maps.k_slab) : (is_v ? &maps.v_blk : &maps.k_blk);
+    tma_load_5d(dst, m, 0, old ? 0 : kh, (old ? t : t - t_old) * kTileN, old ? unit : smp, 0, &bars[B_KVFULL + t]);
   };
   if (warp == kTmaWarp && lane == 0) {
     *abort_flag = 0;
@@ -259,7 +255,10 @@ __global__ void __launch_bounds__(320, 1) attn_block_onepass(const __grid_consta
     fence_async_smem();
     named_bar_sync(1, 256);
     if (tid == 0) {
-      for (int c = 0; c < L::kChunks; ++c) tma_store_5d(&maps.o, stage + c * 16384, c * 64, 0, kh, 0, smp);
+#pragma unroll 1
+      for (int i0 = 0; i0 < a.I; i0 += 32 / a.g)   // 32 rows at a time
+        for (int c = 0; c < L::kChunks; ++c)
+          tma_store_5d(&maps.o, stage + c * 16384 + i0 * a.g * 128, c * 64, 0, kh, i0, smp);
       tma_store_commit_and_wait();
     }
   }

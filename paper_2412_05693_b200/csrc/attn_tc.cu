@@ -1,8 +1,8 @@
 // bf16 tensor-core path of the block forward pass (Sec. 3.2) for sm_100a:
-//   attn_fwd_split (attn_fwd_split.cuh) and, for large grids, attn_fwd_pair (attn_fwd_pair.cuh):
+//   attn_fwd_pair (attn_fwd_pair.cuh):
 //                 out = softmax(scale q k^T) v over the cached pairs and the block's causal pairs, plus the
 //                 log2-sum-exp of every query row.  QK^T and PV run on tcgen05 with TMA-staged
-//                 tiles and TMEM accumulators; an SM works on two tiles of 128 query rows at a time.
+//                 tiles and TMEM accumulators; an SM works on two tiles of 128 query rows, or two key tiles, at a time.
 //   score_tc    : sum_weights += sum_i attn_weights[i].  Recomputes the transposed logits S^T = K Q^T so that
 //                 a TMEM lane is a key; each thread then sums exp2(s - lse) over the queries of its own key
 //                 in a fixed order (deterministic, no atomics).
@@ -26,10 +26,10 @@ constexpr float kRescaleThreshold = 8.0f;  // stale row max is kept until the tr
 
 struct TcMaps {
   CUtensorMap q;       // 5-d: (d, g, Hkv, I, nsamples)
-  CUtensorMap o;       // same shape over the output
-  CUtensorMap k_slab;  // 3-d: (d, n_old, units)
+  CUtensorMap o;       // same shape over the output, boxes of 32 rows (a warp's)
+  CUtensorMap k_slab;  // 5-d: (64, 1, n_old, units, d / 64): a box is a whole tile of keys
   CUtensorMap v_slab;
-  CUtensorMap k_blk;   // 4-d: (d, Hkv, I, nsamples)
+  CUtensorMap k_blk;   // 5-d: (64, Hkv, I, nsamples, d / 64), likewise
   CUtensorMap v_blk;
 };
 
@@ -49,12 +49,11 @@ struct TcArgs {
   int first_row;     // query rows below it add nothing to the column sums (rules that look at the last queries only)
   int overwrite;     // 1: the column sums replace sum_weights instead of being added
   int key_tiles;     // key tiles per CTA of the score pass (QRES)
-  int row_tiles;     // row tiles per CTA of attn_fwd_pair: 2 or 1
+  int across;        // attn_fwd_pair: 1 = row tiles in order over all caches (grid.x = caches), 0 = within a cache
   float* sum_sq;     // rule 4: sums of squared weights (cached pairs / the block's pairs), else null
   float* new_sq;
 };
 
-#include "attn_fwd_split.cuh"
 #include "attn_fwd_pair.cuh"
 #include "attn_onepass.cuh"
 
@@ -110,10 +109,8 @@ score_tc(const __grid_constant__ TcMaps maps, const TcArgs a) {
 
   auto load_keys = [&](unsigned char* dst, int kt, uint64_t* bar) {
     mbar_expect_tx(bar, L::kTileBytes);
-    for (int c = 0; c < L::kChunks; ++c) {
-      if (kt < t_old) tma_load_3d(dst + c * 16384, &maps.k_slab, c * 64, kt * kTileN, unit, bar);
-      else tma_load_4d(dst + c * 16384, &maps.k_blk, c * 64, kh, (kt - t_old) * kTileN, smp, bar);
-    }
+    const bool old = kt < t_old;
+    tma_load_5d(dst, old ? &maps.k_slab : &maps.k_blk, 0, old ? 0 : kh, (old ? kt : kt - t_old) * kTileN, old ? unit : smp, 0, bar);
   };
   auto load_queries = [&](unsigned char* dst, int qt, uint64_t* bar) {
     mbar_expect_tx(bar, L::kTileBytes);
@@ -316,21 +313,23 @@ bool build_maps(int d, const CacheView& c, const BlockArgs& a, TcMaps* m) {
     cuuint64_t str[4] = {D * e, (cuuint64_t)c.g * D * e, (cuuint64_t)c.Hq * D * e, (cuuint64_t)a.I * c.Hq * D * e};
     cuuint32_t box[5] = {64, (cuuint32_t)c.g, 1, (cuuint32_t)(kTileM / c.g), 1};
     if (!encode(&m->q, a.q, 5, dims, str, box)) return false;
+    box[3] = (cuuint32_t)(32 / c.g);
     if (!encode(&m->o, a.out, 5, dims, str, box)) return false;
   }
   {
-    cuuint64_t dims[3] = {D, (cuuint64_t)(c.n_old > 0 ? c.n_old : 1), units};
-    cuuint64_t str[2] = {D * e, (cuuint64_t)c.cap * D * e};
-    cuuint32_t box[3] = {64, kTileN, 1};
-    if (!encode(&m->k_slab, c.k_slab, 3, dims, str, box)) return false;
-    if (!encode(&m->v_slab, c.v_slab, 3, dims, str, box)) return false;
+    // a tile of keys in one copy: the 64-element chunks of a row are the outermost dimension
+    cuuint64_t dims[5] = {64, 1, (cuuint64_t)(c.n_old > 0 ? c.n_old : 1), units, D / 64};
+    cuuint64_t str[4] = {D * e, D * e, (cuuint64_t)c.cap * D * e, 128};
+    cuuint32_t box[5] = {64, 1, kTileN, 1, (cuuint32_t)(d / 64)};
+    if (!encode(&m->k_slab, c.k_slab, 5, dims, str, box)) return false;
+    if (!encode(&m->v_slab, c.v_slab, 5, dims, str, box)) return false;
   }
   {
-    cuuint64_t dims[4] = {D, (cuuint64_t)c.Hkv, (cuuint64_t)a.I, (cuuint64_t)c.nsamples};
-    cuuint64_t str[3] = {D * e, (cuuint64_t)c.Hkv * D * e, (cuuint64_t)a.I * c.Hkv * D * e};
-    cuuint32_t box[4] = {64, 1, kTileN, 1};
-    if (!encode(&m->k_blk, a.k, 4, dims, str, box)) return false;
-    if (!encode(&m->v_blk, a.v, 4, dims, str, box)) return false;
+    cuuint64_t dims[5] = {64, (cuuint64_t)c.Hkv, (cuuint64_t)a.I, (cuuint64_t)c.nsamples, D / 64};
+    cuuint64_t str[4] = {D * e, (cuuint64_t)c.Hkv * D * e, (cuuint64_t)a.I * c.Hkv * D * e, 128};
+    cuuint32_t box[5] = {64, 1, kTileN, 1, (cuuint32_t)(d / 64)};
+    if (!encode(&m->k_blk, a.k, 5, dims, str, box)) return false;
+    if (!encode(&m->v_blk, a.v, 5, dims, str, box)) return false;
   }
   return true;
 }
@@ -346,26 +345,13 @@ TcArgs make_args(const CacheView& c, const BlockArgs& a) {
   t.overwrite = rule_overwrites(c.rule) ? 1 : 0;
   t.sum_sq = c.sum_sq; t.new_sq = a.new_sq;
   t.key_tiles = 1;
-  t.row_tiles = 2;
+  t.across = 0;
   return t;
 }
 
 // maps of the call in flight: built by the forward launcher, reused by the score launcher
 thread_local TcMaps g_maps;            // per thread: handles used from different threads do not share them
 thread_local const void* g_maps_q = nullptr;
-
-template <int D, bool PAD>
-cudaError_t launch_fwd_split(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
-  using L = SplitSmem<D>;
-  static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(attn_fwd_split<D, PAD>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
-  const int R = a.I * c.g;
-  dim3 grid((R + kTileM - 1) / kTileM, c.nsamples * c.Hkv);
-  ProfileScope prof(kAttnFwd, st);
-  attn_fwd_split<D, PAD><<<grid, L::kThreads, L::kTotal, st>>>(g_maps, make_args(c, a));
-  count_launch();
-  return cudaGetLastError();
-}
 
 // the forward launch of the call in flight has taken the column sums as well: no score pass follows
 thread_local bool g_scores_done = false;
@@ -389,19 +375,19 @@ cudaError_t launch_onepass(const CacheView& c, const BlockArgs& a, cudaStream_t 
   return cudaGetLastError();
 }
 
-template <int D>
+template <int D, bool PAD, bool SPLIT>
 cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
   using L = PairSmem<D>;
   static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(attn_fwd_pair<D>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
-  const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
+  if (cudaError_t e = configured.ensure(attn_fwd_pair<D, PAD, SPLIT>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
+  const int tiles = (a.I * c.g + kTileM - 1) / kTileM, units = c.nsamples * c.Hkv;
   TcArgs args = make_args(c, a);
-  // One tile per CTA while each has an SM to itself (8 caches, a block of 512: 29 us against 34 on half as many SMs; 32
-  // caches of 4 tiles 23 against 25; 24 caches of 10 tiles 47 against 31): a row's arithmetic is the same either way.
-  args.row_tiles = tiles * c.nsamples * c.Hkv <= sm_count() ? 1 : 2;
+  // Row tiles in order over all caches (the longest first) where the call's keys and values stay in L2: 32 caches of 512
+  // pairs and a block of 512 40.3 us, cache by cache 43.3; 192 caches of 499, 74 MB, the same; 1024 caches 1380 / 1254.
+  args.across = (size_t)units * (c.n_old + a.I) * D * 4 <= (size_t)64 << 20;
+  const int groups = SPLIT ? tiles : (tiles + 1) / 2;
   ProfileScope prof(kAttnFwd, st);
-  const dim3 grid((tiles + args.row_tiles - 1) / args.row_tiles, c.nsamples * c.Hkv);
-  attn_fwd_pair<D><<<grid, L::kThreads, L::kTotal, st>>>(g_maps, args);
+  attn_fwd_pair<D, PAD, SPLIT><<<args.across ? dim3(units, groups) : dim3(groups, units), L::kThreads, L::kTotal, st>>>(g_maps, args);
   count_launch();
   return cudaGetLastError();
 }
@@ -409,14 +395,13 @@ cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t
 template <int D>
 cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
   if (onepass_applies(c, a)) return launch_onepass<D>(c, a, st);
-  // Two tiles per CTA (launch_fwd_pair) where the handle's batch makes 1024 pairs of tiles or more (512 pairs at d = 64:
-  // 99 against 96 us for one tile per CTA, 768 pairs at d = 128: 104 against 102, 1152 pairs at d = 64: 156 against 162,
-  // 3072 pairs at d = 128: 549 against 563).  The handle's caches decide and not the call's: the two kernels round
-  // differently, and outputs do not depend on how a batch is cut into sample ranges -- ranges of a padded handle that
-  // hold no padding included, since there is no padding instance of the pair kernel.
   const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
-  if (!c.padded && (long long)(tiles / 2) * c.layer_units >= 1024) return launch_fwd_pair<D>(c, a, st);
-  return c.left_pad != nullptr ? launch_fwd_split<D, true>(c, a, st) : launch_fwd_split<D, false>(c, a, st);
+  // Both groups on one row tile while every row tile of the handle's batch has an SM to itself (128 row tiles of 12 key tiles
+  // 24.4 us, two row tiles per CTA 35.1; 256 row tiles 35.2 / 35.4).  The handle's caches decide and not the call's: the
+  // sums of a row are cut differently, and outputs do not depend on how a batch is cut into sample ranges.
+  if ((long long)tiles * c.layer_units <= sm_count())
+    return c.left_pad != nullptr ? launch_fwd_pair<D, true, true>(c, a, st) : launch_fwd_pair<D, false, true>(c, a, st);
+  return c.left_pad != nullptr ? launch_fwd_pair<D, true, false>(c, a, st) : launch_fwd_pair<D, false, false>(c, a, st);
 }
 
 template <int D, bool SQ, int EMU, bool QRES>

@@ -336,6 +336,42 @@ def test_forward_on_pairs_of_row_tiles_is_bitwise_independent_of_sample_ranges(b
         assert_same_run(base, run_free(wl, micro=1, pads=pads))
 
 
+# few row tiles: the two softmax groups of a CTA take the key tiles of one row tile in turn
+SPLIT_GRIDS = [(1, 1, 1, 128, 131, 0),    # two row tiles: one key tile (the second group has none), then two
+               (2, 2, 4, 64, 200, 129),   # cached tiles end in a single key; up to four key tiles
+               (1, 4, 8, 128, 70, 640),   # a row tile of 16 inputs, the last one ragged
+               (2, 1, 2, 64, 385, 257)]
+
+
+@pytest.mark.parametrize("b,Hkv,g,d,B,K", SPLIT_GRIDS)
+def test_forward_with_key_tiles_taken_in_turn(b, Hkv, g, d, B, K):
+    # plain keys, then one NaN, inf or -inf in a key of every cache; the logits of the first query are all -inf in the last
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen).bfloat16()
+    n = K + B
+    q, k, v = f(b, n, g * Hkv, d), f(b, n, Hkv, d), f(b, n, Hkv, d)
+    q[..., 3] = q[..., 3].abs() + 0.1                      # (an infinite element of a key gives logits of one sign)
+    hidden = torch.ones(n, n, device="cuda", dtype=torch.bool).triu(1)
+    for value in (None, float("nan"), float("inf"), -float("inf")):
+        if value is not None:
+            for u in range(b * Hkv):
+                k[u // Hkv, n // 2, u % Hkv, 3] = value
+        if value == -float("inf"):
+            k[:, 0, :, 3] = value
+        cache = bm.BatchMaxCache(bm.Config(batch=b, n_q_heads=g * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=n, block_max=max(B, K)))
+        parts = [cache.prefill_block(*(x[:, :K].contiguous() for x in (q, k, v)), 0)] if K else []
+        parts.append(cache.prefill_block(*(x[:, K:].contiguous() for x in (q, k, v)), K))
+        assert cache.status() == 0
+        out = torch.cat(parts, 1).float()
+        cache.close()
+        for s in range(b):
+            logits = torch.einsum("ihgd,jhd->hgij", q[s].float().view(n, Hkv, g, d), k[s].float()) / d ** 0.5
+            want = torch.einsum("hgij,jhd->ihgd", logits.masked_fill_(hidden, -float("inf")).softmax(-1), v[s].float())
+            want = want.reshape(n, g * Hkv, d)
+            assert torch.equal(torch.isnan(out[s]), torch.isnan(want))
+            assert (out[s] - want).nan_to_num_(0.0).abs().max() < 2e-2
+
+
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS[1:3])
 def test_forward_on_pairs_of_row_tiles_with_nan_and_inf_keys(b, Hkv, g, d, B, K, value):
