@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
   const bool q_real = a.pos >= pad;
 
   // queries of the group -> smem (fp32); the step's pair -> row n_old of the cache
+#pragma unroll 1
   for (int t = tid; t < G * D; t += kDecThreads) {
     const T* qp = reinterpret_cast<const T*>(a.q) + ((size_t)smp * c.Hq + kh * G) * D;
     s.q[t] = (float)qp[t];
@@ -97,6 +98,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
     T* dst = (tid < LPR ? kslab : vslab) + (size_t)c.n_old * D + pc * V;
     if (row_ok(c, c.n_old)) st_global_16(dst, ld_global_16(src));
   }
+#pragma unroll 1
   for (int j = tid; j < n1; j += kDecThreads) s.id[j] = (j < c.n_old) ? c.kv_ids[base + j] : a.pos;
   __syncthreads();
 
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
 #pragma unroll
       for (int e = 0; e < V; ++e) qr[h][e] = s.q[h * D + lr * V + e];
     // ---- logits (log2 domain): scale * log2(e) * <q_h, k_j>
+#pragma unroll 1
     for (int it = 0; it < n_iter; ++it) {
       const int j0 = it * RPI + slot;
       uint4 raw[kUnroll];
@@ -154,6 +157,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
 #pragma unroll
   for (int h = 0; h < G; ++h) {
     float m = -INFINITY;
+#pragma unroll 1
     for (int j = tid; j < n1; j += kDecThreads) m = fmaxf(m, s.p[h * n1p + j]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -167,6 +171,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
     for (int w = 0; w < kDecWarps; ++w) m = fmaxf(m, s.wred[h * kDecWarps + w]);
     mx[h] = m;
     float t = 0.f;
+#pragma unroll 1
     for (int j = tid; j < n1; j += kDecThreads) {
       const float e = ex2f(s.p[h * n1p + j] - m);
       s.p[h * n1p + j] = e;
@@ -189,6 +194,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
   // ---- normalise, sum_weights += attn_weights (group's heads added in a fixed order), eviction candidate
   float best_ave = INFINITY;
   int best_j = -1;
+#pragma unroll 1
   for (int j = tid; j < n1; j += kDecThreads) {
     float add = 0.f;
 #pragma unroll
@@ -238,6 +244,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
     hole = best_j;
     if (c.moved != nullptr && tid == 0) atomicAdd(&c.moved[unit & 15], (unsigned long long)(n1 - 1 - hole));
     // sum_weights / kv_ids in their final places: rows behind the hole move up by one
+#pragma unroll 1
     for (int j = tid; j < n1; j += kDecThreads) {
       if (j < hole) { if (j >= 0) c.sum_weights[base + j] = s.score[j]; }
       else if (j > hole) { c.sum_weights[base + j - 1] = s.score[j]; c.kv_ids[base + j - 1] = s.id[j]; }
@@ -254,6 +261,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
   for (int h = 0; h < G; ++h)
 #pragma unroll
     for (int e = 0; e < V; ++e) acc[h][e] = 0.f;
+#pragma unroll 1
   for (int it = 0; it < n_iter; ++it) {
     const int j0 = it * RPI + slot;
     uint4 raw[kUnroll];
@@ -287,6 +295,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
   }
   // K rows behind the hole: same one-row shift (re-read, mostly from L2: the logits pass just streamed them)
   if (evict_one) {
+#pragma unroll 1
     for (int it = hole / RPI; it < n_iter; ++it) {
       const int j0 = it * RPI + slot;
       uint4 raw[kUnroll];
@@ -318,6 +327,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_kernel(CacheView c, Decode
       for (int e = 0; e < V; ++e) s.ored[(warp * G + h) * D + lr * V + e] = acc[h][e];
   }
   __syncthreads();
+#pragma unroll 1
   for (int t = tid; t < G * D; t += kDecThreads) {
     float tot = 0.f;
 #pragma unroll

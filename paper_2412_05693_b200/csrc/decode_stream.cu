@@ -100,6 +100,7 @@ __device__ __forceinline__ void arrive_cluster(uint32_t addr) {
 __device__ __forceinline__ void wait_cluster(uint64_t* b, uint32_t parity, volatile int* abort_flag, int* status) {
   const uint32_t addr = smem_u32(b);
   if (*abort_flag) return;
+#pragma unroll 1
   for (int it = 0; it < kWaitLimit; ++it) {
     uint32_t ok;
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\nselp.b32 %0, 1, 0, p;\n}\n"
@@ -162,6 +163,7 @@ __device__ __forceinline__ void move_rows_up(const CacheView& c, const unsigned 
                                              const CUtensorMap* map, int unit, __nv_bfloat16* slab, int lane) {
   constexpr int TR = kTile / (2 * D), PR = D / 8, CH = D / 64;
   const int lo8 = (lo + 7) & ~7, plain_end = min(lo8, hi);
+#pragma unroll 1
   for (int x = lane; x < (plain_end - lo) * PR; x += 32) {
     const int row = lo + x / PR, pc = x % PR;
     if (row_ok(c, row - 1))
@@ -235,10 +237,13 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   const int empty_count = kCWarps + 1 + (k_in_ring ? 1 : 0);
   if (tid == 0) {
     *abort_flag = 0;
+#pragma unroll 1
     for (int s = 0; s < NS; ++s) { mbar_init(&bars[L::B_FULL + s], 1); mbar_init(&bars[L::B_EMPTY + s], empty_count); }
+#pragma unroll 1
     for (int x = 0; x < kMoveTiles; ++x) mbar_init(&bars[L::B_KM + x], 1);
     mbar_init(&bars[L::B_HOLE], 1);
     mbar_init(&bars[L::B_MOVED], 2);
+#pragma unroll 1
     for (int x = 0; x < 5; ++x) mbar_init(&bars[L::B_X + x], 1);
     mbar_fence_init();
   }
@@ -271,7 +276,9 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
     // ---------------------------------------------------------------- producer
     if (lane == 0) {
       int e = 0, slot = 0, ph = 0;
+#pragma unroll 1
       for (int unit = cl0; unit < a.units; unit += n_cl)
+#pragma unroll 1
         for (int x = 0; x < kt + vt; ++x, ++e) {
           if (e >= NS) mbar_wait(&bars[L::B_EMPTY + slot], ph ^ 1, abort_flag, c.status);
           const bool is_v = x >= kt;
@@ -285,6 +292,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         }
       if (k_in_ring && shift) {   // the K tiles behind the pair that leaves, once more
         mbar_wait(&bars[L::B_HOLE], 0, abort_flag, c.status);
+#pragma unroll 1
         for (int x = max(0, (*s_hole + 1) / TR - t0); x < vt; ++x, ++e) {
           if (e >= NS) mbar_wait(&bars[L::B_EMPTY + slot], ph ^ 1, abort_flag, c.status);
           mbar_expect_tx(&bars[L::B_FULL + slot], kTile);
@@ -298,10 +306,12 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   } else if (warp == kCWarps + 1) {
     // ---------------------------------------------------------------- V rows behind the pair that leaves; the step's V row
     int slot = 0, ph = 0, it = 0;
+#pragma unroll 1
     for (int unit = cl0; unit < a.units; unit += n_cl, ++it) {
       T* vslab = reinterpret_cast<T*>(c.v_slab) + (size_t)unit * c.cap * D;
       uint4 own = make_uint4(0u, 0u, 0u, 0u);  // the step's own row
       if (lane < PR) own = ld_global_16(reinterpret_cast<const T*>(a.v) + (size_t)unit * D + lane * 8);
+#pragma unroll 1
       for (int x = 0; x < kt; ++x) {          // (K tiles: the consumers')
         mbar_wait(&bars[L::B_FULL + slot], ph, abort_flag, c.status);
         arrive_one(&bars[L::B_EMPTY + slot], lane);
@@ -309,6 +319,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       }
       mbar_wait(&bars[L::B_HOLE], it & 1, abort_flag, c.status);
       const int hole = *s_hole;
+#pragma unroll 1
       for (int x = 0; x < vt; ++x) {
         mbar_wait(&bars[L::B_FULL + slot], ph, abort_flag, c.status);
         __syncwarp();
@@ -339,11 +350,13 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   } else if (warp == kCWarps + 2) {
     // ---------------------------------------------------------------- K rows behind the pair that leaves; the step's K row
     int e = 0, it = 0;                        // K-move tiles so far: tile e sits in buffer e % kMoveTiles
+#pragma unroll 1
     for (int unit = cl0; unit < a.units; unit += n_cl, ++it) {
       T* kslab = reinterpret_cast<T*>(c.k_slab) + (size_t)unit * c.cap * D;
       uint4 own = make_uint4(0u, 0u, 0u, 0u);
       if (lane < PR) own = ld_global_16(reinterpret_cast<const T*>(a.k) + (size_t)unit * D + lane * 8);
       if (k_in_ring)
+#pragma unroll 1
         for (int f = 0; f < kt + vt; ++f) {
           mbar_wait(&bars[L::B_FULL + f % NS], (f / NS) & 1, abort_flag, c.status);
           arrive_one(&bars[L::B_EMPTY + f % NS], lane);
@@ -371,6 +384,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           move_rows_up<D>(c, tile, g0, lo, min(g0 + TR, n_old), &maps.k_st, unit, kslab, lane);
         };
         if (a.single) {
+#pragma unroll 1
           for (int x = x0; x < vt; ++x) {
             const int f = a.keep_k ? x : kt + vt + x - x0;   // the tile's place in the order of the ring
             mbar_wait(&bars[L::B_FULL + f % NS], (f / NS) & 1, abort_flag, c.status);
@@ -378,6 +392,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
             if (k_in_ring && vt - x > NS) {                  // its place is needed once more: every arrival is this warp's
               moves_have_read<0>();
               if (lane == 0)
+#pragma unroll 1
                 for (int y = 0; y < empty_count; ++y) mbar_arrive(&bars[L::B_EMPTY + f % NS]);
             }
           }
@@ -385,6 +400,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           // kMoveTiles - 1 tiles are on their way while one is being stored (their rows lie above everything stored so far)
           int ahead = x0;
           for (; ahead < min(vt, x0 + kMoveTiles - 1); ++ahead) fetch(ahead, e + ahead - x0);
+#pragma unroll 1
           for (int x = x0; x < vt; ++x, ++e) {
             if (ahead < vt) {   // into the buffer of the tile before this one
               moves_have_read<0>();
@@ -425,6 +441,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
     // kv_ids and sum_weights of a cache's rows into buffer b; they arrive while the cache before it is worked on
     auto fetch_rows = [&](int unit, int b) {
       const size_t base = (size_t)unit * c.cap;
+#pragma unroll 1
       for (int jl = tid; jl < nr; jl += kConsumers) {
         const int j = r0 + jl;
         if (j < n_old) {
@@ -457,6 +474,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
     int slot = 0, ph = 0, it = 0;
+#pragma unroll 1
     for (int unit = cl0; unit < a.units; unit += n_cl, ++it) {
       const int smp = unit / c.Hkv, next = unit + n_cl;
       const size_t base = (size_t)unit * c.cap;
@@ -468,6 +486,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       asm volatile("cp.async.commit_group;" ::: "memory");
       // ---- logits (log2 domain)
       float mx0 = -INFINITY, mx1 = -INFINITY;              // running maxima of heads 2 tq, 2 tq + 1
+#pragma unroll 1
       for (int t = 0; t < kt; ++t) {
         mbar_wait(&bars[L::B_FULL + slot], ph, abort_flag, c.status);
         const int jl0 = t * TR + wr;                        // first row of this warp's 16, local
@@ -536,6 +555,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         float m2[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) m2[h] = -INFINITY;
+#pragma unroll 1
         for (int jl = tid; jl < nr; jl += kConsumers) {
           float e[G];
           ld_heads<G>(&s_p[jl * G], e);
@@ -563,6 +583,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         float t[G], ms[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) { t[h] = 0.f; ms[h] = mc[h] == -INFINITY ? 0.f : mc[h]; }   // (a piece of padding only)
+#pragma unroll 1
         for (int jl = tid; jl < nr; jl += kConsumers) {
           float e[G];
           ld_heads<G>(&s_p[jl * G], e);
@@ -641,9 +662,11 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       auto better = [&](uint32_t ok, int oj, int oi) {
         if (ok < best_key || (ok == best_key && oi > best_id)) { best_key = ok; best_j = oj; best_id = oi; }
       };
+#pragma unroll 1
       for (int jl = nr + tid; jl < vt * TR; jl += kConsumers)   // rows of the last tile past the cache carry no weight
 #pragma unroll
         for (int h = 0; h < G; ++h) s_pb[h * PBS + jl] = __float2bfloat16_rn(0.f);
+#pragma unroll 1
       for (int jl = tid; jl < nr; jl += kConsumers) {
         const int j = r0 + jl, id = s_id[jl];
         float e[G];
@@ -713,6 +736,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           if (c.fill) { if (hole < n_old) atomicAdd(&c.moved[unit & 15], 1ull); }
           else atomicAdd(&c.moved[unit & 15], (unsigned long long)(n1 - 1 - hole));
         }
+#pragma unroll 1
         for (int jl = tid; jl < nr; jl += kConsumers) {
           const int j = r0 + jl;
           // rows behind the hole move up by one; in an unordered cache only the step's own pair moves, into the hole's row
@@ -724,6 +748,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       }
       // ---- out^T = V^T p^T: warp = (16 elements of the head dimension, key group)
       float oacc[2][4] = {};
+#pragma unroll 1
       for (int x = 0; x < vt; ++x) {
         constexpr int NK = TR / 16 / KH;                    // steps of 16 keys per tile and warp
         mbar_wait(&bars[L::B_FULL + slot], ph, abort_flag, c.status);
@@ -812,6 +837,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
                         mapa(smem_u32(&bars[L::B_X + 2]), d >> ldc));
             }
         wait_cluster(&bars[L::B_X + 2], it & 1, abort_flag, c.status);
+#pragma unroll 1
         for (int x = tid; x < G * dc; x += kConsumers) {
           float part[kMaxCluster];
 #pragma unroll

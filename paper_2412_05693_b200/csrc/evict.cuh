@@ -100,6 +100,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
   // rules follow in a pass of their own.
   const int pad = sample_left_pad(c, smp);
   const bool plain = c.rule == 0 && pad == 0 && !e.recent && target < n_c;
+#pragma unroll 1
   for (int t = tid; t < 1024; t += NT) s.hist[t] = 0;
 #pragma unroll 4
   for (int j = tid; j < n_c; j += NT) {
@@ -126,6 +127,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
       if (j >= pool_body) b = 0x7f800000u;
       else {
         float m = s.score[j];
+#pragma unroll 1
         for (int x = max(0, j - pool_half); x < min(pool_body, j + pool_half + 1); ++x) m = fmaxf(m, s.score[x]);
         b = __float_as_uint(m);
       }
@@ -141,9 +143,11 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
   auto radix_kth_largest = [&](auto key_of, int need, uint32_t& out_key, int& out_need_eq, int& out_eq) {
     uint32_t prefix = 0, mask = 0;
     int count = 0;
+#pragma unroll 1
     for (int pass = 0; pass < 4; ++pass) {
       const int shift = 24 - 8 * pass;
       uint32_t* hist = s.hist + 256 * pass;
+#pragma unroll 2
       for (int j = tid; j < n_c; j += NT) {
         uint32_t b;
         if (key_of(j, b) && (b & mask) == prefix) atomicAdd(&hist[(b >> shift) & 255u], 1u);
@@ -179,6 +183,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     out_key = prefix;
     out_need_eq = need;
     out_eq = count;
+#pragma unroll 1
     for (int t = tid; t < 1024; t += NT) s.hist[t] = 0;   // (the next select's first barrier is behind other barriers)
   };
 
@@ -189,6 +194,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     const int chunk = (n_c + NT - 1) / NT;
     const int jb = min(tid * chunk, n_c), je = min(jb + chunk, n_c);
     int nfree = 0, nsrc = 0;
+#pragma unroll 1
     for (int j = jb; j < je; ++j) {
       const bool k = stays(j);
       nfree += (j < target && (j >= n_old || !k));
@@ -196,6 +202,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     }
     int fb, sb, nf;   // as many rows to fill as candidates to move
     block_exclusive_scan2<NT>(nfree, nsrc, s.wsum, fb, sb, &nf);
+#pragma unroll 1
     for (int j = jb; j < je; ++j) {
       const bool k = stays(j);
       if (j < target && (j >= n_old || !k)) s.dst[fb++] = j;
@@ -203,6 +210,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     }
     __syncthreads();
     if (c.moved != nullptr && tid == 0) atomicAdd(&c.moved[unit & 15], (unsigned long long)nf);
+#pragma unroll 1
     for (int k = tid; k < nf; k += NT) {
       const int j = s.src[k], r = s.dst[k];
       if (!row_ok(c, r)) continue;
@@ -213,6 +221,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     constexpr int PRF = D * (int)sizeof(T) / 16;
     T* kslab = reinterpret_cast<T*>(c.k_slab) + base * D;
     T* vslab = reinterpret_cast<T*>(c.v_slab) + base * D;
+#pragma unroll 1
     for (int x0 = 0; x0 < nf * PRF; x0 += 4 * NT) {
       uint4 kb[4], vb[4];
 #pragma unroll
@@ -245,6 +254,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
 
   int first_moved = n_old;   // rows before it keep their place and their contents
   if (target >= n_c) {
+#pragma unroll 1
     for (int r = tid; r < n_c; r += NT) s.src[r] = r;
     __syncthreads();
   } else if (FILL && e.recent) {  // Algorithm 3's rule on an unordered cache: the `target` highest positions stay
@@ -255,6 +265,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     fill_rows([&](int j) { return s.id[j] >= id_thr; });
     return;
   } else if (e.recent) {  // Algorithm 3's rule: the most recent pairs stay, whatever their weights
+#pragma unroll 1
     for (int r = tid; r < target; r += NT) s.src[r] = n_c - target + r;
     first_moved = 0;
     __syncthreads();
@@ -273,6 +284,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
       // rule 4 (Sec. 2 / Sec. 3.2, RoCo): the n_std candidates whose weights have the largest standard deviation,
       // sqrt(E[w^2] - E[w]^2) over the g * (curr_id + 1 - kv_ids) weights received, stay whatever their average
       // (ties: lower position first); they enter the ranking below as +inf, the others with their average
+#pragma unroll 1
       for (int j = tid; j < n_c; j += NT) {
         const float cnt = gf * (float)(e.curr_id + 1 - s.id[j]);
         const float sq = j < n_old ? c.sum_sq[base + j] : e.new_sq[(size_t)unit * e.I + (j - n_old)];
@@ -286,9 +298,11 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
       const int chunk = (n_c + NT - 1) / NT;
       const int jb = min(tid * chunk, n_c), je = min(jb + chunk, n_c);
       int eq = 0;
+#pragma unroll 1
       for (int j = jb; j < je; ++j) eq += (s.bits[j] == thr_s);
       int unused, eq_before;
       block_exclusive_scan2<NT>(0, eq, s.wsum, unused, eq_before);
+#pragma unroll 1
       for (int j = jb; j < je; ++j) {       // every thread rewrites its own chunk only
         const uint32_t b = s.bits[j];
         const bool prot = b > thr_s || (b == thr_s && eq_before < need_s);
@@ -296,6 +310,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
         s.bits[j] = prot ? 0x7f800000u : ave_bits(j);
       }
     } else if (!plain) {
+#pragma unroll 1
       for (int j = tid; j < n_c; j += NT) s.bits[j] = ave_bits(j);   // one division per candidate, not one per pass
     }
     if (!plain) __syncthreads();
@@ -322,6 +337,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     const int chunk = (n_c + NT - 1) / NT;
     const int jb = min(tid * chunk, n_c), je = min(jb + chunk, n_c);
     int gt = 0, eq = 0;
+#pragma unroll 1
     for (int j = jb; j < je; ++j) {
       const uint32_t b = s.bits[j];
       gt += (b > thr);
@@ -329,6 +345,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     }
     int gt_before, eq_before, first_out = n_old;
     block_exclusive_scan2<NT>(gt, eq, s.wsum, gt_before, eq_before);
+#pragma unroll 1
     for (int j = jb; j < je; ++j) {
       const uint32_t b = s.bits[j];
       const bool tie = b == thr, stays = b > thr || (tie && eq_before < need_eq);
@@ -347,6 +364,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
   if (c.moved != nullptr && tid == 0 && share.rank == 0 && first_moved < target)   // stable compaction: every row from there on moves
     atomicAdd(&c.moved[unit & 15], (unsigned long long)(target - first_moved));
 
+#pragma unroll 1
   for (int r = share.rank == 0 ? first_moved + tid : target; r < target; r += NT) {
     const int j = s.src[r];
     if (!row_ok(c, r) || j < 0 || j >= n_c) continue;
@@ -356,9 +374,11 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
   if (c.sum_sq != nullptr && share.rank == 0) {
     // rule 4: the sums of squares take the same places; they pass through shared memory (the ranking values are no
     // longer needed), so that every load has completed before the first store
+#pragma unroll 1
     for (int j = tid; j < n_c; j += NT)
       s.bits[j] = __float_as_uint(j < n_old ? c.sum_sq[base + j] : e.new_sq[(size_t)unit * e.I + (j - n_old)]);
     __syncthreads();
+#pragma unroll 1
     for (int r = first_moved + tid; r < target; r += NT)
       if (row_ok(c, r)) c.sum_sq[base + r] = __uint_as_float(s.bits[s.src[r]]);
   }
@@ -375,6 +395,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     const T* blk = (pc < PR ? reinterpret_cast<const T*>(e.blk_k) : reinterpret_cast<const T*>(e.blk_v)) +
                    ((size_t)smp * e.I * c.Hkv + kh) * D + (pc % PR) * (16 / sizeof(T));
     const int RS = NT / PC;                      // rows between two pieces of a thread
+#pragma unroll 1
     for (int r0 = first_moved; r0 < target; r0 += RC) {
       uint4 buf[W];
       bool mv[W];
@@ -400,6 +421,7 @@ __device__ inline void evict_body_impl(const CacheView& c, int unit, int smp, in
     constexpr int RC = NT * U / PR;              // rows per chunk
     T* kslab = reinterpret_cast<T*>(c.k_slab) + base * D;
     T* vslab = reinterpret_cast<T*>(c.v_slab) + base * D;
+#pragma unroll 1
     for (int r0 = first_moved; r0 < target; r0 += RC) {
       uint4 kb[U], vb[U];
       bool mv[U];
