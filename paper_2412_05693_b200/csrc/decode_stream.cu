@@ -183,7 +183,9 @@ __device__ __forceinline__ void moves_have_read() {
   __syncwarp();
 }
 
-template <int D, int G>
+// SHARED: clusters of 2, 4 or 8 CTAs own a cache together, and a CTA works on one cache only; instances of their own, so
+// that neither kind carries the other's code
+template <int D, int G, bool SHARED>
 __global__ void __launch_bounds__(kThreads, 1)
 decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constant__ StreamMaps maps) {
   using T = __nv_bfloat16;
@@ -201,7 +203,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   // The K move's tiles pass through two tiles of their own -- or, when the CTA has no further cache to prefetch, through
   // the ring behind the V tiles (all of its tiles are then free for them), or they are still in the ring.
   unsigned char* kst = ring + NS * kTile;
-  float* s_p = reinterpret_cast<float*>(kst + (a.single ? 0 : kMoveTiles * kTile));   // [RC][G] logits, then exp2(logit - maximum of the CTA)
+  float* s_p = reinterpret_cast<float*>(kst + (SHARED || a.single ? 0 : kMoveTiles * kTile));   // [RC][G] logits, then exp2(logit - maximum of the CTA)
   float* s_sw2 = s_p + (size_t)RC * G;                // [2][RC] sum_weights of this cache and of the next one
   int* s_id2 = reinterpret_cast<int*>(s_sw2 + 2 * RC);   // [2][RC] kv_ids, likewise
   T* s_pb = reinterpret_cast<T*>(s_id2 + 2 * RC);     // [G][RC + 8] the exponentials as bf16
@@ -219,9 +221,12 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   volatile int* s_hole = abort_flag + 1;
   float* s_enew = const_cast<float*>(reinterpret_cast<volatile float*>(s_hole + 1));   // [G] exponentials of the step's own pair
 
-  uint32_t rank, C;
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  uint32_t rank = 0, C = 1;
+  if (SHARED) {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  }
+  const bool single = SHARED || a.single;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_old = c.n_old, n1 = n_old + 1;
   const int tiles = (n1 + TR - 1) / TR;
@@ -233,7 +238,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   const int cl0 = blockIdx.x / C, n_cl = gridDim.x / C;
 
   // a ring tile is given back by the consumers, the V-move warp and, where its own tiles follow in the ring, the K-move warp
-  const bool k_in_ring = a.single && !a.keep_k;
+  const bool k_in_ring = single && !a.keep_k;
   const int empty_count = kCWarps + 1 + (k_in_ring ? 1 : 0);
   if (tid == 0) {
     *abort_flag = 0;
@@ -252,7 +257,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
     prefetch(&maps.k_ld); prefetch(&maps.v_ld); prefetch(&maps.k_st); prefetch(&maps.v_st);
   }
   __syncthreads();
-  if (C > 1) {   // the peers' barriers exist
+  if (SHARED) {   // the peers' barriers exist
     asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   }
@@ -342,7 +347,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       const bool mine = c.fill && a.evict_one ? (hole >= r0 && hole < r0 + nr) : (has_new && !(shift && r0 == n_old));
       if (hole != n_old && mine && lane < PR && row_ok(c, dst))
         st_global_16(vslab + (size_t)dst * D + lane * 8, own);
-      if (C > 1) first_row_up(0, vslab, hole, own);
+      if (SHARED) first_row_up(0, vslab, hole, own);
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[L::B_MOVED]);
     }
@@ -383,7 +388,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           }
           move_rows_up<D>(c, tile, g0, lo, min(g0 + TR, n_old), &maps.k_st, unit, kslab, lane);
         };
-        if (a.single) {
+        if (single) {
 #pragma unroll 1
           for (int x = x0; x < vt; ++x) {
             const int f = a.keep_k ? x : kt + vt + x - x0;   // the tile's place in the order of the ring
@@ -417,7 +422,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       const bool mine = c.fill && a.evict_one ? (hole >= r0 && hole < r0 + nr) : (has_new && !(shift && r0 == n_old));
       if (hole != n_old && mine && lane < PR && row_ok(c, dst))
         st_global_16(kslab + (size_t)dst * D + lane * 8, own);
-      if (C > 1) first_row_up(1, kslab, hole, own);
+      if (SHARED) first_row_up(1, kslab, hole, own);
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[L::B_MOVED]);
     }
@@ -539,14 +544,16 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       }
       asm volatile("cp.async.wait_group 1;" ::: "memory");  // this cache's ids and sums have arrived
       named_bar_sync(1, kConsumers);
-      auto all_warps = [&](const float* per_warp, float (&r)[G], auto op) {   // [warps][G] folded in a fixed order
-        ld_heads<G>(per_warp, r);
+      // [warps][G] folded into every thread: a lane takes one warp's value of one head (four heads at a time)
+      auto all_warps = [&](const float* per_warp, float (&r)[G], auto op) {
+        static_assert(kCWarps == 8, "");
 #pragma unroll
-        for (int w = 1; w < kCWarps; ++w) {
-          float t[G];
-          ld_heads<G>(per_warp + w * G, t);
+        for (int q = 0; q < G; q += 4) {
+          float t = per_warp[(lane & 7) * G + min(G - 1, q + (lane >> 3))];
 #pragma unroll
-          for (int h = 0; h < G; ++h) r[h] = op(r[h], t[h]);
+          for (int off = 4; off > 0; off >>= 1) t = op(t, __shfl_xor_sync(0xffffffffu, t, off));
+#pragma unroll
+          for (int h = q; h < min(G, q + 4); ++h) r[h] = __shfl_sync(0xffffffffu, t, 8 * (h - q));
         }
       };
       float mc[G];
@@ -601,58 +608,52 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
       }
       named_bar_sync(1, kConsumers);
       float f[G];                                           // weight of a pair = its exponential * f
-      if (C == 1) {
+      if (!SHARED) {
         all_warps(s_wsum, f, [](float x, float y) { return x + y; });
 #pragma unroll
         for (int h = 0; h < G; ++h) f[h] = q_real ? 1.f / f[h] : 0.f;
       } else {
         if (tid == 0) mbar_expect_tx(&bars[L::B_X], C * 2 * G * 4);
-        if (tid < (int)C) {                                 // this CTA's statistics to every peer
-          const uint32_t dst = mapa(smem_u32(s_xstat + rank * 2 * G), tid), bar = mapa(smem_u32(&bars[L::B_X]), tid);
+        if (warp == 0) {                                    // this CTA's statistics to every peer
           float t[G];
           all_warps(s_wsum, t, [](float x, float y) { return x + y; });
-          if constexpr (G % 4 == 0) {
+          if (lane < (int)C) {
+            const uint32_t dst = mapa(smem_u32(s_xstat + rank * 2 * G), lane), bar = mapa(smem_u32(&bars[L::B_X]), lane);
+            if constexpr (G % 4 == 0) {
 #pragma unroll
-            for (int h = 0; h < G; h += 4) {
-              st_peer4(dst + 4 * h, __float_as_uint(mc[h]), __float_as_uint(mc[h + 1]), __float_as_uint(mc[h + 2]),
-                       __float_as_uint(mc[h + 3]), bar);
-              st_peer4(dst + 4 * (G + h), __float_as_uint(t[h]), __float_as_uint(t[h + 1]), __float_as_uint(t[h + 2]),
-                       __float_as_uint(t[h + 3]), bar);
-            }
-          } else {
+              for (int h = 0; h < G; h += 4) {
+                st_peer4(dst + 4 * h, __float_as_uint(mc[h]), __float_as_uint(mc[h + 1]), __float_as_uint(mc[h + 2]),
+                         __float_as_uint(mc[h + 3]), bar);
+                st_peer4(dst + 4 * (G + h), __float_as_uint(t[h]), __float_as_uint(t[h + 1]), __float_as_uint(t[h + 2]),
+                         __float_as_uint(t[h + 3]), bar);
+              }
+            } else {
 #pragma unroll
-            for (int h = 0; h < G; ++h) {
-              st_peer(dst + 4 * h, mc[h], bar);
-              st_peer(dst + 4 * (G + h), t[h], bar);
+              for (int h = 0; h < G; ++h) {
+                st_peer(dst + 4 * h, mc[h], bar);
+                st_peer(dst + 4 * (G + h), t[h], bar);
+              }
             }
           }
         }
         wait_cluster(&bars[L::B_X], it & 1, abort_flag, c.status);
-        // lane p holds what CTA p said; the sum runs over the lanes in a fixed order (with a loop over the peers, head by
-        // head, and a releasing barrier at the end a step on 8 caches of 1024 pairs took 8.2 us instead of 6.6)
-        float m[G], t[G];
-        {
-          const float* from = s_xstat + (lane & (kMaxCluster - 1)) * 2 * G;
-          const bool there = (lane & (kMaxCluster - 1)) < (int)C;
+        // a lane holds what one CTA said about one head (four heads at a time); the sum runs over the lanes in a fixed order
 #pragma unroll
-          for (int h = 0; h < G; ++h) { m[h] = there ? from[h] : -INFINITY; t[h] = there ? from[G + h] : 0.f; }
+        for (int q = 0; q < G; q += 4) {
+          const int p = lane & (kMaxCluster - 1), h = min(G - 1, q + (lane >> 3));
+          const bool there = p < (int)C;
+          const float m = there ? s_xstat[p * 2 * G + h] : -INFINITY, own = s_xstat[rank * 2 * G + h];
+          float t = there ? s_xstat[p * 2 * G + G + h] : 0.f, top = m;
+#pragma unroll
+          for (int off = kMaxCluster / 2; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
+          t = m == -INFINITY ? 0.f : t * ex2(m - top);
+#pragma unroll
+          for (int off = kMaxCluster / 2; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+          // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
+          const float fh = (q_real && (own != -INFINITY || top == -INFINITY)) ? ex2(own - top) / t : 0.f;
+#pragma unroll
+          for (int y = q; y < min(G, q + 4); ++y) f[y] = __shfl_sync(0xffffffffu, fh, 8 * (y - q));
         }
-        float top[G];
-#pragma unroll
-        for (int h = 0; h < G; ++h) top[h] = m[h];
-#pragma unroll
-        for (int off = kMaxCluster / 2; off > 0; off >>= 1)
-#pragma unroll
-          for (int h = 0; h < G; ++h) top[h] = fmaxf(top[h], __shfl_xor_sync(0xffffffffu, top[h], off));
-#pragma unroll
-        for (int h = 0; h < G; ++h) t[h] = m[h] == -INFINITY ? 0.f : t[h] * ex2(m[h] - top[h]);
-#pragma unroll
-        for (int off = kMaxCluster / 2; off > 0; off >>= 1)
-#pragma unroll
-          for (int h = 0; h < G; ++h) t[h] += __shfl_xor_sync(0xffffffffu, t[h], off);
-#pragma unroll
-        for (int h = 0; h < G; ++h)   // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
-          f[h] = (q_real && (mc[h] != -INFINITY || top[h] == -INFINITY)) ? ex2(mc[h] - top[h]) / t[h] : 0.f;
       }
       // ---- sum_weights += attn_weights (heads added in a fixed order), candidate for eviction, bf16 exponentials
       // (the pair with the smallest ranking value leaves; ties: the higher position -- kv_ids, not rows: the rows of an
@@ -713,8 +714,8 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         warp_best();
         if (lane == 0) s_best[warp] = make_int4((int)best_key, best_j, best_id, 0);
         named_bar_sync(1, kConsumers);
-        if (C == 1 || warp == 0) read_best(s_best, kCWarps);
-        if (C > 1) {
+        if (!SHARED || warp == 0) read_best(s_best, kCWarps);
+        if (SHARED) {
           if (tid == 0) mbar_expect_tx(&bars[L::B_X + 1], C * 16);
           if (tid < (int)C)
             st_peer4(mapa(smem_u32(s_xbest + rank), tid), best_key, (uint32_t)best_j, (uint32_t)best_id, 0u,
@@ -808,7 +809,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
         }
       }
       T* op = reinterpret_cast<T*>(a.out) + (size_t)unit * G * D;
-      if (C == 1) {
+      if (!SHARED) {
         if (kg == 0)
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf)
@@ -854,7 +855,7 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
   // No CTA of a cluster leaves while a peer may still write into its shared memory.  It has waited for all that is sent
   // to it (B_X, B_PREV), so the barrier need not order memory (a releasing arrival waits for the global
   // stores); it is there for a CTA whose waits gave up.
-  if (C > 1) {
+  if (SHARED) {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
@@ -927,10 +928,17 @@ cudaError_t launch_stream(const CacheView& c, StreamArgs a, cudaStream_t st, boo
       !encode_slab_rows_map(&m.v_st, c.v_slab, D, c.n_old - 1, c.cap, a.units, 8))
     return cudaSuccess;
   *taken = true;
-  static SmemConfigured configured;
-  if (cudaError_t err = configured.ensure(decode_stream_kernel<D, G>, p.smem); err != cudaSuccess) return err;
   ProfileScope prof(kDecode, st);
-  const cudaError_t err = launch_dependent_cluster(decode_stream_kernel<D, G>, dim3(p.grid), dim3(kThreads), p.smem, p.C, st, c, a, m);
+  cudaError_t err;
+  if (p.C > 1) {
+    static SmemConfigured configured;
+    if ((err = configured.ensure(decode_stream_kernel<D, G, true>, p.smem)) != cudaSuccess) return err;
+    err = launch_dependent_cluster(decode_stream_kernel<D, G, true>, dim3(p.grid), dim3(kThreads), p.smem, p.C, st, c, a, m);
+  } else {
+    static SmemConfigured configured;
+    if ((err = configured.ensure(decode_stream_kernel<D, G, false>, p.smem)) != cudaSuccess) return err;
+    err = launch_dependent(decode_stream_kernel<D, G, false>, dim3(p.grid), dim3(kThreads), p.smem, st, c, a, m);
+  }
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
