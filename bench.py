@@ -336,15 +336,13 @@ def forward_kernel(wl):
 
 
 def decode_kernel(wl):
-    """The kernel of an evicting decode step on caches of K pairs that do not stay in L2 (or do, where there is no more than
-    one per SM), by the library's rule (stream_is_faster in csrc/decode_mma.cu); None where neither table row applies."""
-    caches, kib, mib = wl.b * wl.Hkv, (wl.K + 1) * wl.d * 4 / 1024, wl.b * wl.Hkv * wl.L * (wl.K + 1) * (4 * wl.d + 8) / 2 ** 20
+    """The kernel of an evicting decode step on caches of K pairs, by the library's rule (stream_is_faster in
+    csrc/decode_mma.cu, on 148 SMs)."""
+    caches, kib = wl.b * wl.Hkv, (wl.K + 1) * wl.d * 4 // 1024
     if wl.dtype != "bf16":
         return None
-    if mib <= 104:
-        return "decode_mma_kernel" if wl.d == 128 and caches > 64 else None
-    return "decode_stream_kernel" if caches <= 148 or kib >= (256 if caches <= 296 else 172 if caches <= 592 else 150) \
-        else "decode_mma_kernel"
+    least = 0 if caches <= 296 else 96 if caches <= 444 else 172 if caches <= 592 else 112
+    return "decode_stream_kernel" if kib >= least else "decode_mma_kernel"
 
 
 def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch, padded=False):

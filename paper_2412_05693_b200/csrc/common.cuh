@@ -29,7 +29,6 @@ struct CacheView {
   int32_t window, pool;     // rule 3: queries observed / recent pairs kept; width of the max-pooling (odd)
   int32_t std_permille;     // rule 4: share of the kept pairs chosen by standard deviation, in 1/1000
   int32_t padded;           // 1: some sample of the handle is left-padded (left_pad is null for calls that meet no padding)
-  int32_t in_l2;            // 1: all of the handle's caches together stay in the L2 cache
   int32_t layer_units;      // caches of the handle in one layer: what a kernel is chosen by where the choice changes the order
                             // of a sum, so that results do not depend on how a batch is cut into sample ranges
 };

@@ -703,39 +703,31 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 }
 
 // Which kernel takes a step: the stream, or this file's kernels.  By the handle's caches of a layer and not the call's, so
-// that sample ranges of a batch take one kernel.  Measured, us per step (stream / this file; d = 128, g = 4, one pair leaves
-// by its average and the rows behind it move up, unless said otherwise):
-//   Caches out of HBM (several layers or ranges in turn): 8 caches of 500 pairs 8.1 / 10.2, 128 caches of 500 11.0 / 12.1,
-//   of 1024 18.4 / 25.3, 192 of 400 15.6 / 16.8, 320 of 400 21.0 / 24.7, 512 of 330 25.2 / 23.5, of 500 29.7 / 31.3, 800 of
-//   320 34.4 / 38.1, 1024 of 1024 95 / 112; d = 64 512 caches of 700 25.6 / 27.7; ranking by raw sums 512 of 330 27.1 /
-//   31.7.  The stream pays once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's
-//   bytes: 150 KB, 172 KB where an SM has up to four caches (and the last round of them is a large part; not under the
-//   other rules or with padding, where this file's instance is the slower one), or 256 KB while this file's kernel holds
-//   every cache of the call at once (two CTAs per SM).
-//   Caches in L2 (a handle of few layers):
-//   - shared by clusters: 64 caches of 512 pairs 9.8 / 9.2 (K in registers, which ends at 640 pairs), of 1024 14.4 / 16.0;
-//   - at most one per SM: 128 caches of 700 pairs 13.1 / 12.2, of 1024 17.4 / 16.2, but where no row moves 1024 11.1 / 15.0
-//     and by raw sums 18.3 / 21.9; by the current query alone, which moves most rows, 28.2 / 27.4; d = 64, g = 1 300 pairs
-//     7.0 / 6.3, g = 4 1024 pairs 11.4 / 12.4;
-//   - more: 192 of 600 18.6 / 15.7, 320 of 330 18.6 / 16.1, 512 of 330 25.0 / 18.0; unordered 320 of 330 17.3 / 15.8, of 500
-//     20.0 / 21.7; d = 64 192 of 1024 18.3 / 15.7, unordered 16.5 / 15.2.
+// that sample ranges of a batch take one kernel.  The stream is the faster one while an SM has at most two caches, and beyond
+// that once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes.  Measured, us
+// per step, launched one by one (stream / this file; d = 128, g = 4, one pair leaves by its average and the rows behind it
+// move up, unless said otherwise):
+//   up to two per SM: 64 caches of 512 pairs 8.6 / 9.9, 128 of 330 8.1 / 8.5, of 700 10.4 / 14.2, of 1024 13.8 / 18.4, 192 of 60
+//   7.7 / 7.7, of 200 9.6 / 10.4, of 600 15.7 / 17.9, unordered 14.1 / 15.8, by raw sums 499 15.3 / 19.6, by the current query 499
+//   20.2 / 23.3; d = 64 128 of 500 7.5 / 9.8, 192 of 120 7.8 / 7.5, of 1024 16.3 / 17.3; g = 8 128 of 700 11.1 / 15.6;
+//   up to three, from 96 KB: 320 of 120 10.1 / 9.9, of 200 13.0 / 14.0, of 500 19.0 / 24.1, 384 of 200 13.3 / 13.8, unordered 12.2 / 12.2,
+//   of 120 10.5 / 9.9; d = 64 384 of 330 13.0 / 12.8;
+//   up to four, from 172 KB (the last round of caches is a large part), or 150 where the pairs that leave are not found by
+//   averages alone: 512 of 330 21.3 / 19.9, of 400 24.7 / 26.6, unordered of 330 20.2 / 18.3, by raw sums 330 22.6 / 25.2, by the
+//   current query 330 25.8 / 27.9, 200 18.3 / 17.3; d = 64 512 of 700 24.0 / 25.7; g = 1 512 of 400 23.3 / 24.4; one step in four
+//   evicting 330 22.4 / 19.8;
+//   more, from 112 KB: 800 of 200 24.5 / 24.2, of 260 30.1 / 34.5, of 400 35.0 / 48.0, 1024 of 150 25.6 / 22.2.
 //   A cut by more than one value per pair follows the stream as a launch of its own: under rule 4 8 caches of 300 pairs
-//   16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 96 of 700 26.1 / 24.7, 512 of 700 69 / 64; unordered with a recent window 512
-//   of 700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
+//   16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 192 of 499 23.6 / 22.9, 512 of 700 69 / 64; unordered with a recent window 512 of
+//   700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
 static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
-  const int sms = sm_count(), n1 = c.n_old + 1, caches = c.layer_units;
-  const size_t bytes = (size_t)n1 * d * 4;
-  const bool plain = c.rule == 0 && !c.padded, moves = one && !c.fill;
-  if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) &&
-      (caches > kMostSharedCaches || (c.rule == 4 && bytes < (size_t)200 << 10))) return false;
-  if (caches <= kMostSharedCaches) return d == 64 || n1 > kBatchTiles * 128 || !c.in_l2 || caches <= sms / 4;
-  if (caches <= sms) {
-    if (!c.in_l2) return true;
-    if (d == 64) return n1 > 512 || !plain || !moves;
-    return n1 > kBatchTiles * 128 && !(moves && (plain || c.rule == 2));
-  }
-  if (c.in_l2 && plain && (moves || d == 64)) return false;
-  return bytes >= (size_t)(caches <= 2 * sms ? 256 : plain && caches <= 4 * sms ? 172 : 150) << 10;
+  const int sms = sm_count(), caches = c.layer_units;
+  const size_t kb = (size_t)(c.n_old + 1) * d * 4 >> 10;
+  if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) && (caches > kMostSharedCaches || (c.rule == 4 && kb < 200))) return false;
+  if (caches <= 2 * sms) return true;
+  if (caches <= 3 * sms) return kb >= 96;
+  if (caches <= 4 * sms) return kb >= (c.rule == 0 && !c.padded ? 172 : 150);
+  return kb >= 112;
 }
 
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,

@@ -245,6 +245,21 @@ def test_decode_with_more_caches_than_two_ctas_per_sm(g):
     assert st["evictions"] >= len(units) * 10
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
+    (24, 8, 4, 128, 60, {}),                              # 192 caches: an SM has up to two, the stream whatever their length
+    (24, 8, 2, 64, 33, dict(rule="sum_recent")),
+    (37, 8, 1, 128, 128, dict(compaction="fill")),        # 296: the most that two per SM make
+    (40, 8, 2, 128, 200, {}),                             # 320: from 96 KB a cache on
+    (40, 8, 2, 128, 190, {}),                             # ... and below, on the other kernel
+    (64, 8, 1, 128, 300, dict(rule="current_query")),     # 512: from 150 KB on under this rule, not under the average
+    (64, 8, 1, 128, 300, {}),
+])
+def test_decode_kernel_by_number_and_length_of_caches(b, Hkv, g, d, K, kw):
+    wl = tiny("by_grid", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 21, B=K, K=K, steps=4, dtype="bf16", d=d)
+    st = run_lockstep(wl, [(0, 0), (b // 2, 3), (b - 1, Hkv - 1)], check_rows_every=1, **kw)
+    assert st["evictions"] >= 3 * 4
+
+
 @pytest.mark.parametrize("K,g", [(511, 4), (512, 1), (600, 4), (639, 2), (640, 4)])
 def test_decode_with_one_cache_per_sm(K, g):
     # few caches of at most 640 pairs: the decode kernel's instance that keeps K in registers and stages V by TMA
