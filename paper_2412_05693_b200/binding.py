@@ -210,8 +210,9 @@ def profile_read():
     return out
 
 
-# What a call passes on every time is kept cheap: small decode steps take 10 us on the GPU, and wrapping every argument
-# in a ctypes object and asking torch for a Stream object took 7 of the 13.7 us a step took on the host.
+# What a call passes on every time is kept cheap: wrapping every argument in a ctypes object and asking torch for a Stream
+# object took 7 of the 13.7 us that a step took on the host.  Blocks and steps of plain tensors on the current stream go
+# through csrc/fastcall.cpp; the code here is the general way.
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
@@ -251,11 +252,17 @@ class BatchMaxCache:
                                          self.workspace.numel(), _stream(stream), C.byref(h)), "bm_cache_create")
         self.h = h
         self._prefill, self._decode = lib().bm_prefill_block, lib().bm_decode_step
+        from . import _fastcall            # (needs torch's libraries, loaded by now)
+        self._fast = _fastcall
+        bf16 = self.tdtype == torch.bfloat16
+        self._fast_prefill = (C.cast(self._prefill, _vp).value, h.value, bf16)   # address, handle, element type
+        self._fast_decode = (C.cast(self._decode, _vp).value, h.value, bf16)
 
     def close(self):
         if getattr(self, "h", None) is not None and self.h:
             lib().bm_cache_destroy(self.h)
             self.h = None
+            self._fast_prefill = self._fast_decode = ()   # (no handle: the native step declines)
 
     def __del__(self):
         try:
@@ -272,10 +279,16 @@ class BatchMaxCache:
     def prefill_block(self, q, k, v, pos0: int, out=None, evict_to: int = -1, layer: int = 0, sample0: int = 0,
                       stream=None):
         """q (ns, I, Hq, d), k/v (ns, I, Hkv, d) contiguous device tensors; returns out (ns, I, Hq, d)."""
-        shape = q.shape
-        assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == self.tdtype
         if out is None:
             out = self.torch.empty_like(q)
+        if stream is None:
+            rc = self._fast.prefill(*self._fast_prefill, q, k, v, out, layer, sample0, evict_to, pos0)
+            if rc is not None:
+                if rc:
+                    _check(rc, "bm_prefill_block")
+                return out
+        shape = q.shape
+        assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == self.tdtype
         self._check_out(out, q)
         rc = self._prefill(self.h, layer, sample0, shape[0], q.data_ptr(), k.data_ptr(), v.data_ptr(), shape[1], pos0,
                            out.data_ptr(), evict_to, _stream(stream))
@@ -298,9 +311,15 @@ class BatchMaxCache:
 
     def decode_step(self, q, k, v, out=None, evict_to: int = -1, layer: int = 0, sample0: int = 0, stream=None):
         """q (ns, Hq, d), k/v (ns, Hkv, d); returns out (ns, Hq, d)."""
-        assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == self.tdtype
         if out is None:
             out = self.torch.empty_like(q)
+        if stream is None:
+            rc = self._fast.decode(*self._fast_decode, q, k, v, out, layer, sample0, evict_to)
+            if rc is not None:
+                if rc:
+                    _check(rc, "bm_decode_step")
+                return out
+        assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and q.dtype == self.tdtype
         self._check_out(out, q)
         rc = self._decode(self.h, layer, sample0, q.shape[0], q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
                           evict_to, _stream(stream))

@@ -1,18 +1,21 @@
-"""Builds libbatchmax.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds libbatchmax.so (the C-ABI library) in-tree with nvcc for sm_100a, and _fastcall.so (the binding's native step).
 
     python -m paper_2412_05693_b200.build [--force] [--verbose] [--debug]
 """
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libbatchmax.so")
 DEBUG_LIB_PATH = os.path.join(PKG_DIR, "libbatchmax_debug.so")   # the checked build: -DBM_DEBUG
+FASTCALL_SRC, FASTCALL_PATH = os.path.join(CSRC, "fastcall.cpp"), os.path.join(PKG_DIR, "_fastcall.so")
 HEADER = os.path.join(os.path.dirname(PKG_DIR), "include", "batchmax.h")
 
 NVCC_FLAGS = [
@@ -33,10 +36,24 @@ def _stale(lib_path: str = LIB_PATH) -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_fastcall(force: bool = False) -> str:
+    """Compile the binding's native step against torch's headers; returns its path."""
+    if not force and os.path.exists(FASTCALL_PATH) and os.path.getmtime(FASTCALL_PATH) >= os.path.getmtime(FASTCALL_SRC):
+        return FASTCALL_PATH
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *("-I" + d for d in inc), "-o", FASTCALL_PATH, FASTCALL_SRC,
+                    "-L" + os.path.join(torch_dir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"], check=True)
+    return FASTCALL_PATH
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     """Compile every .cu under csrc/ into one shared library; returns its path.  debug: the checked build
     (row-index checks in the kernels, guards behind the slabs), libbatchmax_debug.so."""
     lib_path = DEBUG_LIB_PATH if debug else LIB_PATH
+    build_fastcall(force)
     if not force and not _stale(lib_path):
         return lib_path
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

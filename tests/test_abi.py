@@ -146,3 +146,36 @@ def test_benchmark_reaches_the_oracle_only_in_its_cpu_legs():
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
     src = open(os.path.join(ROOT, "bench.py")).read()
     assert src.count("from oracle import") == 1 and "tests.lockstep" not in src
+
+
+def test_native_step_declines_what_it_does_not_handle_and_checks_like_the_general_way():
+    import torch
+    from paper_2412_05693_b200.build import build_fastcall
+    build_fastcall()
+    from paper_2412_05693_b200 import _fastcall
+    q, kv = torch.zeros(2, 4, 64), torch.zeros(2, 2, 64)
+    calls = []
+
+    @C.CFUNCTYPE(C.c_int32, C.c_void_p, C.c_int32, C.c_int32, C.c_int32, *[C.c_void_p] * 4, C.c_int32, C.c_void_p)
+    def fake(h, layer, sample0, ns, pq, pk, pv, po, evict_to, stream):
+        calls.append((h, layer, sample0, ns, pq, pk, pv, po, evict_to))
+        return 3
+
+    addr = C.cast(fake, C.c_void_p).value
+
+    def step(q=q, k=kv, v=kv, out=None, layer=1, sample0=2, evict_to=-1, bf16=False):
+        return _fastcall.decode(addr, 77, bf16, q, k, v, torch.empty_like(q) if out is None else out, layer, sample0, evict_to)
+
+    assert _fastcall.decode() is None                                    # a closed handle
+    subclass = type("Sub", (torch.Tensor,), {})
+    assert step(q=q.as_subclass(subclass)) is None and step(layer=True) is None and step(layer=1.0) is None
+    assert step(evict_to=1 << 40) is None and step(k=None) is None and step(k=[1]) is None
+    for bad in (dict(q=q.bfloat16()), dict(bf16=True), dict(k=kv.transpose(1, 2)), dict(out=torch.zeros(2, 4, 32)),
+                dict(out=torch.zeros(2, 64, 4).transpose(1, 2)), dict(out=q.bfloat16())):
+        with pytest.raises(AssertionError):
+            step(**bad)
+    assert calls == []
+    if torch.cuda.is_available():                                        # (asks for the current stream)
+        out = torch.empty_like(q)
+        assert step(out=out, evict_to=9) == 3
+        assert calls == [(77, 1, 2, 2, q.data_ptr(), kv.data_ptr(), kv.data_ptr(), out.data_ptr(), 9)]
