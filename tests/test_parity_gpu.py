@@ -509,6 +509,23 @@ def test_f32_kernels_by_grid_size(b, Hkv, g, d, B, K):
     run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1)
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
+    (2, 4, 1, 64, 31, {}),                                # 32 pairs with the step's own: 8 rows for each CTA of four
+    (1, 3, 8, 128, 203, {}),                              # shared by eight, uneven pieces
+    (3, 2, 2, 64, 191, dict(compaction="fill")),          # a cut that follows as a launch of its own
+    (5, 4, 4, 128, 150, dict(rule="sum_recent")),
+    (5, 4, 4, 64, 97, dict(rule="current_query")),
+    (2, 4, 4, 128, 130, dict(rule="average_std")),
+    (4, 4, 4, 128, 790, {}),                              # too long for four, shared by eight
+    (20, 4, 1, 64, 40, {}),                               # 80 caches: not shared
+])
+def test_f32_decode_with_caches_shared_by_clusters(b, Hkv, g, d, K, kw):
+    wl = tiny("f32_shared", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 40, B=K, K=K, steps=6, dtype="f32", d=d)
+    run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1, **kw)
+    if not kw:
+        assert_same_run(run_free(wl), run_free(wl, micro=1))
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", [
     (4, 4, 4, 128, 256, 1280),   # the whole batch would share a key tile among 2 CTAs, a single sample among 8
     (4, 4, 4, 128, 256, 512),    # ... 4 and 8
