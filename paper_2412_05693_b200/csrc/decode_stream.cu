@@ -21,7 +21,10 @@
 // exchanges by plain remote stores and releasing arrivals, which wait for the sender's global stores; 8.2 with a loop
 // over the peers' statistics and a releasing barrier at the end), 128
 // caches 16.8 / 19.1, 1024 caches 95 / 112 (5.9 against 5.0 TB/s of algorithmic bytes), 3072 caches 267 / 304 (6.3 TB/s),
-// 1024 caches without groups 88 / 104 (6.3 TB/s).  Not kept: tiles of 32 KB with two tiles' fragments in flight per warp
+// 1024 caches without groups 88 / 104 (6.3 TB/s).  Since then per-row loops stay rolled, clusters have instances of their own and
+// statistics are folded across lanes: 88 KB of code became 44 and 54, where an SM's instruction cache holds 32, and a
+// replayed step on 8 caches went from 6.2 to 5.5 us, on 32 layers of 32 caches of 512 pairs from 8.0 to 7.1, on 1024 caches from 92
+// to 91.  Not kept: tiles of 32 KB with two tiles' fragments in flight per warp
 // (spills; 111 against 94 us at 1024 caches), the per-row loops four rows at a time (+2 to 8 %), sums and ids written by
 // a warp of their own (+5 to 15 %: one warp's stores are on the chain to the next cache).
 #include <algorithm>
