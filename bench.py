@@ -341,7 +341,7 @@ def decode_kernel(wl):
     caches, kib = wl.b * wl.Hkv, (wl.K + 1) * wl.d * 4 // 1024
     if wl.dtype != "bf16":
         return None
-    least = 0 if caches <= 296 else 96 if caches <= 444 else 172 if caches <= 592 else 112
+    least = 0 if caches <= 148 else (80 if wl.d == 64 else 48) if caches <= 296 else 96 if caches <= 444 else 172 if caches <= 592 else 112
     return "decode_stream_kernel" if kib >= least else "decode_mma_kernel"
 
 

@@ -703,12 +703,13 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 }
 
 // Which kernel takes a step: the stream, or this file's kernels.  By the handle's caches of a layer and not the call's, so
-// that sample ranges of a batch take one kernel.  The stream is the faster one while an SM has at most two caches, and beyond
+// that sample ranges of a batch take one kernel.  The stream is the faster one while an SM has at most one cache, and beyond
 // that once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes.  Measured, us
 // per step, launched one by one (stream / this file; d = 128, g = 4, one pair leaves by its average and the rows behind it
 // move up, unless said otherwise):
-//   up to two per SM: 64 caches of 512 pairs 8.6 / 9.9, 128 of 330 8.1 / 8.5, of 700 10.4 / 14.2, of 1024 13.8 / 18.4, 192 of 60
-//   7.7 / 7.7, of 200 9.6 / 10.4, of 600 15.7 / 17.9, unordered 14.1 / 15.8, by raw sums 499 15.3 / 19.6, by the current query 499
+//   up to one per SM: 64 caches of 512 pairs 8.6 / 9.9, 128 of 330 8.1 / 8.5, of 700 10.4 / 14.2, of 1024 13.8 / 18.4;
+//   up to two, from 48 KB, at d = 64 (twice the rows) from 80 (below that a pass over 288 caches of 284 pairs was 3 % slower): 192
+//   of 60 7.7 / 7.7, of 120 7.8 / 8.7, of 200 9.6 / 10.4, of 600 15.7 / 17.9, unordered 14.1 / 15.8, by raw sums 499 15.3 / 19.6, by the current query 499
 //   20.2 / 23.3; d = 64 128 of 500 7.5 / 9.8, 192 of 120 7.8 / 7.5, of 1024 16.3 / 17.3; g = 8 128 of 700 11.1 / 15.6;
 //   up to three, from 96 KB: 320 of 120 10.1 / 9.9, of 200 13.0 / 14.0, of 500 19.0 / 24.1, 384 of 200 13.3 / 13.8, unordered 12.2 / 12.2,
 //   of 120 10.5 / 9.9; d = 64 384 of 330 13.0 / 12.8;
@@ -724,7 +725,8 @@ static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
   const int sms = sm_count(), caches = c.layer_units;
   const size_t kb = (size_t)(c.n_old + 1) * d * 4 >> 10;
   if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) && (caches > kMostSharedCaches || (c.rule == 4 && kb < 200))) return false;
-  if (caches <= 2 * sms) return true;
+  if (caches <= sms) return true;
+  if (caches <= 2 * sms) return kb >= (d == 64 ? 80 : 48);
   if (caches <= 3 * sms) return kb >= 96;
   if (caches <= 4 * sms) return kb >= (c.rule == 0 && !c.padded ? 172 : 150);
   return kb >= 112;

@@ -246,8 +246,8 @@ def test_decode_with_more_caches_than_two_ctas_per_sm(g):
 
 
 @pytest.mark.parametrize("b,Hkv,g,d,K,kw", [
-    (24, 8, 4, 128, 60, {}),                              # 192 caches: an SM has up to two, the stream whatever their length
-    (24, 8, 2, 64, 33, dict(rule="sum_recent")),
+    (24, 8, 4, 128, 100, {}),                             # 192 caches: up to two per SM, the stream from 48 KB a cache on
+    (24, 8, 2, 64, 33, dict(rule="sum_recent")),          # ... and below, on the other kernel
     (37, 8, 1, 128, 128, dict(compaction="fill")),        # 296: the most that two per SM make
     (40, 8, 2, 128, 200, {}),                             # 320: from 96 KB a cache on
     (40, 8, 2, 128, 190, {}),                             # ... and below, on the other kernel
