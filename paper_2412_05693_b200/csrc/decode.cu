@@ -372,6 +372,10 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
   return r;
 }
+// 2^n, exactly, for a whole n <= 0, or -inf; NaN stays NaN
+__device__ __forceinline__ float pow2_whole(float n) {
+  return n >= -126.f ? __int_as_float(((int)n + 127) << 23) : n < 0.f ? 0.f : n;
+}
 __device__ __forceinline__ void st_peer(const void* p, uint32_t rank, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(p, rank)), "f"(v) : "memory");
 }
@@ -437,25 +441,28 @@ __global__ void __launch_bounds__(kShThreads) decode_shared_kernel(CacheView c, 
   asm volatile("cp.async.wait_group 1;" ::: "memory");
   __syncthreads();
 
-  // ---- logits (log2 domain): four threads per row, each every fourth 16-byte piece
-  const float sc2 = a.scale * kLog2e;
+  // ---- logits, unscaled: four threads per row, each every fourth 16-byte piece
 #pragma unroll 1
   for (int j0 = 0; j0 < nr; j0 += kShThreads / 4) {
     const int jl = j0 + (tid >> 2), sub = tid & 3;
     const float* kr = sK + min(jl, nr - 1) * LD;
-    float dot[G];
+    // (four sums per head: one chain of 32 products made the weights' error against 64 bits a quarter larger)
+    float4 acc[G];
 #pragma unroll
-    for (int h = 0; h < G; ++h) dot[h] = 0.f;
+    for (int h = 0; h < G; ++h) acc[h] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int pc = sub; pc < D4; pc += 4) {
       const float4 k4 = *reinterpret_cast<const float4*>(kr + 4 * pc);
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         const float4 q4 = *reinterpret_cast<const float4*>(sQ + h * D + 4 * pc);
-        dot[h] = fmaf(q4.x, k4.x, dot[h]); dot[h] = fmaf(q4.y, k4.y, dot[h]);
-        dot[h] = fmaf(q4.z, k4.z, dot[h]); dot[h] = fmaf(q4.w, k4.w, dot[h]);
+        acc[h].x = fmaf(q4.x, k4.x, acc[h].x); acc[h].y = fmaf(q4.y, k4.y, acc[h].y);
+        acc[h].z = fmaf(q4.z, k4.z, acc[h].z); acc[h].w = fmaf(q4.w, k4.w, acc[h].w);
       }
     }
+    float dot[G];
+#pragma unroll
+    for (int h = 0; h < G; ++h) dot[h] = (acc[h].x + acc[h].y) + (acc[h].z + acc[h].w);
 #pragma unroll
     for (int off = 1; off < 4; off <<= 1)
 #pragma unroll
@@ -463,14 +470,17 @@ __global__ void __launch_bounds__(kShThreads) decode_shared_kernel(CacheView c, 
     if (sub == 0 && jl < nr) {
       const bool masked = q_real && sId[jl] < pad;       // padding pairs are masked
 #pragma unroll
-      for (int h = 0; h < G; ++h) sP[h * rows + jl] = masked ? -INFINITY : dot[h] * sc2;
+      for (int h = 0; h < G; ++h) sP[h * rows + jl] = masked ? -INFINITY : dot[h];
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");   // V too: after the first exchange nobody reads the cache
   __syncthreads();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-  // ---- a warp per head: maximum, exponentials relative to it, their sum; to every peer
+  // ---- a warp per head: maximum, exponentials, their sum; to every peer.  The exponentials (log2 domain) are relative to the
+  // maximum's next whole number, so that the factor between two CTAs' references is a power of two and a weight has the error of
+  // one exponential, and a logit is scaled and its reference subtracted with one rounding.
+  const float sc2 = a.scale * kLog2e;
   if (warp < G) {
     float* p = sP + warp * rows;
     float m = -INFINITY, t = 0.f;
@@ -478,9 +488,10 @@ __global__ void __launch_bounds__(kShThreads) decode_shared_kernel(CacheView c, 
     for (int jl = lane; jl < nr; jl += 32) m = fmaxf(m, p[jl]);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+    m = ceilf(m * sc2);
     const float ref = m == -INFINITY ? 0.f : m;          // (a piece of padding only)
 #pragma unroll 1
-    for (int jl = lane; jl < nr; jl += 32) { const float e = ex2f(p[jl] - ref); p[jl] = e; t += e; }
+    for (int jl = lane; jl < nr; jl += 32) { const float e = ex2f(fmaf(p[jl], sc2, -ref)); p[jl] = e; t += e; }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     if (lane < (int)C) {
@@ -495,11 +506,11 @@ __global__ void __launch_bounds__(kShThreads) decode_shared_kernel(CacheView c, 
     for (uint32_t p = 0; p < C; ++p) top = fmaxf(top, sStat[p * 2 * G + tid]);
     for (uint32_t p = 0; p < C; ++p) {                   // fixed order
       const float m = sStat[p * 2 * G + tid];
-      t += m == -INFINITY ? 0.f : sStat[(p * 2 + 1) * G + tid] * ex2f(m - top);
+      t += m == -INFINITY ? 0.f : sStat[(p * 2 + 1) * G + tid] * pow2_whole(m - top);
     }
     const float own = sStat[rank * 2 * G + tid];
     // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
-    sF[tid] = (q_real && (own != -INFINITY || top == -INFINITY)) ? ex2f(own - top) / t : 0.f;
+    sF[tid] = (q_real && (own != -INFINITY || top == -INFINITY)) ? pow2_whole(own - top) / t : 0.f;
   }
   __syncthreads();
 

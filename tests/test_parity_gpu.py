@@ -526,6 +526,40 @@ def test_f32_decode_with_caches_shared_by_clusters(b, Hkv, g, d, K, kw):
         assert_same_run(run_free(wl), run_free(wl, micro=1))
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,bound", [
+    (1, 8, 1, 128, 900, 2.5e-7),      # shared by eight
+    (4, 4, 4, 128, 512, 2.15e-7),     # by eight, 64 rows each
+    (1, 8, 1, 128, 100, 2.0e-7),      # by four
+    (1, 1, 8, 64, 300, 1.8e-7),
+])
+def test_f32_decode_weights_of_shared_caches_against_64_bits(b, Hkv, g, d, K, bound):
+    # 2-norm of a step's weights (the rule keeps the last step's alone) from 64 bits, relative.  The bounds are what a CTA with a
+    # cache of its own leaves on these inputs (2.26e-7, 1.94e-7, 1.81e-7, 1.62e-7) and a tenth; clusters that summed 32
+    # products in one chain and multiplied two approximate exponentials were at 3.07e-7, 2.47e-7, 2.34e-7 and 1.73e-7
+    num = den = 0.0
+    for seed in range(6):
+        gen = torch.Generator("cuda").manual_seed(seed)
+        draw = lambda *n: [torch.randn(b, *n, h, d, device="cuda", generator=gen) * s
+                           for h, s in ((g * Hkv, 1.5), (Hkv, 1.0), (Hkv, 1.0))]
+        cache = bm.BatchMaxCache(bm.Config(batch=b, n_q_heads=g * Hkv, n_kv_heads=Hkv, head_dim=d, kv_max=K + 4, block_max=K,
+                                           dtype="f32", rule="current_query"))
+        prompt = draw(K)
+        cache.prefill_block(*prompt, 0)
+        keys = prompt[1].double()
+        for _ in range(4):
+            q, k, v = draw()
+            cache.decode_step(q, k, v)
+            keys = torch.cat([keys, k[:, None].double()], 1)
+            logits = torch.einsum("bhgd,bnhd->bhgn", q.double().view(b, Hkv, g, d), keys) / d ** 0.5
+            want = torch.softmax(logits, -1).sum(2)
+            for smp, kh in [(x, h) for x in range(b) for h in range(Hkv)]:
+                got = cache.export(0, smp, kh)[1].double().to("cuda")
+                num += (got - want[smp, kh]).square().sum().item()
+                den += want[smp, kh].square().sum().item()
+        cache.close()
+    assert (num / den) ** 0.5 < bound
+
+
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", [
     (4, 4, 4, 128, 256, 1280),   # the whole batch would share a key tile among 2 CTAs, a single sample among 8
     (4, 4, 4, 128, 256, 512),    # ... 4 and 8
