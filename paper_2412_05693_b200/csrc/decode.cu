@@ -506,11 +506,11 @@ __global__ void __launch_bounds__(kShThreads) decode_shared_kernel(CacheView c, 
     for (uint32_t p = 0; p < C; ++p) top = fmaxf(top, sStat[p * 2 * G + tid]);
     for (uint32_t p = 0; p < C; ++p) {                   // fixed order
       const float m = sStat[p * 2 * G + tid];
-      t += m == -INFINITY ? 0.f : sStat[(p * 2 + 1) * G + tid] * pow2_whole(m - top);
+      const float l = sStat[(p * 2 + 1) * G + tid];
+      t += m == -INFINITY ? l : l * pow2_whole(m - top); // (-inf: a piece without weight, whose sum is 0, or NaN logits alone)
     }
-    const float own = sStat[rank * 2 * G + tid];
-    // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
-    sF[tid] = (q_real && (own != -INFINITY || top == -INFINITY)) ? pow2_whole(own - top) / t : 0.f;
+    // (a piece without weight: 0; a cache whose logits are all -inf, or that holds a NaN: NaN)
+    sF[tid] = q_real ? pow2_whole(sStat[rank * 2 * G + tid] - top) / t : 0.f;
   }
   __syncthreads();
 

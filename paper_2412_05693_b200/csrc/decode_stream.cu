@@ -649,11 +649,11 @@ decode_stream_kernel(const CacheView c, const StreamArgs a, const __grid_constan
           float t = there ? s_xstat[p * 2 * G + G + h] : 0.f, top = m;
 #pragma unroll
           for (int off = kMaxCluster / 2; off > 0; off >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, off));
-          t = m == -INFINITY ? 0.f : t * ex2(m - top);
+          if (m != -INFINITY) t *= ex2(m - top);   // (-inf: a piece without weight, whose sum is 0, or NaN logits alone)
 #pragma unroll
           for (int off = kMaxCluster / 2; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-          // (a piece without weight: 0; a cache whose logits are all -inf: NaN)
-          const float fh = (q_real && (own != -INFINITY || top == -INFINITY)) ? ex2(own - top) / t : 0.f;
+          // (a piece without weight: 0; a cache whose logits are all -inf, or that holds a NaN: NaN)
+          const float fh = q_real ? ex2(own - top) / t : 0.f;
 #pragma unroll
           for (int y = q; y < min(G, q + 4); ++y) f[y] = __shfl_sync(0xffffffffu, fh, 8 * (y - q));
         }

@@ -307,6 +307,41 @@ def test_evicting_decode_step_with_a_nan_query(b, Hkv, g, d, K, dtype, kw):
     assert torch.equal(ids, before[0]) and torch.equal(k_rows, before[2]) and torch.equal(v_rows, before[3])
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,dtype", [
+    (1, 3, 2, 64, 40, "f32"),            # shared by four CTAs, ten rows each
+    (2, 4, 4, 128, 300, "f32"),          # by eight
+    (1, 4, 2, 128, 1024, "bf16"),        # the stream over a cluster of eight
+    (4, 8, 4, 128, 1024, "bf16"),        # ... of four
+])
+def test_evicting_decode_step_with_nan_keys_in_one_part_of_a_shared_cache(b, Hkv, g, d, K, dtype):
+    # the first half of one cache's keys is NaN (whole shares of some of the CTAs): every weight of the cache is NaN, its
+    # highest position leaves, and no other cache changes
+    wl = tiny("nan_keys", b=b, Hq=g * Hkv, Hkv=Hkv, s=K, B=K, K=K, steps=1, dtype=dtype, d=d)
+    inp = Inputs(wl, "cuda")
+    prompt, (q, k, v) = inp.block(0, 0, K), (x[:, 0].contiguous() for x in inp.block(0, K, 1))
+    smp, kh = b // 2, Hkv - 1
+    states, outs = [], []
+    for nan in (False, True):
+        cache = bm.BatchMaxCache(make_config(wl))
+        cache.prefill_block(*prompt, 0)
+        ids, sums, k_rows, v_rows = cache.export(0, smp, kh, rows=True)
+        if nan:
+            k_rows = k_rows.clone()
+            k_rows[:K // 2] = float("nan")
+            cache.import_(ids, sums, k_rows, v_rows, 0, smp, kh)
+        outs.append(cache.decode_step(q, k, v, evict_to=K).view(b, Hkv, g * d))
+        assert cache.status() == 0
+        states.append({u: cache.export(0, *u, rows=True) for u in all_units(wl)})
+        cache.close()
+    for u, want in states[0].items():
+        if u != (smp, kh):
+            assert all(torch.equal(x, y) for x, y in zip(states[1][u], want)) and torch.equal(outs[0][u], outs[1][u])
+    assert torch.isnan(outs[1][smp, kh]).all()
+    got = states[1][(smp, kh)]
+    assert torch.isnan(got[1]).all()
+    assert torch.equal(got[0], ids) and torch.equal(got[2].nan_to_num(), k_rows.nan_to_num()) and torch.equal(got[3], v_rows)
+
+
 # the forward kernel with two row tiles per CTA: the handle's batch makes 1024 pairs of tiles
 PAIR_GRIDS = [(64, 16, 1, 64, 200, 150),     # the second tile ragged, and it sees one key tile more than the first
               (64, 16, 1, 128, 300, 129),    # three tiles: the last CTA's second tile has no rows
