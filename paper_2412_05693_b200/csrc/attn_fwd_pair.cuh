@@ -436,8 +436,10 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
         const float m0 = x == 0 ? m_used : __uint_as_float(om), m1 = x == 0 ? __uint_as_float(om) : m_used;
         const float l0 = x == 0 ? l : __uint_as_float(ol), l1 = x == 0 ? __uint_as_float(ol) : l;
         const float m = max3_nan(m0, m1, -INFINITY);
-        const float w0 = m0 == -INFINITY && m != -INFINITY ? 0.f : ex2(m0 - m), w1 = m1 == -INFINITY ? 0.f : ex2(m1 - m);
-        const float lt = (w0 == 0.f ? 0.f : l0 * w0) + (w1 == 0.f ? 0.f : l1 * w1);
+        // a group that saw no key is left out; one whose weight is too small for fp32 is not, since its sums may be NaN
+        const bool out0 = m0 == -INFINITY && m != -INFINITY, out1 = m1 == -INFINITY;
+        const float w0 = out0 ? 0.f : ex2(m0 - m), w1 = out1 ? 0.f : ex2(m1 - m);
+        const float lt = (out0 ? 0.f : l0 * w0) + (out1 ? 0.f : l1 * w1);
         const float inv = real_row ? 1.f / lt : 0.f;
         const float f0 = w0 * inv, f1 = w1 * inv;
         const int col0 = x * (D / 2);
@@ -449,8 +451,8 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
           tmem_ld32(tm_o0 + D + lane_addr + col0 + 32 * cc, o1);
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; ++e)   // (a group without weight may hold anything)
-            o0[e] = __float_as_uint((w0 == 0.f ? 0.f : __uint_as_float(o0[e]) * f0) + (w1 == 0.f ? 0.f : __uint_as_float(o1[e]) * f1));
+          for (int e = 0; e < 32; ++e)   // (a group that is left out may hold anything)
+            o0[e] = __float_as_uint((out0 ? 0.f : __uint_as_float(o0[e]) * f0) + (out1 ? 0.f : __uint_as_float(o1[e]) * f1));
 #pragma unroll
           for (int p = 0; p < 4; ++p) {
             uint32_t w[4];

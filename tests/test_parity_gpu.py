@@ -422,6 +422,25 @@ def test_forward_with_key_tiles_taken_in_turn(b, Hkv, g, d, B, K):
             assert (out[s] - want).nan_to_num_(0.0).abs().max() < 2e-2
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("nan_at,large_at", [(5, 3 * 128 + 7), (128 + 9, 4 * 128 + 1), (2 * 128, 128)])
+def test_forward_with_key_tiles_taken_in_turn_keeps_a_nan_far_below_the_maximum(d, nan_at, large_at):
+    # the key tiles with the NaN go to one group, a logit 250 (log2) above everything else to the other: the first group's weight
+    # is too small for fp32, and every row is NaN all the same, as softmax has it
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen).bfloat16()
+    K, B = 640, 64
+    q, k, v = f(1, K + B, 1, d), f(1, K + B, 1, d), f(1, K + B, 1, d)
+    q[..., 3] = q[..., 3].abs() + 1.0
+    cache = bm.BatchMaxCache(bm.Config(batch=1, n_q_heads=1, n_kv_heads=1, head_dim=d, kv_max=K + B, block_max=K))
+    k[0, large_at, 0, 3] = 2000.0
+    k[0, nan_at, 0, 3] = float("nan")
+    cache.prefill_block(*(x[:, :K].contiguous() for x in (q, k, v)), 0)
+    out = cache.prefill_block(*(x[:, K:].contiguous() for x in (q, k, v)), K)
+    assert torch.isnan(out).all() and cache.status() == 0
+    cache.close()
+
+
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 @pytest.mark.parametrize("b,Hkv,g,d,B,K", PAIR_GRIDS[1:3])
 def test_forward_on_pairs_of_row_tiles_with_nan_and_inf_keys(b, Hkv, g, d, B, K, value):
