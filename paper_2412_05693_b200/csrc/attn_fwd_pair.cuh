@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
     int n = 0;                                    // key tiles so far
     for (int k = 0;; ++k) {
       const Item it = read_item(k);
-      const bool go = __all_sync(0xffffffffu, it.T > 0);   // (lanes may see a wait give up at different times)
+      // Threads may see a wait give up at different times.  A SPLIT item has barriers of both groups: they enter it together or not at all.
+      const bool go = SPLIT ? named_bar_all(1, 256, it.T > 0) : __all_sync(0xffffffffu, it.T > 0);
       if (lane == 0) item_read(k);
       if (!go) break;
       const int nx = x ? it.n1 : it.n0, rt = x ? it.rt1 : it.rt0, row = rt * kTileM + r;

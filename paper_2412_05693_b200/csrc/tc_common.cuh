@@ -276,6 +276,13 @@ __device__ __forceinline__ uint32_t sw128_offset(int r, int pc) {
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
+// ... and whether all of them say so
+__device__ __forceinline__ bool named_bar_all(int id, int nthreads, bool x) {
+  int all;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 p, %1, 0;\nbar.red.and.pred q, %2, %3, p;\nselp.b32 %0, 1, 0, q;\n}\n"
+               : "=r"(all) : "r"((int)x), "r"(id), "r"(nthreads) : "memory");
+  return all != 0;
+}
 
 }  // namespace tc
 }  // namespace bm

@@ -422,6 +422,47 @@ def test_forward_with_key_tiles_taken_in_turn(b, Hkv, g, d, B, K):
             assert (out[s] - want).nan_to_num_(0.0).abs().max() < 2e-2
 
 
+@pytest.mark.parametrize("d,pads", [(64, None), (128, None), (128, [0, 130, 37, 0])])
+def test_forward_with_key_tiles_taken_in_turn_on_few_free_sms(d, pads):
+    # another stream's kernels hold 140 SMs, so that the CTAs that start on the others take several work items each: exchange
+    # columns, output stage and barriers are used again, and nothing changes
+    gen = torch.Generator(device="cuda").manual_seed(13)
+    f = lambda *s: torch.randn(*s, device="cuda", generator=gen).bfloat16()
+    long = [f(35, 4096, 4, 128) for _ in range(3)]
+    holder = bm.BatchMaxCache(bm.Config(batch=35, n_q_heads=4, n_kv_heads=4, head_dim=128, kv_max=8192, block_max=4096))
+    holder.prefill_block(*long, 0)
+    long = [x[:, :128].contiguous() for x in long]
+    blocks = [[f(4, I, h, d) for h in (32, 16, 16)] for I in (300, 128)]
+
+    def run():
+        cache = bm.BatchMaxCache(bm.Config(batch=4, n_q_heads=32, n_kv_heads=16, head_dim=d, kv_max=500, block_max=300))
+        if pads is not None:
+            cache.set_left_pad(pads)
+        cache.prefill_block(*blocks[0], 0)
+        torch.cuda.synchronize()
+        held = torch.empty_like(long[0])
+        for t in range(6 if others else 0):
+            with torch.cuda.stream(side):
+                holder.prefill_block(*long, 4096 + at[0], out=held, evict_to=4096)
+                at[0] += 128
+        out = cache.prefill_block(*blocks[1], 300)         # 128 row tiles
+        torch.cuda.synchronize()
+        assert cache.status() == 0 and holder.status() == 0
+        sums = [cache.export(0, s, h)[1] for s in range(4) for h in range(16)]
+        cache.close()
+        return out, torch.cat(sums)
+
+    side, at = torch.cuda.Stream(), [0]
+    torch.cuda.synchronize()
+    others = False
+    want = run()
+    others = True
+    for _ in range(4):
+        got = run()
+        assert all(torch.equal(x, y) for x, y in zip(got, want))
+    holder.close()
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("nan_at,large_at", [(5, 3 * 128 + 7), (128 + 9, 4 * 128 + 1), (2 * 128, 128)])
 def test_forward_with_key_tiles_taken_in_turn_keeps_a_nan_far_below_the_maximum(d, nan_at, large_at):
