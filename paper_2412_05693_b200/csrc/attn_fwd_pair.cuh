@@ -2,8 +2,10 @@
 //
 // Warps 0-3: softmax of A (a thread per query row), 4-7: of B, 8: issues every S = Q.K^T, 9 and 10: issue O += P.V of A and
 // of B, 11: TMA producer, which also asks for the CTA's next work item.  A work item is
-//   two row tiles of a cache, one for each group (they share the K and V tiles), or
-//   SPLIT: one row tile, whose key tiles the groups take in turn; their two partial outputs meet at the end.
+//   kPairs: two row tiles of a cache, one for each group (they share the K and V tiles), or
+//   kAny: two row tiles of any caches, each with key tiles of its own, loaded in turn, or a single row tile (a row's arithmetic is
+//   that of kPairs), or
+//   kSplit: one row tile, whose key tiles the groups take in turn; their two partial outputs meet at the end.
 //
 // Tensor memory, 512 columns: O_A | O_B (D each) | P_A | P_B (64 each, bf16 pairs) | S (128 at D = 128, shared by the
 // groups; two of 128 at D = 64).  A group reads its 128 logits of a row into registers at once and gives S back, so the
@@ -37,20 +39,23 @@ struct PairSmem {
   static constexpr int kThreads = 384;
 };
 
-template <int D, bool PAD, bool SPLIT>
+enum Items { kPairs, kAny, kSplit };   // what a work item is (above)
+
+template <int D, bool PAD, Items ITEMS>
 __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ TcMaps maps, const TcArgs a) {
   using L = PairSmem<D>;
+  constexpr bool SPLIT = ITEMS == kSplit, ANY = ITEMS == kAny;
   constexpr int kQkWarp = 8, kPvWarp = 9 /* A; 10: B */, kTmaWarp = 11, NS = L::kStages;
   constexpr int NSB = D == 128 ? 1 : 2;                  // logit buffers
   constexpr int B_QFULL = 0, B_QFREE = 2, B_KFULL = 4, B_KFREE = B_KFULL + NS, B_VFULL = B_KFREE + NS, B_VFREE = B_VFULL + NS,
                 B_SFULL = B_VFREE + NS, B_SFREE = B_SFULL + 2, B_P = B_SFREE + 2 /* [half][group] */, B_PV = B_P + 4 /* likewise */,
                 B_RESP = B_PV + 4, B_NEXT = B_RESP + 1, B_NEXTFREE = B_NEXT + 2, B_COUNT = B_NEXTFREE + 2;
-  static_assert(8 * B_COUNT + 5 * 16 + 8 <= 512, "");
+  static_assert(8 * B_COUNT + 7 * 16 + 8 <= 512, "");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* resp = sm + L::kBars;                   // response to the request for a work item, 16 bytes
-  int4* items = reinterpret_cast<int4*>(sm + L::kBars + 16);   // [2][2]: this work item and the next
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBars + 80);
+  int4* items = reinterpret_cast<int4*>(sm + L::kBars + 16);   // [2][2]: this work item and the next; [2]: kAny, the second group's caches
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::kBars + 112);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -58,25 +63,35 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
   const int R = a.I * a.g, qpt = kTileM / a.g;   // query rows of a cache; inputs (positions) covered by a row tile
   const int t_old = (a.n_old + kTileN - 1) / kTileN;
 
+  struct Place { int unit, smp, kh; };           // cache, its sample, its head
   struct Item { int unit, smp, kh, rt0, rt1, n0, n1, T; };   // row tile and number of key tiles of either group; key tiles loaded
   // Written by the producer, m-th item into place m % 2 (T = 0: there is none).  Row tiles are handed out last first (a later
-  // tile sees more of the block's own keys): within a cache, or (a.across) over all caches.
+  // tile sees more of the block's own keys): within a cache, or (a.across, kAny) over all caches.
   auto write_item = [&](int m, bool there, int bx, int by) {
     Item it;
-    it.unit = a.across ? bx : by;
+    const int row_tiles = ANY ? (R + kTileM - 1) / kTileM : 0, second = ANY ? a.any * bx + a.any - 1 : 0;
+    it.unit = ANY ? a.any * bx % a.units : a.across ? bx : by;
     it.smp = it.unit / a.Hkv;
     it.kh = it.unit - it.smp * a.Hkv;
     const int grp = a.across ? (int)gridDim.y - 1 - by : (int)gridDim.x - 1 - bx;
     // key tiles a row tile sees: the cached ones and the block's up to its last input; no rows, no tiles
     auto n_tiles = [&](int rt) { return rt * qpt >= a.I ? 0 : t_old + min(a.I - 1, rt * qpt + qpt - 1) / kTileN + 1; };
-    it.rt0 = SPLIT ? grp : 2 * grp;
-    it.rt1 = SPLIT ? grp : 2 * grp + 1;
+    it.rt0 = ANY ? row_tiles - 1 - a.any * bx / a.units : SPLIT ? grp : 2 * grp;
+    it.rt1 = ANY ? row_tiles - 1 - second / a.units : SPLIT ? grp : 2 * grp + 1;
     it.n0 = n_tiles(it.rt0);
-    it.n1 = SPLIT ? it.n0 / 2 : n_tiles(it.rt1);
-    it.T = SPLIT ? it.n0 : max(it.n0, it.n1);
+    it.n1 = SPLIT ? it.n0 / 2 : ANY && (a.any < 2 || it.rt1 < 0) ? 0 : n_tiles(it.rt1);
+    it.T = SPLIT ? it.n0 : ANY ? it.n0 + it.n1 : max(it.n0, it.n1);
     if (SPLIT) it.n0 -= it.n1;
     items[2 * (m & 1)] = make_int4(it.unit, it.smp, it.kh, there ? it.T : 0);
     items[2 * (m & 1) + 1] = make_int4(it.rt0, it.rt1, it.n0, it.n1);
+    if (ANY) {
+      const int unit = second % a.units, smp = unit / a.Hkv;
+      items[4 + (m & 1)] = make_int4(unit, smp, unit - smp * a.Hkv, 0);
+    }
+  };
+  auto place = [&](const Item& it, int m, int x) {   // of group x's row tile
+    if (ANY && x == 1) { const int4 u = items[4 + (m & 1)]; return Place{u.x, u.y, u.z}; }
+    return Place{it.unit, it.smp, it.kh};
   };
   auto read_item = [&](int m) {
     if (m > 0) mbar_wait(&bars[B_NEXT + (m & 1)], ((m - 1) >> 1) & 1, abort_flag, a.status);
@@ -86,7 +101,11 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
     return it;
   };
   auto item_read = [&](int m) { mbar_arrive(&bars[B_NEXTFREE + (m & 1)]); };   // once per warp
-  auto takes = [&](const Item& it, int x, int j) { return SPLIT ? (j & 1) == x : j < (x ? it.n1 : it.n0); };   // group x, key tile j
+  // kAny: the group whose key tile is the j-th that is loaded: in turn, then what the longer one has left
+  auto owner = [&](const Item& it, int j) { return j < 2 * min(it.n0, it.n1) ? j & 1 : it.n0 > it.n1 ? 0 : 1; };
+  auto takes = [&](const Item& it, int x, int j) {   // group x, j-th key tile
+    return SPLIT ? (j & 1) == x : ANY ? owner(it, j) == x : j < (x ? it.n1 : it.n0);
+  };
   if (warp == kTmaWarp && lane == 0) {
     *abort_flag = 0;
 #pragma unroll 1
@@ -118,6 +137,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
         for (bool more = true; more; ++k) {
           const Item it = read_item(k);          // (its own)
           const bool two = !SPLIT && it.n1 > 0;  // query tiles
+          const Place own[2] = {place(it, k, 0), place(it, k, 1)};
 #pragma unroll 1
           for (int e = 0; e <= it.T; ++e) {
             if (e == it.T - 1) {                 // (not earlier: a CTA that is ahead should find the item still there)
@@ -135,8 +155,8 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
                 mbar_expect_tx(&bars[B_QFULL + x], L::kTileBytes);
 #pragma unroll 1
                 for (int c = 0; c < L::kChunks; ++c)
-                  tma_load_5d(sm + L::kQ + x * L::kTileBytes + c * 16384, &maps.q, c * 64, 0, it.kh, (x ? it.rt1 : it.rt0) * qpt,
-                              it.smp, &bars[B_QFULL + x]);
+                  tma_load_5d(sm + L::kQ + x * L::kTileBytes + c * 16384, &maps.q, c * 64, 0, x ? own[1].kh : own[0].kh,
+                              (x ? it.rt1 : it.rt0) * qpt, x ? own[1].smp : own[0].smp, &bars[B_QFULL + x]);
               }
 #pragma unroll 1
             for (int is_v = 0; is_v < 2; ++is_v) {   // K_e, V_{e-1}
@@ -148,10 +168,13 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
               if (n >= NS) wait((is_v ? B_VFREE : B_KFREE) + s, n / NS - 1);
               ++n;
               mbar_expect_tx(bar, L::kTileBytes);
-              const bool old = j < t_old;
+              const int both = ANY ? min(it.n0, it.n1) : 0;        // key tiles that the groups take in turn
+              const int t = j < 2 * both ? j >> 1 : j - both;      // the tile's place in its cache
+              const Place& of = ANY && owner(it, j) ? own[1] : own[0];
+              const bool old = t < t_old;
               const CUtensorMap* m = old ? (is_v ? &maps.v_slab : &maps.k_slab) : (is_v ? &maps.v_blk : &maps.k_blk);
-              tma_load_5d(sm + (is_v ? L::kV : L::kK) + s * L::kTileBytes, m, 0, old ? 0 : it.kh, (old ? j : j - t_old) * kTileN,
-                          old ? it.unit : it.smp, 0, bar);
+              tma_load_5d(sm + (is_v ? L::kV : L::kK) + s * L::kTileBytes, m, 0, old ? 0 : of.kh, (old ? t : t - t_old) * kTileN,
+                          old ? of.unit : of.smp, 0, bar);
             }
           }
           wait(B_RESP, k);
@@ -188,6 +211,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
           item_read(k);
           if (it.T == 0) break;
           wait(B_QFULL, qc0++);
+          bool q1_there = false;
 #pragma unroll 1
           for (int j = 0; j < it.T; ++j, ++kc) {
             wait(B_KFULL + kc % NS, kc / NS);
@@ -195,7 +219,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
 #pragma unroll 1
             for (int x = 0; x < 2; ++x) {
               if (!takes(it, x, j)) continue;
-              if (x == 1 && j == 0 && !SPLIT) wait(B_QFULL + 1, qc1++);
+              if (x == 1 && !SPLIT && (ANY ? !q1_there : j == 0)) { wait(B_QFULL + 1, qc1++); q1_there = true; }
               // the logits that the buffer holds have been read
               const int before = NSB == 2 ? x : last, n = before == 0 ? sc0 : sc1;
               if (before >= 0 && n > 0) poll(B_SFREE + before, n - 1);
@@ -261,6 +285,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
     int n = 0;                                    // key tiles so far
     for (int k = 0;; ++k) {
       const Item it = read_item(k);
+      const Place own = place(it, k, x);
       // Threads may see a wait give up at different times.  A SPLIT item has barriers of both groups: they enter it together or not at all.
       const bool go = SPLIT ? named_bar_all(1, 256, it.T > 0) : __all_sync(0xffffffffu, it.T > 0);
       if (lane == 0) item_read(k);
@@ -269,9 +294,9 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
       const int i_row = min(a.I - 1, row >> g_log);   // rows past the block's end behave like its last input
       // Left padding: a padding pair is masked for every real query.  Among the block's own keys padding is a prefix of
       // positions; among the cached pairs it is whatever kv_ids say (the rows of an unordered cache are in no order).
-      const int pad = PAD ? a.left_pad[it.smp] : 0;
+      const int pad = PAD ? a.left_pad[own.smp] : 0;
       const bool real_row = !PAD || a.pos0 + i_row >= pad;
-      const int* ids = a.kv_ids + (size_t)it.unit * a.cap;
+      const int* ids = a.kv_ids + (size_t)own.unit * a.cap;
       int id4[4];
       auto fetch_ids = [&](int j) {               // of this warp's lanes, for the mask of a cached key tile
 #pragma unroll
@@ -390,7 +415,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
         fence_async_smem();
         __syncwarp();
         if (lane == 0) {
-          if (i_warp < a.I) tma_store_5d(&maps.o, stage, chunk * 64, 0, it.kh, i_warp, it.smp);
+          if (i_warp < a.I) tma_store_5d(&maps.o, stage, chunk * 64, 0, own.kh, i_warp, own.smp);
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
       };
@@ -419,7 +444,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
               *reinterpret_cast<uint4*>(stage + sw128_offset(lane, p)) = make_uint4(w[4 * p], w[4 * p + 1], w[4 * p + 2], w[4 * p + 3]);
             store(cc);
           }
-          if (row < R) a.lse2[(size_t)it.unit * R + row] = real_row ? m_used + log2f(l) : INFINITY;  // +inf: no weights
+          if (row < R) a.lse2[(size_t)own.unit * R + row] = real_row ? m_used + log2f(l) : INFINITY;  // +inf: no weights
         }
       } else {
         // the groups exchange a row's (maximum, sum) through their P columns; either finishes half of the row's elements
@@ -466,7 +491,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_pair(const __grid_constant__ 
         if (D == 64) fence_async_smem();
         named_bar_sync(1, 256);                   // both outputs have been read: the next item may replace them
         if (D == 128 || x == 0) store(D == 128 ? x : 0);
-        if (x == 0 && row < R) a.lse2[(size_t)it.unit * R + row] = real_row ? m + log2f(lt) : INFINITY;
+        if (x == 0 && row < R) a.lse2[(size_t)own.unit * R + row] = real_row ? m + log2f(lt) : INFINITY;
       }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");

@@ -50,6 +50,8 @@ struct TcArgs {
   int overwrite;     // 1: the column sums replace sum_weights instead of being added
   int key_tiles;     // key tiles per CTA of the score pass (QRES)
   int across;        // attn_fwd_pair: 1 = row tiles in order over all caches (grid.x = caches), 0 = within a cache
+  int any;           // attn_fwd_pair<kAny>: row tiles of a work item, 1 or 2
+  int units;         // caches of the call
   float* sum_sq;     // rule 4: sums of squared weights (cached pairs / the block's pairs), else null
   float* new_sq;
 };
@@ -345,7 +347,8 @@ TcArgs make_args(const CacheView& c, const BlockArgs& a) {
   t.overwrite = rule_overwrites(c.rule) ? 1 : 0;
   t.sum_sq = c.sum_sq; t.new_sq = a.new_sq;
   t.key_tiles = 1;
-  t.across = 0;
+  t.across = 0; t.any = 1;
+  t.units = c.nsamples * c.Hkv;
   return t;
 }
 
@@ -375,33 +378,50 @@ cudaError_t launch_onepass(const CacheView& c, const BlockArgs& a, cudaStream_t 
   return cudaGetLastError();
 }
 
-template <int D, bool PAD, bool SPLIT>
-cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+template <int D, bool PAD, Items ITEMS>
+cudaError_t launch_fwd_pair(const CacheView& c, const BlockArgs& a, const TcArgs& args, dim3 grid, cudaStream_t st) {
   using L = PairSmem<D>;
   static SmemConfigured configured;
-  if (cudaError_t e = configured.ensure(attn_fwd_pair<D, PAD, SPLIT>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
-  const int tiles = (a.I * c.g + kTileM - 1) / kTileM, units = c.nsamples * c.Hkv;
+  if (cudaError_t e = configured.ensure(attn_fwd_pair<D, PAD, ITEMS>, (size_t)(L::kTotal)); e != cudaSuccess) return e;
+  ProfileScope prof(kAttnFwd, st);
+  attn_fwd_pair<D, PAD, ITEMS><<<grid, L::kThreads, L::kTotal, st>>>(g_maps, args);
+  count_launch();
+  return cudaGetLastError();
+}
+
+// What the forward kernel's work items are.
+template <int D, bool PAD>
+cudaError_t launch_fwd_items(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
+  const int tiles = (a.I * c.g + kTileM - 1) / kTileM, units = c.nsamples * c.Hkv, groups = (tiles + 1) / 2, sms = sm_count();
+  const long long all = (long long)tiles * units;
   TcArgs args = make_args(c, a);
   // Row tiles in order over all caches (the longest first) where the call's keys and values stay in L2: 32 caches of 512
   // pairs and a block of 512 40.3 us, cache by cache 43.3; 192 caches of 499, 74 MB, the same; 1024 caches 1380 / 1254.
   args.across = (size_t)units * (c.n_old + a.I) * D * 4 <= (size_t)64 << 20;
-  const int groups = SPLIT ? tiles : (tiles + 1) / 2;
-  ProfileScope prof(kAttnFwd, st);
-  attn_fwd_pair<D, PAD, SPLIT><<<args.across ? dim3(units, groups) : dim3(groups, units), L::kThreads, L::kTotal, st>>>(g_maps, args);
-  count_launch();
-  return cudaGetLastError();
+  // Both groups on one row tile while every row tile of the handle's batch has an SM to itself (128 row tiles of 12 key tiles
+  // 24.4 us, two row tiles per CTA 35.1; 256 row tiles 35.2 / 35.4).  The handle's caches decide and not the call's: the
+  // sums of a row are cut differently, and outputs do not depend on how a batch is cut into sample ranges.
+  if ((long long)tiles * c.layer_units <= sms)
+    return launch_fwd_pair<D, PAD, kSplit>(c, a, args, args.across ? dim3(units, tiles) : dim3(tiles, units), st);
+  // Row tiles of any caches: one by one while a call's (a sample range's) have an SM each, and two by two where caches with an
+  // odd number of them would leave items with a single one (which take four sevenths of a pair's time) and need a round more.
+  // Beyond two rounds keys and values that are loaded once per row tile cost more than that.  us per prefill call (forward, column
+  // sums, cut), pairs / any: one sample of 64, 32 row tiles of 8 caches, 1024 pairs 61.4 / 53.2, 16 of them, 512 pairs 42.0 / 38.0;
+  // three row tiles of 80 caches, 512 pairs 50.4 / 44.5, 1024 pairs 72.3 / 62.5, of 176 caches 77.0 / 72.8; one of 176 48.2 / 44.5, of
+  // 320 69.6 / 71.4, of 512 at d = 64 122.5 / 109.8; three of 320 caches 123.7 / 130.2.
+  auto rounds = [&](long long items) { return (items + sms - 1) / sms; };
+  const long long twos = rounds((all + 1) / 2);
+  if (all <= sms || (twos <= 2 && 7 * twos < (tiles == 1 ? 4 : 7) * rounds((long long)groups * units))) {
+    args.any = all <= sms ? 1 : 2;
+    return launch_fwd_pair<D, PAD, kAny>(c, a, args, dim3((unsigned)((all + args.any - 1) / args.any)), st);
+  }
+  return launch_fwd_pair<D, PAD, kPairs>(c, a, args, args.across ? dim3(units, groups) : dim3(groups, units), st);
 }
 
 template <int D>
 cudaError_t launch_fwd_t(const CacheView& c, const BlockArgs& a, cudaStream_t st) {
   if (onepass_applies(c, a)) return launch_onepass<D>(c, a, st);
-  const int tiles = (a.I * c.g + kTileM - 1) / kTileM;
-  // Both groups on one row tile while every row tile of the handle's batch has an SM to itself (128 row tiles of 12 key tiles
-  // 24.4 us, two row tiles per CTA 35.1; 256 row tiles 35.2 / 35.4).  The handle's caches decide and not the call's: the
-  // sums of a row are cut differently, and outputs do not depend on how a batch is cut into sample ranges.
-  if ((long long)tiles * c.layer_units <= sm_count())
-    return c.left_pad != nullptr ? launch_fwd_pair<D, true, true>(c, a, st) : launch_fwd_pair<D, false, true>(c, a, st);
-  return c.left_pad != nullptr ? launch_fwd_pair<D, true, false>(c, a, st) : launch_fwd_pair<D, false, false>(c, a, st);
+  return c.left_pad != nullptr ? launch_fwd_items<D, true>(c, a, st) : launch_fwd_items<D, false>(c, a, st);
 }
 
 template <int D, bool SQ, int EMU, bool QRES>

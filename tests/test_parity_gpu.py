@@ -386,6 +386,27 @@ def test_forward_on_pairs_of_row_tiles_is_bitwise_independent_of_sample_ranges(b
         assert_same_run(base, run_free(wl, micro=1, pads=pads))
 
 
+# row tiles of any caches in a work item: one each where a call's have an SM each, two where caches with an odd number of them
+# would leave many items with a single one
+ANY_GRIDS = [(25, 7, 2, 128, 60, 600, {}),                     # a ragged tile per cache, 175 of them: the last item has one
+             (16, 5, 1, 64, 300, 200, dict(pads=True)),        # three tiles of 80 caches, padding
+             (10, 8, 4, 128, 77, 200, {}),                     # three tiles per cache, 240: an item's tiles see different numbers of keys
+             (16, 11, 8, 64, 41, 0, dict(compaction="fill")),  # 528 of them, two rounds; no cached pairs at first
+             (60, 8, 2, 128, 64, 260, dict(rule="current_query"))]   # 480 caches with a tile each
+
+
+@pytest.mark.parametrize("b,Hkv,g,d,B,K,kw", ANY_GRIDS)
+def test_forward_on_row_tiles_of_any_caches(b, Hkv, g, d, B, K, kw):
+    # whole calls against the oracle; a row's arithmetic does not depend on the tile beside it, so that single samples' calls, whose
+    # items have one tile each, give the same bits
+    kw = dict(kw)
+    pads = [(37 * s) % (B + K) for s in range(b)] if kw.pop("pads", False) else None
+    wl = tiny("any", b=b, Hq=g * Hkv, Hkv=Hkv, s=K + 2 * B if K else 3 * B, B=B, K=max(K, B), steps=0, dtype="bf16", d=d)
+    run_lockstep(wl, [(0, 0), (b // 2, Hkv // 2), (b - 1, Hkv - 1)], check_rows_every=2, pads=pads, **kw)
+    base = run_free(wl, pads=pads)
+    assert_same_run(base, run_free(wl, micro=1, pads=pads))
+
+
 # few row tiles: the two softmax groups of a CTA take the key tiles of one row tile in turn
 SPLIT_GRIDS = [(1, 1, 1, 128, 131, 0),    # two row tiles: one key tile (the second group has none), then two
                (2, 2, 4, 64, 200, 129),   # cached tiles end in a single key; up to four key tiles
