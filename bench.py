@@ -336,13 +336,9 @@ def forward_kernel(wl):
 
 
 def decode_kernel(wl):
-    """The kernel of an evicting decode step on caches of K pairs, by the library's rule (stream_is_faster in
-    csrc/decode_mma.cu, on 148 SMs)."""
-    caches, kib = wl.b * wl.Hkv, (wl.K + 1) * wl.d * 4 // 1024
-    if wl.dtype != "bf16":
-        return None
-    least = 0 if caches <= 148 else (80 if wl.d == 64 else 48) if caches <= 296 else 96 if caches <= 444 else 172 if caches <= 592 else 112
-    return "decode_stream_kernel" if kib >= least else "decode_mma_kernel"
+    """The kernel of the most recent decode step, which is one of this workload's, as the library reports it."""
+    import paper_2412_05693_b200 as bm
+    return {2: "decode_mma_kernel", 3: "decode_mma_kernel", 4: "decode_stream_kernel", 5: "decode_stream_kernel"}.get(bm.last_decode_path())
 
 
 def forward_roofline(wl, attn_ms, attn_n, pk, pk_src, clocks, samples_per_launch, padded=False):

@@ -323,6 +323,9 @@ uint64_t bm_kernel_launch_count(void);
  * query rows, I * g, against at most four tiles of 128 keys, cached and new counted apart; no padding; not the
  * current-query rule). */
 int32_t bm_last_prefill_path(void);
+/* Which kernel the calling thread's last bm_decode_step used.  fp32: 0 = a CTA per cache, 1 = clusters that share a cache.  bf16: 2 = a
+ * CTA per cache, 3 = the same with all of K in registers, 4 = the stream, 5 = the stream over clusters that share a cache. */
+int32_t bm_last_decode_path(void);
 const char* bm_status_string(bm_status_t s);
 /* Text of the CUDA error behind the calling thread's most recent BM_ERR_CUDA from a kernel launch ("no error" if
  * none).  After BM_ERR_CUDA the state of the call's sample range is undefined: some of the call's kernels may have

@@ -12,6 +12,7 @@ from .binding import (  # noqa: F401
     cache_bytes_per_sample,
     debug_build,
     kernel_launch_count,
+    last_decode_path,
     last_prefill_path,
     lib,
     max_batch,

@@ -76,6 +76,7 @@ SIGNATURES = {
     "bm_profile_read": (_i32, [_i32, C.POINTER(C.c_float), C.POINTER(_i32)]),
     "bm_kernel_launch_count": (C.c_uint64, []),
     "bm_last_prefill_path": (_i32, []),
+    "bm_last_decode_path": (_i32, []),
     "bm_status_string": (C.c_char_p, [_i32]),
     "bm_last_cuda_error": (C.c_char_p, []),
 }
@@ -177,6 +178,10 @@ def kernel_launch_count() -> int:
 
 def last_prefill_path() -> int:
     return int(lib().bm_last_prefill_path())
+
+
+def last_decode_path() -> int:
+    return int(lib().bm_last_decode_path())
 
 
 KERNEL_CLASSES = {"attn_fwd": 0, "score": 1, "evict": 2, "decode": 3}

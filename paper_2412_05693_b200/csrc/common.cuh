@@ -29,6 +29,7 @@ struct CacheView {
   int32_t window, pool;     // rule 3: queries observed / recent pairs kept; width of the max-pooling (odd)
   int32_t std_permille;     // rule 4: share of the kept pairs chosen by standard deviation, in 1/1000
   int32_t padded;           // 1: some sample of the handle is left-padded (left_pad is null for calls that meet no padding)
+  int32_t in_l2;            // 1: all of the handle's caches together stay in the L2 cache
   int32_t layer_units;      // caches of the handle in one layer: what a kernel is chosen by where the choice changes the order
                             // of a sum, so that results do not depend on how a batch is cut into sample ranges
 };
@@ -138,6 +139,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 extern unsigned long long g_launch_count;
+extern thread_local int g_last_decode_path;   // (api.cu) what bm_last_decode_path reports
 inline void count_launch(int n = 1) { g_launch_count += (unsigned long long)n; }
 
 // Optional per-launch timing: when enabled, a ProfileScope brackets a launch with two CUDA events.

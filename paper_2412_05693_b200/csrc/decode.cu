@@ -646,6 +646,7 @@ cudaError_t launch_shared(const CacheView& c, DecodeArgs a, int C, cudaStream_t 
   cudaError_t err;
   {
     ProfileScope prof(kDecode, st);
+    g_last_decode_path = 1;
     err = launch_dependent_cluster(decode_shared_kernel<D, G>, dim3(c.nsamples * c.Hkv * C), dim3(kShThreads), smem, C, st, c, a, rows);
     count_launch();
   }
@@ -667,6 +668,7 @@ cudaError_t launch_t(const CacheView& c, const DecodeArgs& a, cudaStream_t st) {
   static SmemConfigured configured;
   if (cudaError_t err = configured.ensure(decode_kernel<T, D, G>, smem); err != cudaSuccess) return err;
   ProfileScope prof(kDecode, st);
+  g_last_decode_path = 0;
   decode_kernel<T, D, G><<<c.nsamples * c.Hkv, kDecThreads, smem, st>>>(c, a);
   count_launch();
   return cudaGetLastError();

@@ -7,7 +7,8 @@
 // Both contractions are invariant under a permutation of the contracted index, and the output index of the
 // second one can be un-permuted when it is written, so every thread loads whole 16-byte pieces of cache
 // rows (coalesced) and the MMA fragment slots are assigned to whatever elements those loads delivered.
-// The instance for grids of at most one cache per SM (KD > 1 below) differs in how rows travel: K is loaded once and
+// The stream (decode_stream.cu) takes most steps; which ones are left to these kernels stream_is_faster says, below.
+// The instance for calls of at most one cache per SM (KD > 1) differs in how rows travel: K is loaded once and
 // kept in registers, V is staged in shared memory by TMA while the softmax phases run and read back with
 // transposing ldmatrix (standard fragment layout), and the rows behind the pair that leaves are written from there.
 #include "evict.cuh"
@@ -640,6 +641,7 @@ cudaError_t launch_nt_p(const CacheView& c, const DecodeArgs& a, cudaStream_t st
   static SmemConfigured configured;
   if (cudaError_t err = configured.ensure(decode_mma_kernel<D, G, NT, PLAIN, KD>, smem); err != cudaSuccess) return err;
   ProfileScope prof(kDecode, st);
+  g_last_decode_path = KD > 1 ? 3 : 2;
   const cudaError_t err =
       launch_dependent(decode_mma_kernel<D, G, NT, PLAIN, KD>, dim3(c.nsamples * c.Hkv), dim3(NT), smem, st, c, a, vmap);
   count_launch();
@@ -704,32 +706,45 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 
 // Which kernel takes a step: the stream, or this file's kernels.  By the handle's caches of a layer and not the call's, so
 // that sample ranges of a batch take one kernel.  The stream is the faster one while an SM has at most one cache, and beyond
-// that once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes.  Measured, us
-// per step, launched one by one (stream / this file; d = 128, g = 4, one pair leaves by its average and the rows behind it
-// move up, unless said otherwise):
-//   up to one per SM: 64 caches of 512 pairs 8.6 / 9.9, 128 of 330 8.1 / 8.5, of 700 10.4 / 14.2, of 1024 13.8 / 18.4;
-//   up to two, from 48 KB, at d = 64 (twice the rows) from 80 (below that a pass over 288 caches of 284 pairs was 3 % slower): 192
-//   of 60 7.7 / 7.7, of 120 7.8 / 8.7, of 200 9.6 / 10.4, of 600 15.7 / 17.9, unordered 14.1 / 15.8, by raw sums 499 15.3 / 19.6, by the current query 499
-//   20.2 / 23.3; d = 64 128 of 500 7.5 / 9.8, 192 of 120 7.8 / 7.5, of 1024 16.3 / 17.3; g = 8 128 of 700 11.1 / 15.6;
-//   up to three, from 96 KB: 320 of 120 10.1 / 9.9, of 200 13.0 / 14.0, of 500 19.0 / 24.1, 384 of 200 13.3 / 13.8, unordered 12.2 / 12.2,
-//   of 120 10.5 / 9.9; d = 64 384 of 330 13.0 / 12.8;
-//   up to four, from 172 KB (the last round of caches is a large part), or 150 where the pairs that leave are not found by
-//   averages alone: 512 of 330 21.3 / 19.9, of 400 24.7 / 26.6, unordered of 330 20.2 / 18.3, by raw sums 330 22.6 / 25.2, by the
-//   current query 330 25.8 / 27.9, 200 18.3 / 17.3; d = 64 512 of 700 24.0 / 25.7; g = 1 512 of 400 23.3 / 24.4; one step in four
-//   evicting 330 22.4 / 19.8;
-//   more, from 112 KB: 800 of 200 24.5 / 24.2, of 260 30.1 / 34.5, of 400 35.0 / 48.0, 1024 of 150 25.6 / 22.2.
-//   A cut by more than one value per pair follows the stream as a launch of its own: under rule 4 8 caches of 300 pairs
-//   16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 192 of 499 23.6 / 22.9, 512 of 700 69 / 64; unordered with a recent window 512 of
-//   700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
+// that once a cache's rows are long enough for its chain (about 4 us) to hide under the next cache's bytes; short groups are
+// cheaper on this file's kernels, the more so where the handle's caches stay in L2.  Measured in whole passes, launched one by one and
+// as replayed graphs (the two agree within 3 %), this file's time / the stream's, at KB of rows per cache; d = 128, one pair leaves
+// by its average and the rows behind it move up, unless said otherwise:
+//   in L2, up to one per SM: everywhere above 1 (1.02 to 2.7) but for 75 to 148 caches of 380 to 640 pairs under the current
+//     query's rule, most of whose rows move: 0.94 to 0.99 (the instance with K in registers; g = 8 1.03);
+//   up to two: 192 caches, g = 4 30 KB 1.17, 100 1.09, 256 1.15; g = 2 50 KB 0.97, 100 0.96, 135 1.04, 256 1.07; g = 1 50 KB 0.91,
+//     100 0.89, 165 0.97, 200 1.03; unordered g = 1 165 KB 0.98, 225 0.98; by raw sums g = 1 100 KB 0.99, 165 1.09;
+//     d = 64: g = 8 25 KB 1.13; g = 4 37 KB 0.97, 50 1.02, unordered 50 0.99, 82 1.01; g = 1 128 KB 0.96, 200 1.01, by raw sums 50
+//     0.95, 82 1.07;
+//   up to three: 384 caches, g = 4 75 KB 1.00, 100 1.05; g = 1 100 KB 0.98, 135 0.97, 165 1.06; by raw sums, 352 caches, g = 1
+//     55 KB 0.96, 100 1.17; d = 64 128 KB 0.93 to 1.03, 150 1.04 to 1.14, by raw sums 50 KB 1.01, 82 1.15;
+//   up to four (the last round of caches is a large part): 480 caches 165 KB 0.88 to 0.91, 200 0.97 to 1.24; by raw sums 100 KB 0.96,
+//     165 1.09; d = 64 150 KB 0.92, 200 1.14;
+//   more: 800 caches 100 KB 0.96 to 1.03, 135 1.16 to 1.21; d = 64 100 KB 1.00 to 1.06.
+//   out of HBM (several layers in turn), one per SM 1.27 and more; 192 caches 30 KB 1.01 to 1.17, d = 64 30 KB 0.97 to 1.09,
+//     50 1.02 to 1.08; 352 caches 60 KB 0.93 to 1.00, 100 1.08, d = 64 30 KB 0.85, 50 1.05; 480 caches 135 KB 0.95, 165 1.02, d = 64
+//     82 KB 0.96, 112 1.04; 800 caches 60 KB 0.92 to 0.99, 100 1.15, d = 64 30 KB 0.84, 50 1.07.
+//   A cut by more than one value per pair follows the stream as a launch of its own, us per step, launched one by one (stream / this
+//   file): under rule 4 8 caches of 300 pairs 16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 192 of 499 23.6 / 22.9, 512 of 700 69 / 64; unordered
+//   with a recent window 512 of 700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
 static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
-  const int sms = sm_count(), caches = c.layer_units;
-  const size_t kb = (size_t)(c.n_old + 1) * d * 4 >> 10;
+  const int caches = c.layer_units, per_sm = (caches + sm_count() - 1) / sm_count(), n1 = c.n_old + 1, row = c.g * d;
+  const size_t kb = (size_t)n1 * d * 4 >> 10;
   if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) && (caches > kMostSharedCaches || (c.rule == 4 && kb < 200))) return false;
-  if (caches <= sms) return true;
-  if (caches <= 2 * sms) return kb >= (d == 64 ? 80 : 48);
-  if (caches <= 3 * sms) return kb >= 96;
-  if (caches <= 4 * sms) return kb >= (c.rule == 0 && !c.padded ? 172 : 150);
-  return kb >= 112;
+  if (per_sm == 1)
+    return !(c.in_l2 && c.rule == 2 && !c.fill && d == 128 && c.g < 8 && caches > kMostSharedCaches && n1 > 380 && n1 <= kBatchTiles * 128);
+  if (!c.in_l2) return kb >= (d == 64 ? (per_sm == 4 ? 112 : 48) : per_sm == 2 ? 24 : per_sm == 4 ? 150 : 72);
+  const bool plain = c.rule == 0 && !c.padded;
+  switch (per_sm) {
+    case 2:
+      if (row >= 512) return kb >= 24;
+      if (row == 256 && d == 64) return kb >= (c.fill ? 80 : 48);
+      if (!plain) return kb >= (d == 64 ? 64 : 128);
+      return kb >= (c.fill ? 256 : row == 256 ? 128 : 200);
+    case 3: return kb >= (!plain ? 64 : d == 128 && row >= 256 ? 96 : 144);
+    case 4: return kb >= (!plain ? 150 : d == 64 ? 172 : 190);
+    default: return kb >= 112;
+  }
 }
 
 cudaError_t launch_decode_mma(int d, const CacheView& c, const void* q, const void* k, const void* v, void* out,

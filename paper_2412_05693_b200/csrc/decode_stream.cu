@@ -932,6 +932,7 @@ cudaError_t launch_stream(const CacheView& c, StreamArgs a, cudaStream_t st, boo
     return cudaSuccess;
   *taken = true;
   ProfileScope prof(kDecode, st);
+  g_last_decode_path = p.C > 1 ? 5 : 4;
   cudaError_t err;
   if (p.C > 1) {
     static SmemConfigured configured;

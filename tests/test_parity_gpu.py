@@ -260,18 +260,52 @@ def test_decode_kernel_by_number_and_length_of_caches(b, Hkv, g, d, K, kw):
     assert st["evictions"] >= 3 * 4
 
 
+@pytest.mark.parametrize("b,Hkv,g,d,K,kw,path", [
+    (18, 8, 1, 64, 60, {}, 4),                             # up to one per SM: the stream
+    (25, 4, 4, 128, 400, dict(rule="current_query"), 3),   # ... but under this rule, 380 to 640 pairs, K in registers
+    (25, 4, 1, 128, 639, dict(rule="current_query"), 3),
+    (25, 4, 1, 128, 640, dict(rule="current_query"), 4),
+    (25, 4, 8, 128, 500, dict(rule="current_query"), 4),
+    (25, 4, 4, 128, 500, dict(rule="current_query", compaction="fill"), 4),
+    (24, 8, 4, 128, 60, {}, 4),                            # 192 caches: from 24 KB on in groups of four,
+    (24, 8, 2, 128, 200, {}, 2), (24, 8, 2, 128, 270, {}, 4),   # 128 KB in groups of two,
+    (24, 8, 1, 128, 390, {}, 2), (24, 8, 1, 128, 420, {}, 4),   # 200 KB without
+    (24, 8, 1, 128, 300, dict(L=4), 4),                    # ... where all layers do not stay in L2
+    (24, 8, 1, 64, 200, dict(rule="sum_recent"), 2), (24, 8, 1, 64, 300, dict(rule="sum_recent"), 4),
+    (48, 8, 1, 128, 270, {}, 2), (48, 8, 1, 128, 300, {}, 4),   # 384
+    (60, 8, 4, 128, 360, {}, 2), (60, 8, 4, 128, 390, {}, 4),   # 480
+])
+def test_decode_kernel_that_the_rule_chooses(b, Hkv, g, d, K, kw, path):
+    kw = dict(kw)
+    wl = tiny("chosen", b=b, Hq=g * Hkv, Hkv=Hkv, s=K, B=K, K=K, steps=3, dtype="bf16", d=d, L=kw.pop("L", 1))
+    run_lockstep(wl, [(0, 0), (b // 2, Hkv // 2), (b - 1, Hkv - 1)], check_rows_every=1, **kw)
+    assert bm.last_decode_path() == path
+
+
+@pytest.mark.parametrize("K,kw", [(380, {}), (300, dict(rule="average_std")), (639, dict(rule="window_pooled")),
+                                  (380, dict(p_dec=2))])
+def test_decode_with_k_in_registers(K, kw):
+    # a handle's caches that two SMs would share, in ranges of at most one per SM, and cuts by several values: the instance that
+    # keeps K in registers, stages V by TMA and moves rows as TMA tiles, against the oracle
+    kw = dict(kw)
+    wl = tiny("k_in_registers", b=24, Hq=8, Hkv=8, s=K + 100, B=K, K=K, steps=5, dtype="bf16", d=128, p_dec=kw.pop("p_dec", 1))
+    run_lockstep(wl, [(0, 0), (5, 3), (6, 0), (23, 7)], check_rows_every=1, micro=6, micro_dec=6, **kw)
+    assert bm.last_decode_path() == 3
+    if not kw:                                             # the whole batch, two CTAs per SM: the same bits
+        assert_same_run(run_free(wl), run_free(wl, micro=6))
+
+
 @pytest.mark.parametrize("K,g", [(511, 4), (512, 1), (600, 4), (639, 2), (640, 4)])
 def test_decode_with_one_cache_per_sm(K, g):
-    # few caches of at most 640 pairs: the decode kernel's instance that keeps K in registers and stages V by TMA
-    # (rows behind the pair that leaves move up as TMA tiles, their first rows and a tail past the staged rows by
-    # plain stores); 641 pairs fall back to the other instance
+    # six caches around whole numbers of tiles: the stream over clusters
     wl = tiny("one_per_sm", b=3, Hq=2 * g, Hkv=2, s=K + 140, B=128, K=K, steps=14, dtype="bf16", d=128)
     st = run_lockstep(wl, all_units(wl), check_rows_every=1)
     assert st["evictions"] >= 6 * 14
 
 
 @pytest.mark.parametrize("b,Hkv,g,d,K,dtype,kw", [
-    (8, 8, 4, 128, 200, "bf16", {}),                            # one cache per SM, in L2: K in registers, moves by TMA
+    (8, 8, 4, 128, 200, "bf16", {}),                            # the stream, one cache per SM
+    (25, 4, 4, 128, 400, "bf16", dict(rule="current_query")),   # K in registers, moves by TMA
     (40, 8, 2, 64, 60, "bf16", {}),                             # small CTAs
     (40, 8, 2, 64, 60, "bf16", dict(compaction="fill")),
     (40, 8, 2, 64, 60, "bf16", dict(rule="sum_recent")),
