@@ -923,9 +923,10 @@ def main(argv=None):
     import torch
     import torch.distributed as dist
     assert torch.cuda.is_available(), "bench.py needs a CUDA device (there is no CPU fallback)"
-    from paper_2412_05693_b200.build import build
+    from paper_2412_05693_b200.build import build, build_fastcall
     if local_rank == 0 or world == 1:
         build()
+        build_fastcall()
     if world > 1:
         dist.init_process_group("nccl", device_id=torch.device("cuda", local_rank))
         dist.barrier()

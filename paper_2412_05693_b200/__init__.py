@@ -18,3 +18,11 @@ from .binding import (  # noqa: F401
     max_batch,
     workspace_bytes,
 )
+
+
+def __getattr__(name):
+    if name == "_fastcall":   # the native step, where one is built for this torch and Python
+        from .binding import fastcall
+        if (module := fastcall()) is not None:
+            return module
+    raise AttributeError(f"module {__name__!r} has no attribute {name!r}")

@@ -6,6 +6,7 @@ inside the library's kernels.  Importing this module without the built library r
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -95,6 +96,28 @@ def lib():
             fn.restype, fn.argtypes = res, args
         _lib = h
     return _lib
+
+
+_fastcall = None   # the native step's module, False: there is none to load
+
+
+def fastcall():
+    """csrc/fastcall.cpp as built for this torch and Python, or None: the general way then takes every call."""
+    global _fastcall
+    if _fastcall is None:
+        from .build import fastcall_path
+        import torch  # noqa: F401  (the module is linked against its libraries)
+        _fastcall = False
+        path = fastcall_path()
+        if path is not None and os.path.exists(path):
+            try:
+                spec = importlib.util.spec_from_file_location(__package__ + "._fastcall", path)
+                module = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(module)
+                _fastcall = module
+            except ImportError:
+                pass
+    return _fastcall or None
 
 
 def _check(code: int, where: str):
@@ -257,8 +280,7 @@ class BatchMaxCache:
                                          self.workspace.numel(), _stream(stream), C.byref(h)), "bm_cache_create")
         self.h = h
         self._prefill, self._decode = lib().bm_prefill_block, lib().bm_decode_step
-        from . import _fastcall            # (needs torch's libraries, loaded by now)
-        self._fast = _fastcall
+        self._fast = fastcall()
         bf16 = self.tdtype == torch.bfloat16
         self._fast_prefill = (C.cast(self._prefill, _vp).value, h.value, bf16)   # address, handle, element type
         self._fast_decode = (C.cast(self._decode, _vp).value, h.value, bf16)
@@ -286,7 +308,7 @@ class BatchMaxCache:
         """q (ns, I, Hq, d), k/v (ns, I, Hkv, d) contiguous device tensors; returns out (ns, I, Hq, d)."""
         if out is None:
             out = self.torch.empty_like(q)
-        if stream is None:
+        if stream is None and self._fast is not None:
             rc = self._fast.prefill(*self._fast_prefill, q, k, v, out, layer, sample0, evict_to, pos0)
             if rc is not None:
                 if rc:
@@ -318,7 +340,7 @@ class BatchMaxCache:
         """q (ns, Hq, d), k/v (ns, Hkv, d); returns out (ns, Hq, d)."""
         if out is None:
             out = self.torch.empty_like(q)
-        if stream is None:
+        if stream is None and self._fast is not None:
             rc = self._fast.decode(*self._fast_decode, q, k, v, out, layer, sample0, evict_to)
             if rc is not None:
                 if rc:

@@ -179,3 +179,51 @@ def test_native_step_declines_what_it_does_not_handle_and_checks_like_the_genera
         out = torch.empty_like(q)
         assert step(out=out, evict_to=9) == 3
         assert calls == [(77, 1, 2, 2, q.data_ptr(), kv.data_ptr(), kv.data_ptr(), out.data_ptr(), 9)]
+
+
+def test_library_builds_without_torch_and_without_the_native_step(monkeypatch):
+    from paper_2412_05693_b200 import build as b
+    monkeypatch.setattr(b, "_stale", lambda path: False)
+    monkeypatch.setattr(b, "build_fastcall", lambda force=False: pytest.fail("the C library needs no native step"))
+    assert b.build() == b.LIB_PATH and b.build(debug=True) == b.DEBUG_LIB_PATH
+
+
+def test_native_step_is_built_for_one_torch_and_one_python(monkeypatch, tmp_path):
+    import importlib.metadata
+    import sysconfig
+    import torch
+    from paper_2412_05693_b200 import build as b
+    name = os.path.basename(b.fastcall_path())
+    assert torch.__version__.replace("+", "_") in name and name.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    monkeypatch.setattr(b, "PKG_DIR", str(tmp_path))
+    seen = []
+
+    def compiler(cmd, check):   # a compiler that fails half way, then one that does not
+        seen.append(cmd[cmd.index("-o") + 1])
+        open(seen[-1], "w").write("half")
+        if len(seen) == 1:
+            raise subprocess.CalledProcessError(1, cmd)
+
+    import subprocess
+    monkeypatch.setattr(b.subprocess, "run", compiler)
+    with pytest.raises(subprocess.CalledProcessError):
+        b.build_fastcall()
+    assert os.listdir(tmp_path) == []                        # never under its own name before it is complete
+    assert b.build_fastcall() == b.fastcall_path() != seen[1] and os.listdir(tmp_path) == [os.path.basename(b.fastcall_path())]
+    assert b.build_fastcall() == b.fastcall_path() and len(seen) == 2
+
+    def absent(name):
+        raise importlib.metadata.PackageNotFoundError(name)
+    monkeypatch.setattr(b.importlib.metadata, "version", absent)
+    assert b.fastcall_path() is None and b.build_fastcall() is None
+
+
+@pytest.mark.parametrize("contents", [None, b"not a library"])
+def test_binding_goes_its_general_way_without_the_native_step(monkeypatch, tmp_path, contents):
+    from paper_2412_05693_b200 import binding, build as b
+    path = str(tmp_path / "_fastcall.so")
+    if contents is not None:
+        open(path, "wb").write(contents)
+    monkeypatch.setattr(b, "fastcall_path", lambda: path)
+    monkeypatch.setattr(binding, "_fastcall", None)
+    assert binding.fastcall() is None

@@ -1153,6 +1153,15 @@ def test_bitwise_reproducible_and_variants_agree(dtype, d):
     assert_same_run(base, run_free(wl, micro=1))        # sample ranges: micro-batched calls
 
 
+@pytest.mark.parametrize("dtype,d", [("bf16", 128), ("f32", 64)])
+def test_handles_without_the_native_step_give_the_same_results(dtype, d, monkeypatch):
+    wl = tiny("general_way", dtype=dtype, d=d, steps=12)
+    base = run_free(wl)
+    monkeypatch.setattr(bm.binding, "_fastcall", False)
+    assert bm.binding.fastcall() is None
+    assert_same_run(base, run_free(wl))
+
+
 @pytest.mark.parametrize("which", ["tiny", "cfg2"])
 def test_cuda_graph_replay_matches_eager_launches(which):
     # the benchmark replays one CUDA graph per step; a captured schedule must leave the same bits as eager launches
