@@ -13,16 +13,16 @@
 // What is left on a group's chain is its own softmax, and the two groups' chains are independent of each other.
 //
 // What bounds it: the two softmax warps that share a scheduler, about 2850 cycles per pair of tiles at d = 64 (their
-// instructions alone take 2100 to 2250, the exponentials 2048 on the special-function unit), and at d = 128 the turns of
-// the one logit buffer, 3150 (the tensor pipe needs 2048: busy 56 %).  Measured at 48 samples, 32 heads in groups of 4,
-// d = 128, a block of 512 against 1024 pairs: 539 -> 479 us (1076 TFLOP/s) against the kernel in which P takes the place of the
-// logits and the next Q.K^T waits for P.V; 128 samples 1399 -> 1254; 4 samples, 512 pairs 45.3 -> 40.3; d = 64, 701
-// pairs, groups of 8 161 -> 139.  What made the difference besides: code that fits the SM's 32 KB instruction cache with
-// room for every role's loop (at 78 KB this kernel took 692 us at 48 samples and 2.5 of every issue slot's waiting warps
-// waited for instructions; at 54 KB 615), hence masks in a rolled loop, rolled waits, one copy per key tile; output through
-// TMA (with plain stores 5 600 cycles per item, 4 100 now).  Not kept: a share of the exponentials as polynomials at d =
-// 128 (a quarter: 513 against 492 us; an eighth 507; at d = 64 none 139, an eighth 135, a quarter 136), softmax warps
-// that poll for their logits (527 against 513), 216 registers for them (530).
+// instructions alone take 2100 to 2250, the exponentials 1792 on the special-function unit, an eighth being polynomials),
+// and at d = 128 the turns of the one logit buffer, 3150 (the tensor pipe needs 2048, and so do the exponentials: both busy
+// 57 %).  Measured at 48 samples, 32 heads in groups of 4, d = 128, a block of 512 against 1024 pairs: 539 -> 479 us (1076
+// TFLOP/s) against the kernel in which P takes the place of the logits and the next Q.K^T waits for P.V; 128 samples 1399
+// -> 1254; 4 samples, 512 pairs 45.3 -> 40.3; d = 64, 701 pairs, groups of 8 161 -> 139.  What made the difference besides:
+// code that fits the SM's 32 KB instruction cache with room for every role's loop (at 78 KB this kernel took 692 us at 48
+// samples and 2.5 of every issue slot's waiting warps waited for instructions; at 54 KB 615), hence masks in a rolled loop,
+// rolled waits, one copy per key tile; output through TMA (with plain stores 5 600 cycles per item, 4 100 now).  Not kept:
+// a share of the exponentials as polynomials at d = 128 (a quarter: 513 against 492 us; an eighth 507; at d = 64 none 139,
+// an eighth 135, a quarter 136), softmax warps that poll for their logits (527 against 513), 216 registers for them (530).
 #pragma once
 
 template <int D>

@@ -666,7 +666,8 @@ def test_f32_kernels_by_grid_size(b, Hkv, g, d, B, K):
     (5, 4, 4, 128, 150, dict(rule="sum_recent")),
     (5, 4, 4, 64, 97, dict(rule="current_query")),
     (2, 4, 4, 128, 130, dict(rule="average_std")),
-    (4, 4, 4, 128, 790, {}),                              # too long for four, shared by eight
+    (4, 4, 4, 128, 790, {}),                              # the most that four hold: 198 rows each
+    (4, 4, 4, 128, 791, {}),                              # 199: shared by eight
     (20, 4, 1, 64, 40, {}),                               # 80 caches: not shared
 ])
 def test_f32_decode_with_caches_shared_by_clusters(b, Hkv, g, d, K, kw):
@@ -674,6 +675,18 @@ def test_f32_decode_with_caches_shared_by_clusters(b, Hkv, g, d, K, kw):
     run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1, **kw)
     if not kw:
         assert_same_run(run_free(wl), run_free(wl, micro=1))
+
+
+@pytest.mark.parametrize("b,Hkv,g,d,K,path", [
+    (4, 4, 4, 128, 1583, 1),                              # 198 rows for each of eight
+    (4, 4, 4, 128, 1584, 0),                              # more than eight hold: a CTA per cache
+    (2, 4, 1, 64, 30, 0), (2, 4, 1, 64, 31, 1),           # from 32 pairs on
+    (18, 4, 2, 64, 50, 1), (19, 4, 2, 64, 50, 0),         # up to half as many caches as SMs
+])
+def test_f32_decode_kernel_by_number_and_length_of_caches(b, Hkv, g, d, K, path):
+    wl = tiny("f32_by_grid", b=b, Hq=g * Hkv, Hkv=Hkv, s=K, B=min(K, 800), K=K, steps=2, dtype="f32", d=d)
+    run_lockstep(wl, [(0, 0), (b - 1, Hkv - 1)], check_rows_every=1)
+    assert bm.last_decode_path() == path
 
 
 @pytest.mark.parametrize("b,Hkv,g,d,K,bound", [
