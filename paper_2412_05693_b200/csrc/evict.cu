@@ -43,10 +43,15 @@ cudaError_t launch_w(const CacheView& c, const EvictArgs& e, int cluster, cudaSt
 // to move: 8 caches from 1024 to 512 32.0 / 31.5, 16 caches from 600 to 300 28.3 / 27.0.  Unordered caches move little and
 // gained nothing (8 caches to 1024 pairs 40.2 / 39.4); as many pieces in flight without a cluster cost 1 to 4 us (128
 // caches from 768 to 512 50.6 / 48.8).
+// Up to two caches per SM in a layer the handle's caches decide, not the call's: sample ranges of such a batch may be in flight
+// together, and clusters of one then take the SMs that the others' kernels need (16 samples, 16 blocks of 256 in a replayed graph,
+// in 4 ranges on 4 streams 1.79 ms with clusters, 1.60 without, in 8 ranges 1.93 / 1.61, in one 1.59).  A range of a larger batch
+// shares as a call of its own does (one sample of 64, 512 pairs more than the 1024 that stay 53.1 / 58.2 us per call).
 template <typename T, int D>
 cudaError_t launch_t(const CacheView& c, const EvictArgs& e, cudaStream_t st) {
   if (c.fill) return launch_w<T, D, true, 8>(c, e, 1, st);
-  const int units = c.nsamples * c.Hkv, cluster = units <= 8 ? 8 : units <= 32 ? 4 : units <= 64 ? 2 : 1;
+  const int units = c.layer_units <= 2 * sm_count() ? c.layer_units : c.nsamples * c.Hkv;
+  const int cluster = units <= 8 ? 8 : units <= 32 ? 4 : units <= 64 ? 2 : 1;
   const size_t bytes = (size_t)e.target * D * 2 * sizeof(T);   // that may move per cache
   if (cluster > 1 && cluster * units <= sm_count() && bytes >= std::max((size_t)256 << 10, (size_t)cluster << 16))
     return launch_w<T, D, false, 16>(c, e, cluster, st);
