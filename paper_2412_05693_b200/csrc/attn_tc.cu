@@ -403,16 +403,20 @@ cudaError_t launch_fwd_items(const CacheView& c, const BlockArgs& a, cudaStream_
   // sums of a row are cut differently, and outputs do not depend on how a batch is cut into sample ranges.
   if ((long long)tiles * c.layer_units <= sms)
     return launch_fwd_pair<D, PAD, kSplit>(c, a, args, args.across ? dim3(units, tiles) : dim3(tiles, units), st);
-  // Row tiles of any caches: one by one while a call's (a sample range's) have an SM each, and two by two where caches with an
-  // odd number of them would leave items with a single one (which take four sevenths of a pair's time) and need a round more.
-  // Beyond two rounds keys and values that are loaded once per row tile cost more than that.  us per prefill call (forward, column
-  // sums, cut), pairs / any: one sample of 64, 32 row tiles of 8 caches, 1024 pairs 61.4 / 53.2, 16 of them, 512 pairs 42.0 / 38.0;
-  // three row tiles of 80 caches, 512 pairs 50.4 / 44.5, 1024 pairs 72.3 / 62.5, of 176 caches 77.0 / 72.8; one of 176 48.2 / 44.5, of
-  // 320 69.6 / 71.4, of 512 at d = 64 122.5 / 109.8; three of 320 caches 123.7 / 130.2.
+  // Row tiles of any caches: one by one for a lone sample range, and two by two where caches with an odd number of them would
+  // leave items with a single one (which take four sevenths of a pair's time) and need a round more.  Beyond two rounds keys and
+  // values that are loaded once per row tile cost more than that.  us per prefill call (forward, column sums, cut), pairs / any: one
+  // sample of 64, 32 row tiles of 8 caches, 1024 pairs 61.4 / 53.2, 16 of them, 512 pairs 42.0 / 38.0; three row tiles of 80 caches,
+  // 512 pairs 50.4 / 44.5, 1024 pairs 72.3 / 62.5, of 176 caches 77.0 / 72.8; one of 176 48.2 / 44.5, of 320 69.6 / 71.4, of 512 at d = 64
+  // 122.5 / 109.8; three of 320 caches 123.7 / 130.2.
+  // A single row tile takes an SM as a pair does, and ranges in flight together pay for it: 16 samples, 16 blocks of 256 in 8 ranges on 8
+  // streams 2.09 ms, in pairs 1.61, in 16 ranges 2.17 / 1.65, where a lone one of these takes 38.0 / 42.0 us per call.  So one by one
+  // where a batch makes many ranges, or a call is small beside the GPU.
   auto rounds = [&](long long items) { return (items + sms - 1) / sms; };
   const long long twos = rounds((all + 1) / 2);
-  if (all <= sms || (twos <= 2 && 7 * twos < (tiles == 1 ? 4 : 7) * rounds((long long)groups * units))) {
-    args.any = all <= sms ? 1 : 2;
+  const bool one = all <= sms && (4 * all <= sms || (long long)groups * c.layer_units >= 1024);
+  if (one || (all > sms && twos <= 2 && 7 * twos < (tiles == 1 ? 4 : 7) * rounds((long long)groups * units))) {
+    args.any = one ? 1 : 2;
     return launch_fwd_pair<D, PAD, kAny>(c, a, args, dim3((unsigned)((all + args.any - 1) / args.any)), st);
   }
   return launch_fwd_pair<D, PAD, kPairs>(c, a, args, args.across ? dim3(units, groups) : dim3(groups, units), st);
