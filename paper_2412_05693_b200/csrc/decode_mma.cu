@@ -720,10 +720,12 @@ size_t decode_mma_smem_bytes(int d, int g, int n_rows, int target) {
 //     55 KB 0.96, 100 1.17; d = 64 128 KB 0.93 to 1.03, 150 1.04 to 1.14, by raw sums 50 KB 1.01, 82 1.15;
 //   up to four (the last round of caches is a large part): 480 caches 165 KB 0.88 to 0.91, 200 0.97 to 1.24; by raw sums 100 KB 0.96,
 //     165 1.09; d = 64 150 KB 0.92, 200 1.14;
-//   more: 800 caches 100 KB 0.96 to 1.03, 135 1.16 to 1.21; d = 64 100 KB 1.00 to 1.06.
+//   more: 640 to 1184 caches 75 KB 0.81 to 0.99, 100 0.96 to 1.04, 135 1.05 to 1.20, by raw sums 50 KB 0.83 to 1.04, 100 1.19 to 1.25; d = 64
+//     82 KB 0.95 to 1.05, 100 1.00 to 1.14, by raw sums 50 KB 0.85 to 1.09, 82 1.14 to 1.23.
 //   out of HBM (several layers in turn), one per SM 1.27 and more; 192 caches 30 KB 1.01 to 1.17, d = 64 30 KB 0.97 to 1.09,
 //     50 1.02 to 1.08; 352 caches 60 KB 0.93 to 1.00, 100 1.08, d = 64 30 KB 0.85, 50 1.05; 480 caches 135 KB 0.95, 165 1.02, d = 64
-//     82 KB 0.96, 112 1.04; 800 caches 60 KB 0.92 to 0.99, 100 1.15, d = 64 30 KB 0.84, 50 1.07.
+//     82 KB 0.96, 112 1.04; 800 caches 75 KB 1.05, 100 1.15, d = 64 37 KB 0.96, 50 1.07; 1184 to 3072 caches 75 KB 0.91 to 0.96, 100 1.00
+//     to 1.05, by raw sums 50 KB 0.98 to 1.03; d = 64 67 KB 0.89 to 0.99, 82 1.00 to 1.13, by raw sums 50 KB 1.06 to 1.17.
 //   A cut by more than one value per pair follows the stream as a launch of its own, us per step, launched one by one (stream / this
 //   file): under rule 4 8 caches of 300 pairs 16.4 / 15.6, 64 caches of 700 22.8 / 24.3, 192 of 499 23.6 / 22.9, 512 of 700 69 / 64; unordered
 //   with a recent window 512 of 700 58 / 48.  (More than one pair by one value: 512 of 700, two every second step, 45.9 / 53.9 per step.)
@@ -733,8 +735,11 @@ static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
   if (cut && !one && (c.rule >= 3 || (c.fill && c.rule == 1)) && (caches > kMostSharedCaches || (c.rule == 4 && kb < 200))) return false;
   if (per_sm == 1)
     return !(c.in_l2 && c.rule == 2 && !c.fill && d == 128 && c.g < 8 && caches > kMostSharedCaches && n1 > 380 && n1 <= kBatchTiles * 128);
-  if (!c.in_l2) return kb >= (d == 64 ? (per_sm == 4 ? 112 : 48) : per_sm == 2 ? 24 : per_sm == 4 ? 150 : 72);
   const bool plain = c.rule == 0 && !c.padded;
+  if (!c.in_l2) {
+    if (per_sm > 6) return kb >= (!plain ? 48 : d == 64 ? 80 : 100);
+    return kb >= (d == 64 ? (per_sm == 4 ? 112 : 48) : per_sm == 2 ? 24 : per_sm == 4 ? 150 : 72);
+  }
   switch (per_sm) {
     case 2:
       if (row >= 512) return kb >= 24;
@@ -743,7 +748,7 @@ static bool stream_is_faster(const CacheView& c, int d, bool cut, bool one) {
       return kb >= (c.fill ? 256 : row == 256 ? 128 : 200);
     case 3: return kb >= (!plain ? 64 : d == 128 && row >= 256 ? 96 : 144);
     case 4: return kb >= (!plain ? 150 : d == 64 ? 172 : 190);
-    default: return kb >= 112;
+    default: return kb >= (plain ? 100 : 80);
   }
 }
 

@@ -274,6 +274,8 @@ def test_decode_kernel_by_number_and_length_of_caches(b, Hkv, g, d, K, kw):
     (24, 8, 1, 64, 200, dict(rule="sum_recent"), 2), (24, 8, 1, 64, 300, dict(rule="sum_recent"), 4),
     (48, 8, 1, 128, 270, {}, 2), (48, 8, 1, 128, 300, {}, 4),   # 384
     (60, 8, 4, 128, 360, {}, 2), (60, 8, 4, 128, 390, {}, 4),   # 480
+    (80, 8, 4, 64, 390, {}, 2), (80, 8, 4, 64, 410, {}, 4),     # 640
+    (150, 8, 4, 64, 230, dict(L=2), 2), (150, 8, 4, 64, 340, dict(L=2), 4),   # 1200, out of HBM
 ])
 def test_decode_kernel_that_the_rule_chooses(b, Hkv, g, d, K, kw, path):
     kw = dict(kw)
