@@ -410,8 +410,9 @@ cudaError_t launch_fwd_items(const CacheView& c, const BlockArgs& a, cudaStream_
   // 512 pairs 50.4 / 44.5, 1024 pairs 72.3 / 62.5, of 176 caches 77.0 / 72.8; one of 176 48.2 / 44.5, of 320 69.6 / 71.4, of 512 at d = 64
   // 122.5 / 109.8; three of 320 caches 123.7 / 130.2.
   // A single row tile takes an SM as a pair does, and ranges in flight together pay for it: 16 samples, 16 blocks of 256 in 8 ranges on 8
-  // streams 2.09 ms, in pairs 1.61, in 16 ranges 2.17 / 1.65, where a lone one of these takes 38.0 / 42.0 us per call.  So one by one
-  // where a batch makes many ranges, or a call is small beside the GPU.
+  // streams 2.09 ms, in pairs 1.61, in 16 ranges 2.17 / 1.65, where a lone one of these takes 38.0 / 42.0 us per call; 64 samples in 16
+  // ranges in flight 3.27 / 3.33, in 32 4.23 / 3.43, a lone sample of them 53.2 / 61.4.  So one by one where a batch makes many ranges,
+  // which are seldom all in flight, or a call is small beside the GPU.
   auto rounds = [&](long long items) { return (items + sms - 1) / sms; };
   const long long twos = rounds((all + 1) / 2);
   const bool one = all <= sms && (4 * all <= sms || (long long)groups * c.layer_units >= 1024);
